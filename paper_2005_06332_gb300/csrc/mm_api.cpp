@@ -11,6 +11,7 @@
 
 #include "mm.h"
 #include "mm_gate_table.h"
+#include "mm_gate_table64.h"
 #include "mm_internal.h"
 #include "mm_layout.h"
 
@@ -92,7 +93,8 @@ struct mm_net {
 
     // device arrays (FP64 path)
     double *V = nullptr, *m = nullptr, *h = nullptr, *n = nullptr;
-    double *area = nullptr, *gax = nullptr, *gsyn = nullptr;
+    double *area = nullptr, *gax = nullptr, *dcon = nullptr, *gsyn = nullptr;
+    double2 *gtab64 = nullptr;        // gate table for dt (mm_gate_table64.h)
     // device arrays (FP32c path)
     int32_t *Vq = nullptr;
     uint32_t *mq = nullptr, *hq = nullptr, *nq = nullptr;
@@ -602,16 +604,13 @@ mm_status build(mm_net *net, const mm_morphologies *morph, const mm_channel_para
     li.group_comps = opt->group_comps > 0 ? opt->group_comps
                    : (opt->precision == MM_FP64 ? kDefaultGroupComps : kDefaultGroupComps32);
     li.max_group_comps = opt->precision == MM_FP64 ? kMaxGroupComps : kMaxGroupComps32;
-    // shared memory per item: FP64 d and rhs per compartment (16 B); FP32c
-    // d, rhs and |g| per compartment (12 B) and per path its contribution
-    // to the parent (d, rhs) and the potential across its head link (12 B)
+    // shared memory per item: FP64 the diagonal and rhs per compartment (16 B);
     // FP32c (active conductance, rhs) pair, the implicit coupling and the
     // passive diagonal as pairs (the diagonal's place holds the rhs's low
     // words until the rhs is final; 24 B per compartment) and per path two
     // words (the head link's current, then the contribution to the parent)
     li.smem_per_comp = opt->precision == MM_FP64 ? 16 : 24;
-    li.smem_per_seg = 0;
-    li.path_items = opt->precision != MM_FP64;
+    li.path_items = true;
     li.smem_per_path = opt->precision == MM_FP64 ? 0 : 8;
     li.giant_smem_limit = opt->precision == MM_FP64 ? 0 : kGiantSmemLimit;
     li.big_smem_limit = opt->precision == MM_FP64 ? 0 : kBigSmemLimit;
@@ -662,6 +661,13 @@ mm_status build(mm_net *net, const mm_morphologies *morph, const mm_channel_para
         ZR(net->n, C);
         ZR(net->area, C);
         ZR(net->gax, C);
+        ZR(net->dcon, C);
+        {
+            std::vector<mmg::Quad64> tab((size_t)mmg::kTab64Quads * mmg::kTab64Intervals);
+            mmg::build_table64(opt->dt_ms, tab.data());
+            UP(net->gtab64, reinterpret_cast<const double2 *>(tab.data()), tab.size());
+            MM_CK(net, cudaStreamSynchronize(net->stream));  // before the host copy goes
+        }
         ZR(net->gsyn, (size_t)std::max<int64_t>(net->nsite, 1));
     } else {
         ZR(net->Vq, C);
@@ -769,6 +775,10 @@ mm_status build(mm_net *net, const mm_morphologies *morph, const mm_channel_para
     if (f64) {
         ia.area = net->area;
         ia.gax = net->gax;
+        ia.dcon = net->dcon;
+        ia.cm_dt = chan->Cm * 1e3 / opt->dt_ms;
+        ia.gimp = opt->scheme == MM_SCHEME_CN ? 0.5 : 1.0;
+        ia.gleak = opt->scheme == MM_SCHEME_CN ? 0.0 : chan->gL * 1e3;
         ia.V = net->V;
         ia.m = net->m;
         ia.h = net->h;
@@ -793,12 +803,13 @@ mm_status build(mm_net *net, const mm_morphologies *morph, const mm_channel_para
         a.n = net->n;
         a.area = net->area;
         a.gax = net->gax;
+        a.dcon = net->dcon;
+        a.gtab = net->gtab64;
         a.stim = net->stim;
         a.user_id = net->user_id;
         a.groups = dgroups;
         a.n_groups = (int32_t)L.groups.size();
         a.meta = dmeta;
-        a.smem_meta = L.max_meta;
         a.site_comp = dsite;
         a.gsyn = net->gsyn;
         a.ring_nrn = net->ring_nrn;
@@ -817,15 +828,12 @@ mm_status build(mm_net *net, const mm_morphologies *morph, const mm_channel_para
         a.fired = net->fired;
         a.fired_words = net->fired_words;
         a.ctl = net->ctl;
-        a.smem_comps = smem_comps;
-        a.smem_segs = smem_segs;
-        a.gNa = chan->gNa;
-        a.gK = chan->gK;
-        a.gL = chan->gL;
+        a.gNa = chan->gNa * 1e3;
+        a.gK = chan->gK * 1e3;
+        a.gL = chan->gL * 1e3;
         a.ENa = chan->ENa;
         a.EK = chan->EK;
         a.EL = chan->EL;
-        a.cm_dt = chan->Cm * 1e3 / opt->dt_ms;
         a.gimp = opt->scheme == MM_SCHEME_CN ? 0.5 : 1.0;
         a.g_implicit = opt->scheme == MM_SCHEME_CN ? 0 : 1;
         a.e_syn = syn ? syn->e_rev_mV : 0.0;
@@ -944,15 +952,15 @@ mm_status build(mm_net *net, const mm_morphologies *morph, const mm_channel_para
     d.fired_words = net->fired_words;
     d.nsite = net->nsite;
 
-    // FP32c carves each item's shared memory from its own sizes (the largest
-    // per-item need of the class); FP64 uses one carve for all items
-    const size_t smem = f64 ? mmk_step_fp64_smem(smem_comps, smem_segs, L.max_meta) : (size_t)std::max<int64_t>(L.max_smem, 16);
+    // each item's shared memory is carved from its own sizes; the launch
+    // provides the largest need of the class
+    const size_t smem = (size_t)std::max<int64_t>(L.max_smem, 16);
     if (smem > kMaxSmem) return fail(net, MM_ENOTSUP, "a work item needs more shared memory than a block has");
     int threads = opt->block_threads > 0 ? opt->block_threads : (f64 ? kStepThreads : 512);
     if (threads != 128 && threads != 256 && threads != 512 && (f64 || threads != 1024))
         return fail(net, MM_EINVAL, "block_threads must be 128, 256 or 512 (or 1024 for MM_FP32C)");
     net->step_threads = threads;
-    net->sa32.smem_bytes = (int32_t)smem;
+    net->sa.smem_bytes = net->sa32.smem_bytes = (int32_t)smem;
     int per_sm = 0;
     if (f64) MM_CKI(net, mmk_step_fp64_blocks_per_sm(threads, (int)smem, &per_sm));
     else MM_CKI(net, mmk_step_fp32c_blocks_per_sm(threads, (int)smem, &per_sm));

@@ -9,54 +9,25 @@
 //     compartment that does not continue its parent's path, its deepest
 //     child, that one's deepest child, and so on down to a leaf -- is one
 //     contiguous index range in which each compartment's parent is the one
-//     before it; an unbranched run of the tree (a "segment") is contiguous
-//     as well;
+//     before it;
 //   * consecutive neurons are packed into work items ("groups") whose
 //     compartments are contiguous; one thread block solves one group at a
 //     time, with the group's Hines diagonal and right-hand side in shared
 //     memory (giant FP32c items: in a global scratch);
-//   * FP32c: the paths of a neuron are sorted by level (0: the path from its
+//   * the paths of a neuron are sorted by level (0: the path from its
 //     soma; level l + 1: paths that hang off a path of level l), so that the
 //     leaves-to-root sweep of Algorithm 1 can run path by path from the
-//     deepest level up and the root-to-leaves sweep from level 0 down;
-//   * FP64: the segments of a group are sorted by height (0 = no child
-//     segment), so that all segments of one height ("wave") can be
-//     eliminated in parallel once the lower waves are done, and substituted
-//     in the reverse order.
+//     deepest level up and the root-to-leaves sweep from level 0 down.
 #pragma once
 #include <stdint.h>
 #include <vector_types.h>
 
 namespace mmk {
 
-// One segment of a group: compartments top .. top+len-1 (group-local), a
-// path from top down to the bottom compartment top+len-1.
-struct SegRec {
-    int32_t top;      // group-local index of the first compartment
-    int32_t len;      // >= 1
-    int32_t parent;   // group-local index of top's parent; -1 for a soma segment
-    int32_t child0;   // first entry of this segment's children in seg_child[]
-    int32_t nchild;   // number of child segments (all hang off the bottom)
-    int32_t neuron;   // soma segment: group-local neuron index; else -1
-};
-
-// Packed form of a segment inside a work item's tree blob (16 bytes;
-// group-local indices fit 15 bits because a work item holds at most 32767
-// compartments and segments).
-struct SegP {
-    int16_t top;      // group-local index of the first compartment
-    int16_t len;      // >= 1
-    int16_t parent;   // group-local index of top's parent; -1 for a soma segment
-    int16_t nchild;   // number of child segments
-    int16_t child0;   // first entry of this segment's children in the blob's child list
-    int16_t neuron;   // soma segment: group-local neuron index; else -1
-    int16_t pseg;     // index of the parent segment in the blob; -1 for a soma segment
-    int16_t pad;
-};
-
-// FP32c work items are solved path by path, by a team of warps per sweep
+// Work items are solved path by path, by a team of warps per sweep
 // bundle (one neuron, or several consecutive small neurons swept together).
-// Per bundle of an item (8 bytes): its paths are path0 .. path0 + npath - 1
+// Per bundle of an item (12 bytes): its compartments are comp0 .. comp0 +
+// ncomp - 1 of the item, its paths path0 .. path0 + npath - 1
 // of the item, sorted by level (0: the paths from the somata) and, within a
 // level, longest first; level l holds paths loffs[loff0 + l] ..
 // loffs[loff0 + l + 1] - 1, and the first mcnt[loff0 + l] entries of that
@@ -66,9 +37,11 @@ struct NrnQ {
     int16_t npath;
     int16_t nlevel;
     int16_t loff0;
+    int16_t comp0;
+    int16_t ncomp;
 };
 
-// A path of an FP32c work item (8 bytes).
+// A path of a work item (8 bytes).
 struct PathQ {
     int16_t head;     // group-local index of the first compartment
     int16_t end;      // one past the last compartment (a leaf)
@@ -92,7 +65,7 @@ typedef uint32_t KidQ;
 // shared memory, solved from a global scratch): NrnG per bundle, PathG per
 // path, KidG per fold entry {path, parent compartment}.
 struct NrnG {
-    int32_t path0, npath, nlevel, loff0;
+    int32_t path0, npath, nlevel, loff0, comp0, ncomp;
 };
 struct PathG {
     int32_t head, end, parent, nflag;  // nflag: neuron index | kPathAloneG
@@ -103,10 +76,7 @@ typedef int2 KidG;
 
 // One work item: a run of whole neurons.  Its tree is one contiguous,
 // 16-byte aligned blob in global memory, staged into shared memory with a
-// single bulk copy.  FP64 items: SegP[nseg] | int16 child[nchild] |
-// int16 wave_off[nwave+1] (wave w holds segments wave_off[w] ..
-// wave_off[w+1]-1; wave 0 holds the leaf segments), padded to 16 bytes.
-// FP32c items: NrnQ[nbundle] | PathQ[npath] (at byte path_off) |
+// single bulk copy: NrnQ[nbundle] | PathQ[npath] (at byte path_off) |
 // KidQ[npath] (fold list, at fold_off) | int16 loffs[] (at loffs_off) |
 // int16 mcnt[] (as many as loffs, at mcnt_off), padded to 16 bytes.
 // Giant FP32c items (beyond shared memory) use the same layout with the
@@ -117,21 +87,18 @@ struct GroupRec {
     int64_t meta_off; // byte offset of the tree blob
     int32_t meta_bytes;
     int32_t ncomp;
-    int32_t nseg;
-    int32_t nchild;
-    int32_t nwave;
     int32_t site0;    // first synaptic site (index into site_comp[] / gsyn[])
     int32_t nsite;
     int32_t neuron0;  // internal id of the first neuron
     int32_t nneuron;
     int32_t npath;
-    int32_t nlevel;   // FP32c: the largest number of path levels of a neuron of the item
-    int32_t path_off; // FP32c: byte offset of PathQ[0] inside the blob
-    int32_t fold_off; // FP32c: byte offset of the fold list
-    int32_t loffs_off;// FP32c: byte offset of the level offsets
-    int32_t mcnt_off; // FP32c: byte offset of the per-level shared-parent counts
+    int32_t nlevel;   // the largest number of path levels of a neuron of the item
+    int32_t path_off; // byte offset of PathQ[0] inside the blob
+    int32_t fold_off; // byte offset of the fold list
+    int32_t loffs_off;// byte offset of the level offsets
+    int32_t mcnt_off; // byte offset of the per-level shared-parent counts
     int32_t pscratch0;// FP32c giant items: first entry in the global per-path scratch
-    int32_t nbundle;  // FP32c: sweep bundles (NrnQ / NrnG records) of the item
+    int32_t nbundle;  // sweep bundles (NrnQ / NrnG records) of the item
     int32_t pad;
 };
 
@@ -151,14 +118,18 @@ enum { MMK_ERR_OVERFLOW = 1, MMK_ERR_NUMERIC = 2, MMK_ERR_TIMEOUT = 4 };
 struct StepArgs {
     double *V, *m, *h, *n;            // state [C]
     const double *area;               // membrane area, cm^2 [C]
-    const double *gax;                // axial conductance to the parent, uS [C] (0 at a soma)
+    const double *gax;                // axial conductance to the parent, uS [C] (0 at a soma), negated at path
+                                      // heads (somata included): their link is assembled per path
+    const double *dcon;               // constant part of the diagonal, uS [C]: C/dt, the leak (backward Euler)
+                                      // and the implicit couplings of the links inside paths
+    const double2 *gtab;              // gate table for dt (mm_gate_table64.h): 18 arrays of 961 16-byte quads
     const double *stim;               // soma current per internal neuron, nA [N]
     const int32_t *user_id;           // internal neuron -> user id [N]
     const GroupRec *groups;
     int32_t n_groups;
     int32_t step_offset;              // step index = ctl->step_base + step_offset
     const unsigned char *meta;        // tree blobs of all work items
-    int32_t smem_meta;                // bytes reserved for the largest blob
+    int32_t smem_bytes;               // dynamic shared memory of the launch (largest item need)
     const int32_t *site_comp;         // group-local compartment of each synaptic site
     double *gsyn;                     // merged synaptic conductance per site, uS
     int32_t *ring_nrn;                // [R * N] spike sources that fired, per step slot
@@ -180,9 +151,8 @@ struct StepArgs {
     uint32_t *fired;                  // deterministic delivery: [R * fired_words] bit per source that
                                       // fired in each step slot (nullptr otherwise)
     DevCtl *ctl;
-    int32_t smem_comps, smem_segs;    // shared-memory capacity of one block (FP64)
-    double gNa, gK, gL, ENa, EK, EL;
-    double cm_dt;                     // Cm * 1e3 / dt: C_i/dt = area_i * cm_dt (nF/ms = uS)
+    double gNa, gK, gL;               // channel densities times 1e3: uS per cm^2 of membrane
+    double ENa, EK, EL;
     double e_syn, threshold, dt, decay;
     // time discretisation (MM_SCHEME_*): the implicit share of each axial
     // coupling (1, or 1/2 for Eq. 2 as printed) and whether the membrane
@@ -359,11 +329,14 @@ struct DeliverArgs {
 
 struct InitArgs {
     const double *L, *diam;           // internal order
-    const int32_t *parent_dist;       // i - parent(i), negated at segment tops (FP64) or path heads (FP32c), 0 at a soma
+    const int32_t *parent_dist;       // i - parent(i), negated at path heads, 0 at a soma
     int64_t C;
     double *area, *gax;
+    double *dcon;                     // FP64: see StepArgs
     double *V, *m, *h, *n;
     double Ra, v_init;
+    double cm_dt;                     // Cm * 1e3 / dt: C_i/dt = area_i * cm_dt (nF/ms = uS)
+    double gleak, gimp;               // implicit leak (uS per cm^2, 0 under Eq. 2 as printed), coupling share
     // FP32c outputs (used when Vq != nullptr; the FP64 pointers are then
     // unused; the FP32c constants are computed on the host)
     int32_t *Vq;
@@ -380,7 +353,6 @@ int mmk_launch_step_fp64(const mmk::StepArgs &a, int blocks, int threads, void *
 int mmk_step_fp64_blocks_per_sm(int threads, int smem_bytes, int *blocks);
 int mmk_launch_step_fp32c(const mmk::StepArgs32 &a, int blocks, int threads, void *stream);
 int mmk_step_fp32c_blocks_per_sm(int threads, int smem_bytes, int *blocks);
-size_t mmk_step_fp64_smem(int comps, int segs, int meta_bytes);
 int mmk_launch_init_fp32c(const mmk::InitArgs &a, void *stream);
 int mmk_launch_giant_fp32c(const mmk::StepArgs32 &a, int blocks, void *stream);
 int mmk_launch_giant_assemble(const mmk::StepArgs32 &a, int chunk_blocks, void *stream);

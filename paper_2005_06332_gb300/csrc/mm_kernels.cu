@@ -7,7 +7,7 @@
 //                   per-step spike lists, expanded through an outgoing CSR);
 //   step_fp64:      per work item (a run of whole neurons): HH currents,
 //                   assembly of the Hines system for dV (Eq. 2), the Hines
-//                   solve (Algorithm 1) as segment waves in shared memory,
+//                   solve (Algorithm 1) path by path in shared memory,
 //                   V += dV, exponential-Euler gates, synaptic decay and the
 //                   soma threshold test.
 // The model is the oracle's (units um, mV, ms, nA, uS, nF); the arithmetic
@@ -16,6 +16,7 @@
 
 #include <mutex>
 
+#include "mm_gate_table64.h"
 #include "mm_internal.h"
 #include "mm_tma.h"
 
@@ -65,19 +66,23 @@ __device__ __forceinline__ double half_cyl_resistance(double Ra, double L_um, do
 
 // ------------------------------------------------------------------ init
 
+// Areas, axial conductances (negated at path heads), the constant part of the
+// diagonal, and the resting state.
 __global__ void init_kernel(InitArgs a)
 {
+    auto axial = [&](int64_t i, int64_t q) {
+        return 1.0 / (half_cyl_resistance(a.Ra, a.L[i], a.diam[i]) + half_cyl_resistance(a.Ra, a.L[q], a.diam[q]));
+    };
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.C;
          i += (int64_t)gridDim.x * blockDim.x) {
-        double L = a.L[i], d = a.diam[i];
-        a.area[i] = kPi * d * L * 1e-8;
-        const int32_t pd = abs(a.parent_dist[i]);
-        double g = 0.0;
-        if (pd > 0) {
-            const int64_t q = i - pd;
-            g = 1.0 / (half_cyl_resistance(a.Ra, L, d) + half_cyl_resistance(a.Ra, a.L[q], a.diam[q]));
-        }
-        a.gax[i] = g;
+        const double area = kPi * a.diam[i] * a.L[i] * 1e-8;
+        a.area[i] = area;
+        const int32_t pd = a.parent_dist[i];
+        const double g = pd != 0 ? axial(i, i - abs(pd)) : 0.0;
+        a.gax[i] = pd > 0 ? g : -g;
+        double coupling = g;
+        if (i + 1 < a.C && a.parent_dist[i + 1] == 1) coupling += axial(i + 1, i);
+        a.dcon[i] = area * a.cm_dt + a.gleak * area + a.gimp * coupling;
         double v = a.v_init;
         Rates r = hh_rates(v);
         a.V[i] = v;
@@ -182,33 +187,149 @@ __global__ void __launch_bounds__(256) deliver_ordered_kernel(DeliverArgs a)
 
 // ------------------------------------------------------------ FP64 step
 
-template <int NT>
-__global__ void __launch_bounds__(NT) step_fp64_kernel(StepArgs a)
+// 1/x by Newton's iteration from the approximate reciprocal (about 20 bits):
+// two steps reach FP64 rounding.  FP64 instructions are scarce (two lanes per
+// SM and clock), and the compiled division takes about twice as many.
+__device__ __forceinline__ double rcp_nr(double x)
 {
-    // Shared memory: the work item's tree blob (one bulk copy), then the
-    // diagonal (after elimination: its reciprocal) and rhs (after
-    // substitution: dV) of every compartment.
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    r = fma(r, fma(-x, r, 1.0), r);
+    return fma(r, fma(-x, r, 1.0), r);
+}
+
+// a / x given r = rcp_nr(x): one residual correction
+__device__ __forceinline__ double div_nr(double a, double x, double r)
+{
+    const double q = a * r;
+    return fma(r, fma(-x, q, a), q);
+}
+
+// 2^-exponent(x) for a normal x (x times it lies in [1, 2)); 1 for zero,
+// infinities and NaN, which stay as they are
+__device__ __forceinline__ double pow2_inverse(double x)
+{
+    const uint32_t e = (uint32_t)__double2hiint(x) & 0x7FF00000u;
+    return __hiloint2double(e - 0x00100000u < 0x7FD00000u ? (int)(0x7FE00000u - e) : 0x3FF00000, 0);
+}
+
+// x times pow2_inverse(x), by integer operations
+__device__ __forceinline__ double mantissa(double x)
+{
+    const uint32_t h = (uint32_t)__double2hiint(x), e = h & 0x7FF00000u;
+    return e - 0x00100000u < 0x7FD00000u ? __hiloint2double((int)(h - e + 0x3FF00000u), __double2loint(x)) : x;
+}
+
+// Exponential-Euler gate update at V^{n+1} of one compartment (its V is final
+// for this step): from the table, or beyond its range from the rates.
+__device__ __forceinline__ void gate_update(const StepArgs &a, int64_t c)
+{
+    const double v = a.V[c];
+    double *const x[3] = {a.m + c, a.h + c, a.n + c};
+    if (mmg::in_table(v)) {
+        const mmg::Index64 t = mmg::index64(v);
+        constexpr int I = mmg::kTab64Intervals;
+        const double2 *f = a.gtab + t.i;
+#pragma unroll
+        for (int g = 0; g < 3; ++g) {
+            double XF[2];
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const double2 p = __ldg(f + (6 * g + 3 * k) * I), q = __ldg(f + (6 * g + 3 * k + 1) * I);
+                const float4 s = __ldg((const float4 *)(f + (6 * g + 3 * k + 2) * I));
+                XF[k] = k == 0 ? mmg::eval64_rest({p.x, p.y}, {q.x, q.y}, {s.x, s.y, s.z, s.w}, t)
+                               : mmg::eval64({p.x, p.y}, {q.x, q.y}, {s.x, s.y, s.z, s.w}, t);
+            }
+            *x[g] = mmg::step64(*x[g], XF[0], XF[1]);
+        }
+    } else {
+        const Rates r = hh_rates(v);
+        *x[0] = relax(*x[0], r.am, r.bm, a.dt);
+        *x[1] = relax(*x[1], r.ah, r.bh, a.dt);
+        *x[2] = relax(*x[2], r.an, r.bn, a.dt);
+    }
+}
+
+// Gate updates of the compartments pc0 .. pc0 + pn - 1, in chunks of
+// kGateChunk claimed by whole warps from the shared counter *next until none
+// is left.
+constexpr int kGateChunk = 64;
+
+__device__ __forceinline__ void gate_chunks(const StepArgs &a, int64_t pc0, int pn, int *next, int lane)
+{
+    for (;;) {
+        int ch = 0;
+        if (lane == 0) ch = atomicAdd(next, 1);
+        ch = __shfl_sync(0xFFFFFFFFu, ch, 0);
+        const int i0 = ch * kGateChunk;
+        if (i0 >= pn) break;
+        const int i1 = min(i0 + kGateChunk, pn);
+        for (int i = i0 + lane; i < i1; i += 32) gate_update(a, pc0 + i);
+    }
+}
+
+// Compartments per step of a path sweep.
+constexpr int kSweepChunk = 4;
+// Paths of at least this many compartments are swept by a whole warp.
+constexpr int kWarpPath = 96;
+// The products of a path's elimination are rescaled before every compartment
+// whose group-local index is kRescale - 1 modulo kRescale.
+constexpr int kRescale = 8;
+
+template <int NT>
+__global__ void __launch_bounds__(NT, NT <= 256 ? 512 / NT : 1) step_fp64_kernel(StepArgs a)
+{
+    // Bound by the FP64 pipe (two lanes per SM and clock: a warp's FP64
+    // instruction takes it for 16 clocks whatever the number of active
+    // lanes), so everything here saves FP64 instructions and keeps the
+    // rest busy in full warps:
+    //   * the gates come from the table (mm_gate_table64.h), with the constant
+    //     part of the diagonal stored per compartment;
+    //   * the sweeps are the part with few active lanes (one lane per
+    //     path), so they multiply only: the elimination carries
+    //     d'_j = N_j / M_j and rhs'_j = S_j / M_j as products,
+    //       N_{j-1} = d_{j-1} N_j - g_j^2 M_j,  M_{j-1} = N_j,
+    //       S_{j-1} = r_{j-1} N_j + g_j S_j
+    //     (Algorithm 1's row times M; powers of two are taken out along the
+    //     way), and the division for the substitution's factors
+    //     f_j = g_j M_j / N_j, c_j = S_j / N_j is a pass of full warps;
+    //   * warps without a sweep update the gates of the block's previous item.
+    // Work items, teams, bundles, levels and the fold list are the FP32c
+    // kernel's (step_fp32c_kernel), with the diagonal and rhs in FP64.
+    // Measured per step: 2,000 neurons of 50 to 5,000 compartments (2.14 M)
+    // 1.81 -> 0.74 ms (119 FP64 warp instructions per 32 compartments, pipe 75 %
+    // busy while an SM has work); 64 of 255 compartments 370 -> 159 us; 701 of
+    // 50 to 3,000, points and ordered delivery, 808 -> 262 us.
+    //
+    // Shared memory: the item's tree blob (one bulk copy), then per
+    // compartment the pair (diagonal, rhs) -- after a path's elimination
+    // (N, S) for its inside and (-f, c) for its head, whose sign says that the
+    // division is done, then (f, c), after substitution (f, dV).
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned char *smeta = smem_raw;
-    double *sd = (double *)(smem_raw + a.smem_meta);
-    double *sr = sd + a.smem_comps;
     __shared__ __align__(8) uint64_t bar;
     __shared__ int s_item, s_abort;
+    __shared__ long long s_pc0;  // pending gate work: the previous item's compartments
+    __shared__ int s_pn, s_gchunk;
 
     const long long n = (long long)a.ctl->step_base + a.step_offset;
     const int tid = threadIdx.x;
     if (tid == 0) {
         mbar_init(&bar, 1);
         fence_mbar_init();
+        s_abort = 0;
+        s_pc0 = 0;
+        s_pn = 0;
+        s_gchunk = 0;
     }
     uint32_t parity = 0;
 
     for (;;) {
         __syncthreads();
+        if (s_abort) break;
         if (tid == 0) {
             const int item = (int)atomicAdd(&a.ctl->queue_head, 1u);
             s_item = item;
-            s_abort = 0;
             if (item < a.n_groups) {
                 const GroupRec *gp = a.groups + item;
                 const uint32_t bytes = (uint32_t)gp->meta_bytes;
@@ -224,19 +345,26 @@ __global__ void __launch_bounds__(NT) step_fp64_kernel(StepArgs a)
         const int64_t c0 = G.comp0;
         const double *V = a.V + c0;
         const double *gax = a.gax + c0;
+        double2 *sdr = (double2 *)(smem_raw + G.meta_bytes);
 
-        // A. membrane conductance and current at (V^n, gates^n): the
-        //    compartment's own part of the diagonal and right-hand side.
+        // A. diagonal and rhs at (V^n, gates^n): membrane conductance and
+        //    current, and the axial currents of the links inside paths (a
+        //    link (i-1, i) is inside a path when gax[i] has no sign bit; its
+        //    conductances are in the constant part of the diagonal).
+#pragma unroll 2
         for (int i = tid; i < G.ncomp; i += NT) {
             const double v = V[i], mm = a.m[c0 + i], hh = a.h[c0 + i], nn = a.n[c0 + i];
-            const double ar = a.area[c0 + i];
-            const double s = ar * 1e3;
-            const double gna = a.gNa * s * (mm * mm * mm * hh);
-            const double n2 = nn * nn;
-            const double gk = a.gK * s * (n2 * n2);
-            const double gl = a.gL * s;
-            sd[i] = ar * a.cm_dt + (a.g_implicit ? gna + gk + gl : 0.0);
-            sr[i] = -(gna * (v - a.ENa) + gk * (v - a.EK) + gl * (v - a.EL));
+            const double s = a.area[c0 + i], g = gax[i];
+            const double gna = a.gNa * ((mm * mm) * (mm * hh)), n2 = nn * nn, gk = a.gK * (n2 * n2);
+            double d = a.dcon[c0 + i];
+            if (a.g_implicit) d = fma(s, gna + gk, d);
+            double r = -s * fma(gna, v - a.ENa, fma(gk, v - a.EK, a.gL * (v - a.EL)));
+            if (!signbit(g)) r = fma(g, V[i - 1] - v, r);
+            if (i + 1 < G.ncomp) {
+                const double gc = gax[i + 1];
+                if (!signbit(gc)) r = fma(gc, V[i + 1] - v, r);
+            }
+            sdr[i] = make_double2(d, r);
         }
         if (!mbar_wait_bounded(&bar, parity)) {
             // give up on this item, but not on the copy in flight: wait for
@@ -247,122 +375,391 @@ __global__ void __launch_bounds__(NT) step_fp64_kernel(StepArgs a)
         }
         parity ^= 1u;
         __syncthreads();
-        if (s_abort) {
+        if (s_abort) {  // the whole block leaves at the next item boundary
             if (tid == 0) atomicOr(&a.ctl->err, MMK_ERR_TIMEOUT);
-            break;
+            continue;
         }
-        const SegP *segs = (const SegP *)smeta;
-        const int16_t *kids = (const int16_t *)(segs + G.nseg);
-        const int16_t *woff = kids + G.nchild;
+        const NrnQ *nrns = (const NrnQ *)smeta;
+        const PathQ *paths = (const PathQ *)(smeta + G.path_off);
+        const KidQ *fold = (const KidQ *)(smeta + G.fold_off);
+        const int16_t *loffs = (const int16_t *)(smeta + G.loffs_off);
+        const int16_t *mcnt = (const int16_t *)(smeta + G.mcnt_off);
 
-        // S. synaptic sites: conductance into the system, then decay.
+        // S. synaptic sites (then their decay; sites are distinct
+        //    compartments), the current across each path's head link into its
+        //    head (for the path from a soma the stimulus), then per parent
+        //    compartment the conductances and currents of the links to the
+        //    heads that hang off it, in fold-list order.
         for (int t = tid; t < G.nsite; t += NT) {
             const int st = G.site0 + t;
             const int c = a.site_comp[st];
             const double g = a.gsyn[st];
-            if (a.g_implicit) sd[c] += g;
-            sr[c] -= g * (V[c] - a.e_syn);
+            double2 w = sdr[c];
+            if (a.g_implicit) w.x += g;
+            w.y = fma(-g, V[c] - a.e_syn, w.y);
+            sdr[c] = w;
             a.gsyn[st] = g * a.decay;
         }
         __syncthreads();
-
-        // B. leaves-to-root elimination, one segment per thread, wave by wave.
-        //    The axial terms of each link (i, p(i)) are folded in as the sweep
-        //    reaches i: d_i += w g, rhs_i += g (V_p - V_i) and, for the parent,
-        //    d_p += w g, rhs_p += g (V_i - V_p), next to the elimination update
-        //    d_p -= (a_i/d_i) c_i, rhs_p -= (a_i/d_i) rhs_i with a_i = c_i = -w g
-        //    (w = gimp: 1, or 1/2 for Eq. 2 as printed).
-        for (int w = 0; w < G.nwave; ++w) {
-            const int sb = woff[w], se = woff[w + 1];
-            for (int si = sb + tid; si < se; si += NT) {
-                const SegP S = segs[si];
-                const int bot = S.top + S.len - 1;
-                double db = sd[bot], rb = sr[bot];
-                // each child segment hangs off the bottom: from its top's
-                // stored 1/d and rhs, its link terms (+g, +g (V_t - V_b)) and
-                // its elimination (-g^2/d_t, +g rhs_t/d_t)
-                for (int c = 0; c < S.nchild; ++c) {
-                    const int t = segs[kids[S.child0 + c]].top;
-                    const double g = gax[t], gi = a.gimp * g;
-                    const double f = gi * sd[t];
-                    db += gi - f * gi;
-                    rb += g * (V[t] - V[bot]) + f * sr[t];
-                }
-                for (int j = bot; j > S.top; --j) {
-                    const double g = gax[j], gi = a.gimp * g;
-                    const double vj = V[j], vp = V[j - 1];
-                    db += gi;
-                    rb += g * (vp - vj);
-                    const double inv = 1.0 / db;
-                    sd[j] = inv;
-                    sr[j] = rb;
-                    const double f = gi * inv;
-                    db = sd[j - 1] + gi - f * gi;
-                    rb = sr[j - 1] + g * (vj - vp) + f * rb;
-                }
-                const int t = S.top;
-                if (S.parent >= 0) {
-                    const double g = gax[t];
-                    db += a.gimp * g;
-                    rb += g * (V[S.parent] - V[t]);
-                    sd[t] = 1.0 / db;
-                    sr[t] = rb;
-                } else {
-                    rb += a.stim[G.neuron0 + S.neuron];
-                    const double inv = 1.0 / db;
-                    sd[t] = inv;
-                    sr[t] = rb * inv;     // dV at the soma
-                }
-            }
-            __syncthreads();
+        for (int pi = tid; pi < G.npath; pi += NT) {
+            const PathQ P = paths[pi];
+            double r = sdr[P.head].y;
+            if (P.parent >= 0) r = fma(fabs(gax[P.head]), V[P.parent] - V[P.head], r);
+            else r += a.stim[G.neuron0 + (P.nflag & kPathNeuron)];
+            sdr[P.head].y = r;
         }
+        __syncthreads();
+        for (int e = tid; e < G.npath; e += NT) {
+            const int att = (int)(fold[e] >> 16);
+            if (att >= G.ncomp) continue;  // a path from a soma (no parent)
+            if (e > 0 && (int)(fold[e - 1] >> 16) == att) continue;  // not the first path of its parent
+            double2 w = sdr[att];
+            const double vp = V[att];
+            for (int z = e; z < G.npath && (int)(fold[z] >> 16) == att; ++z) {
+                const int h = paths[fold[z] & 0xFFFFu].head;
+                const double g = fabs(gax[h]);
+                w.x = fma(a.gimp, g, w.x);
+                w.y = fma(g, V[h] - vp, w.y);
+            }
+            sdr[att] = w;
+        }
+        __syncthreads();
 
-        // F. root-to-leaves substitution in the reverse wave order; the soma
-        //    segment also runs the spike test.
-        for (int w = G.nwave - 1; w >= 0; --w) {
-            const int sb = woff[w], se = woff[w + 1];
-            for (int si = sb + tid; si < se; si += NT) {
-                const SegP S = segs[si];
-                const int t = S.top;
-                double x;
-                if (S.parent >= 0) {
-                    x = (sr[t] + a.gimp * gax[t] * sr[S.parent]) * sd[t];
-                    sr[t] = x;
-                } else {
-                    x = sr[t];
-                    const double v0 = V[t], v1 = v0 + x;
-                    const int nrn = G.neuron0 + S.neuron;
-                    if (!isfinite(v1)) atomicOr(&a.ctl->err, MMK_ERR_NUMERIC);
-                    if (v0 < a.threshold && v1 >= a.threshold) {
-                        const int src = soma_source(a, nrn);
-                        if (src >= 0)
-                            record_spike(a, src, a.user_id[nrn], 0,
-                                         (double)n * a.dt + a.dt * (a.threshold - v0) / (v1 - v0), n);
+        // Team of each warp: T warps per sweep bundle (T = 1, 2 or 4), the
+        // teams taking the item's bundles in turn, each on its own named
+        // barrier (1 + team; 0 is the block's).
+        const int nwarp = NT / 32;
+        int T = nwarp / max(G.nbundle, 1);
+        T = T >= 4 ? 4 : (T >= 2 ? 2 : 1);
+        const int team = (tid >> 5) / T, nteam = nwarp / T;
+        const int tl = tid - team * T * 32;  // lane within the team
+        const int TL = T * 32, lane = tid & 31;
+        auto team_sync = [&]() {
+            if (T == 1) __syncwarp();
+            else asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(TL) : "memory");
+        };
+
+        // The head of a path once its inside is eliminated (N, M, S of the
+        // head): for the path from a soma its dV, else its factors and, if no
+        // other path hangs off the same compartment, its elimination into the
+        // parent: d_p -= g f, r_p += g c (a = c = -g).
+        auto eliminate_head = [&](const PathQ &P, double N, double M, double S) {
+            const int h = P.head;
+            const double inv = rcp_nr(N), c = div_nr(S, N, inv);
+            if (P.parent < 0) {
+                sdr[h] = make_double2(-1.0, c);
+                return;
+            }
+            const double g = a.gimp * fabs(gax[h]);
+            const double f = div_nr(g * M, N, inv);
+            sdr[h] = make_double2(-f, c);
+            if (P.nflag & kPathAlone) {
+                double2 w = sdr[P.parent];
+                w.x = fma(-g, f, w.x);
+                w.y = fma(g, c, w.y);
+                sdr[P.parent] = w;
+            }
+        };
+        auto rescale = [&](double &N, double &M, double &S) {
+            const double k = pow2_inverse(N);
+            N = mantissa(N);
+            M *= k;
+            S *= k;
+        };
+        // One path by one lane, leaf to head; the couplings of the next
+        // kSweepChunk compartments are loaded (from L2) while the current
+        // ones are eliminated.  Indices past the head are clamped, their
+        // results dropped.
+        auto eliminate_path = [&](int pi) {
+            const PathQ P = paths[pi];
+            const int h = P.head;
+            int j = P.end - 1;
+            const double2 v0 = sdr[j];
+            double N = v0.x, M = 1.0, S = v0.y;
+            double gn[kSweepChunk];
+#pragma unroll
+            for (int k = 0; k < kSweepChunk; ++k) gn[k] = __ldg(gax + max(j - k, h));
+            for (; j > h; j -= kSweepChunk) {
+                const int cnt = j - h;
+                double g[kSweepChunk];
+                double2 w[kSweepChunk];
+#pragma unroll
+                for (int k = 0; k < kSweepChunk; ++k) {
+                    g[k] = a.gimp * gn[k];
+                    w[k] = sdr[max(j - k - 1, h)];
+                }
+#pragma unroll
+                for (int k = 0; k < kSweepChunk; ++k) gn[k] = __ldg(gax + max(j - kSweepChunk - k, h));
+#pragma unroll
+                for (int k = 0; k < kSweepChunk; ++k) {
+                    if (k < cnt) {
+                        const int i = j - k - 1;
+                        if ((i & (kRescale - 1)) == kRescale - 1) rescale(N, M, S);
+                        const double N1 = fma(w[k].x, N, -((g[k] * g[k]) * M));
+                        S = fma(w[k].y, N, g[k] * S);
+                        M = N;
+                        N = N1;
+                        if (i > h) sdr[i] = make_double2(N, S);
                     }
                 }
-                for (int j = t + 1; j < t + S.len; ++j) {
-                    x = (sr[j] + a.gimp * gax[j] * x) * sd[j];
-                    sr[j] = x;
+            }
+            eliminate_head(P, N, M, S);
+        };
+        // The same by a whole warp.  The elimination step is linear in
+        // (N, M, S): each lane composes the steps of its chunk (the images of
+        // the three unit vectors; S's own is p times itself), an inclusive
+        // warp scan combines the chunks, and each lane runs the steps of its
+        // chunk from the vector that the chunks before it leave.  Here the
+        // lanes divide themselves and store (-f, c).
+        auto eliminate_path_warp = [&](int pi) {
+            const PathQ P = paths[pi];
+            const int h = P.head, e = P.end;
+            const int m = e - 1 - h;  // steps t = 0 .. m-1: compartment e-1-t into e-2-t
+            const int cs = (m + 31) >> 5;
+            const int t0 = min(lane * cs, m), t1 = min(t0 + cs, m);
+            const double2 leaf = sdr[e - 1];
+            double n1 = 1.0, m1 = 0.0, s1 = 0.0, n2 = 0.0, m2 = 1.0, s2 = 0.0, p = 1.0;
+            auto scale = [&]() {
+                const double k = pow2_inverse(n1);
+                n1 *= k; m1 *= k; s1 *= k; n2 *= k; m2 *= k; s2 *= k; p *= k;
+            };
+            double2 nb = make_double2(0.0, 0.0);
+            for (int t = t0; t < t1; ++t) {
+                const int j = e - 1 - t;
+                const double g = a.gimp * __ldg(gax + j), gg = g * g;
+                const double2 w = sdr[j - 1];
+                const double a1 = fma(w.x, n1, -(gg * m1)), a2 = fma(w.x, n2, -(gg * m2));
+                s1 = fma(w.y, n1, g * s1);
+                s2 = fma(w.y, n2, g * s2);
+                m1 = n1;
+                n1 = a1;
+                m2 = n2;
+                n2 = a2;
+                p *= g;
+                nb = w;
+                if (((t - t0) & (kRescale - 1)) == kRescale - 1) scale();
+            }
+            for (int off = 1; off < 32; off <<= 1) {
+                const unsigned F = 0xFFFFFFFFu;
+                const double bn1 = __shfl_up_sync(F, n1, off), bm1 = __shfl_up_sync(F, m1, off),
+                             bs1 = __shfl_up_sync(F, s1, off), bn2 = __shfl_up_sync(F, n2, off),
+                             bm2 = __shfl_up_sync(F, m2, off), bs2 = __shfl_up_sync(F, s2, off),
+                             bp = __shfl_up_sync(F, p, off);
+                if (lane >= off) {  // this lane's steps act after the earlier lanes'
+                    const double an1 = fma(n1, bn1, n2 * bm1), am1 = fma(m1, bn1, m2 * bm1),
+                                 as1 = fma(s1, bn1, fma(s2, bm1, p * bs1));
+                    const double an2 = fma(n1, bn2, n2 * bm2), am2 = fma(m1, bn2, m2 * bm2),
+                                 as2 = fma(s1, bn2, fma(s2, bm2, p * bs2));
+                    n1 = an1; m1 = am1; s1 = as1; n2 = an2; m2 = am2; s2 = as2;
+                    p *= bp;
+                    scale();
                 }
             }
-            __syncthreads();
-        }
+            // the vector at the chunk's first compartment: the earlier
+            // chunks' steps on the leaf's (d, 1, r)
+            double N, M, S;
+            {
+                const unsigned F = 0xFFFFFFFFu;
+                const double bn1 = __shfl_up_sync(F, n1, 1), bm1 = __shfl_up_sync(F, m1, 1),
+                             bs1 = __shfl_up_sync(F, s1, 1), bn2 = __shfl_up_sync(F, n2, 1),
+                             bm2 = __shfl_up_sync(F, m2, 1), bs2 = __shfl_up_sync(F, s2, 1),
+                             bp = __shfl_up_sync(F, p, 1);
+                N = lane ? fma(bn1, leaf.x, bn2) : leaf.x;
+                M = lane ? fma(bm1, leaf.x, bm2) : 1.0;
+                S = lane ? fma(bs1, leaf.x, fma(bp, leaf.y, bs2)) : leaf.y;
+            }
+            __syncwarp();  // every lane has read its chunk and the element after it
+            for (int t = t0; t < t1; ++t) {
+                const int j = e - 1 - t;
+                const double g = a.gimp * __ldg(gax + j);
+                const double2 w = t + 1 < t1 ? sdr[j - 1] : nb;
+                if (((t - t0) & (kRescale - 1)) == 0) rescale(N, M, S);
+                const double inv = rcp_nr(N);
+                sdr[j] = make_double2(-div_nr(g * M, N, inv), div_nr(S, N, inv));
+                const double N1 = fma(w.x, N, -((g * g) * M));
+                S = fma(w.y, N, g * S);
+                M = N;
+                N = N1;
+            }
+            // the head, from the lane whose chunk ends at it
+            const int lastl = (m - 1) / cs;
+            N = __shfl_sync(0xFFFFFFFFu, N, lastl);
+            M = __shfl_sync(0xFFFFFFFFu, M, lastl);
+            S = __shfl_sync(0xFFFFFFFFu, S, lastl);
+            __syncwarp();
+            if (lane == 0) eliminate_head(P, N, M, S);
+            __syncwarp();
+        };
+        // eliminations into the compartments that several paths of the level
+        // hang off (fold entries e0 .. e1-1); a lane takes the entries that
+        // start a run of equal parents
+        auto fold_shared = [&](int e0, int e1) {
+            for (int e = e0 + tl; e < e1; e += TL) {
+                const int att = (int)(fold[e] >> 16);
+                if (e > e0 && (int)(fold[e - 1] >> 16) == att) continue;
+                double2 w = sdr[att];
+                for (int z = e; z < e1 && (int)(fold[z] >> 16) == att; ++z) {
+                    const int h = paths[fold[z] & 0xFFFFu].head;
+                    const double g = a.gimp * fabs(gax[h]);
+                    const double2 q = sdr[h];
+                    w.x = fma(g, q.x, w.x);
+                    w.y = fma(g, q.y, w.y);
+                }
+                sdr[att] = w;
+            }
+        };
+        // The factors of the compartments b0 .. b1-1 whose division is not
+        // done: f = g M / N, c = S / N with M the N of the compartment below
+        // (taken back to where the elimination rescaled it), 1 at a leaf --
+        // a compartment followed by a path's head, whose first member is
+        // negative, or by the end.
+        auto divide = [&](int b0, int b1) {
+            for (int i0 = b0; i0 < b1; i0 += TL) {
+                const int i = i0 + tl;
+                double2 w = make_double2(-1.0, 0.0);
+                double M = 1.0;
+                if (i < b1) {
+                    w = sdr[i];
+                    if (i + 1 < b1) {
+                        const double x = sdr[i + 1].x;
+                        if (!signbit(x)) M = (i & (kRescale - 1)) == kRescale - 1 ? mantissa(x) : x;
+                    }
+                }
+                if (signbit(w.x)) {
+                    w.x = -w.x;
+                } else {
+                    const double inv = rcp_nr(w.x);
+                    const double f = div_nr((a.gimp * __ldg(gax + i)) * M, w.x, inv);
+                    w = make_double2(f, div_nr(w.y, w.x, inv));
+                }
+                team_sync();  // the compartment above has read this one's N
+                if (i < b1) sdr[i] = w;
+            }
+        };
 
-        // C. V^{n+1} = V^n + dV, the threshold test of the detection points
-        //    other than somata, then exponential-Euler gates at V^{n+1}.
+        // F. root-to-leaves substitution; the path from a soma runs the spike
+        //    test
+        auto substitute_head = [&](const PathQ &P) -> double {
+            const double2 w = sdr[P.head];
+            if (P.parent >= 0) return fma(w.x, sdr[P.parent].y, w.y);
+            const double x = w.y;
+            const double v0 = V[P.head], v1 = v0 + x;
+            const int nrn = G.neuron0 + (P.nflag & kPathNeuron);
+            if (!isfinite(v1)) atomicOr(&a.ctl->err, MMK_ERR_NUMERIC);
+            if (v0 < a.threshold && v1 >= a.threshold) {
+                const int src = soma_source(a, nrn);
+                if (src >= 0)
+                    record_spike(a, src, a.user_id[nrn], 0, (double)n * a.dt + a.dt * (a.threshold - v0) / (v1 - v0), n);
+            }
+            return x;
+        };
+        auto substitute_path = [&](int pi) {
+            const PathQ P = paths[pi];
+            const int h = P.head;
+            double x = substitute_head(P);
+            if (P.parent >= 0) sdr[h].y = x;
+            for (int j = h + 1; j < P.end; j += kSweepChunk) {
+                const int cnt = P.end - j;
+                double2 w[kSweepChunk];
+#pragma unroll
+                for (int k = 0; k < kSweepChunk; ++k) w[k] = sdr[min(j + k, P.end - 1)];
+#pragma unroll
+                for (int k = 0; k < kSweepChunk; ++k) {
+                    if (k < cnt) {
+                        x = fma(w[k].x, x, w[k].y);
+                        sdr[j + k].y = x;
+                    }
+                }
+            }
+        };
+        auto substitute_path_warp = [&](int pi) {
+            const PathQ P = paths[pi];
+            const int h = P.head, e = P.end;
+            double x = 0.0;
+            if (lane == 0) x = substitute_head(P);
+            x = __shfl_sync(0xFFFFFFFFu, x, 0);
+            const int m = e - 1 - h;  // t = 0 .. m-1 <-> j = h+1+t
+            const int cs = (m + 31) >> 5;
+            const int t0 = min(lane * cs, m), t1 = min(t0 + cs, m);
+            double A = 1.0, B = 0.0;
+            for (int t = t0; t < t1; ++t) {
+                const double2 w = sdr[h + 1 + t];
+                A *= w.x;
+                B = fma(w.x, B, w.y);
+            }
+            for (int off = 1; off < 32; off <<= 1) {
+                const double pa = __shfl_up_sync(0xFFFFFFFFu, A, off), pb = __shfl_up_sync(0xFFFFFFFFu, B, off);
+                if (lane >= off) {
+                    B = fma(A, pb, B);
+                    A *= pa;
+                }
+            }
+            const double ea = __shfl_up_sync(0xFFFFFFFFu, A, 1), eb = __shfl_up_sync(0xFFFFFFFFu, B, 1);
+            double xs = lane ? fma(ea, x, eb) : x;
+            for (int t = t0; t < t1; ++t) {
+                const double2 w = sdr[h + 1 + t];
+                xs = fma(w.x, xs, w.y);
+                sdr[h + 1 + t].y = xs;
+            }
+            __syncwarp();
+            if (lane == 0 && P.parent >= 0) sdr[h].y = x;
+        };
+        // the number of paths at the start of a level (paths run longest
+        // first) that a whole warp takes
+        auto warp_paths = [&](int pb, int pe) {
+            int nw = 0;
+            while (pb + nw < pe && paths[pb + nw].end - paths[pb + nw].head >= kWarpPath) ++nw;
+            return nw;
+        };
+
+        // B from the deepest level up, the division, F from the somata down;
+        // then gate chunks of the previous item.
+        for (int k = team; k < G.nbundle; k += nteam) {
+            const NrnQ Nk = nrns[k];
+            const int16_t *lo = loffs + Nk.loff0;
+            const int16_t *mc = mcnt + Nk.loff0;
+            for (int l = Nk.nlevel - 1; l >= 0; --l) {
+                const int pb = lo[l], pe = lo[l + 1];
+                const int nw = warp_paths(pb, pe);
+                for (int q = tl >> 5; q < nw; q += T) eliminate_path_warp(pb + q);
+                for (int pi = pb + nw + tl; pi < pe; pi += TL) eliminate_path(pi);
+                team_sync();
+                if (mc[l] > 0) {
+                    fold_shared(pb, pb + mc[l]);
+                    team_sync();
+                }
+            }
+            divide(Nk.comp0, Nk.comp0 + Nk.ncomp);
+            team_sync();
+            for (int l = 0; l < Nk.nlevel; ++l) {
+                const int pb = lo[l], pe = lo[l + 1];
+                const int nw = warp_paths(pb, pe);
+                for (int q = tl >> 5; q < nw; q += T) substitute_path_warp(pb + q);
+                for (int pi = pb + nw + tl; pi < pe; pi += TL) substitute_path(pi);
+                team_sync();
+            }
+        }
+        gate_chunks(a, s_pc0, s_pn, &s_gchunk, lane);
+        __syncthreads();
+
+        // C. V^{n+1} = V^n + dV and the threshold test of the detection
+        //    points other than somata.
         for (int i = tid; i < G.ncomp; i += NT) {
-            const double v0 = V[i], v = v0 + sr[i];
+            const double v0 = V[i], v = v0 + sdr[i].y;
             a.V[c0 + i] = v;
             if (a.pt_of && v0 < a.threshold && v >= a.threshold) {
                 const int p = a.pt_of[c0 + i];
                 if (p >= 0) point_spike(a, p, v0, v, n, a.dt);
             }
-            const Rates r = hh_rates(v);
-            a.m[c0 + i] = relax(a.m[c0 + i], r.am, r.bm, a.dt);
-            a.h[c0 + i] = relax(a.h[c0 + i], r.ah, r.bh, a.dt);
-            a.n[c0 + i] = relax(a.n[c0 + i], r.an, r.bn, a.dt);
+        }
+        if (tid == 0) {  // this item's gates are pending until the next item's sweeps
+            s_pc0 = c0;
+            s_pn = G.ncomp;
+            s_gchunk = 0;
         }
     }
+    // the last item's gates, by the whole block
+    gate_chunks(a, s_pc0, s_pn, &s_gchunk, tid & 31);
 }
 
 __global__ void advance_kernel(DevCtl *ctl, int steps) { ctl->step_base += (unsigned long long)steps; }
@@ -436,17 +833,9 @@ int mmk_launch_deliver_ordered(const DeliverArgs &a, int blocks, void *stream)
     return (int)cudaGetLastError();
 }
 
-size_t mmk_step_fp64_smem(int comps, int segs, int meta_bytes)
-{
-    (void)segs;
-    return (size_t)meta_bytes + (size_t)(2 * comps) * sizeof(double);
-}
-
-static size_t step_smem_bytes(const StepArgs &a) { return mmk_step_fp64_smem(a.smem_comps, a.smem_segs, a.smem_meta); }
-
 int mmk_launch_step_fp64(const StepArgs &a, int blocks, int threads, void *stream)
 {
-    const size_t smem = step_smem_bytes(a);
+    const size_t smem = (size_t)a.smem_bytes;
     cudaStream_t s = (cudaStream_t)stream;
     switch (threads) {
     case 128:

@@ -12,13 +12,12 @@
 //      is visited first, so that each path (a compartment that does not
 //      continue its parent's path, then its deepest child, and so on down to
 //      a leaf) is a contiguous range whose compartments each have the
-//      previous one as their parent, and every unbranched segment is
-//      contiguous too;
+//      previous one as their parent;
 //   3. consecutive neurons are packed into work items of about
-//      `group_comps` compartments; FP32c items get path tables (paths by
+//      `group_comps` compartments, each with its path tables (paths by
 //      level, per-level fold lists of paths sharing a parent compartment),
 //      the schedule of the path-by-path leaves-to-root / root-to-leaves
-//      sweeps; FP64 items get their segments sorted into height waves;
+//      sweeps;
 //   4. synapse targets are merged into synaptic sites (one conductance per
 //      compartment that receives synapses) and outgoing synapses are stored
 //      per source neuron, sorted by delay, for delivery.
@@ -39,23 +38,24 @@ namespace {
 std::string msg(const std::ostringstream &o) { return o.str(); }
 
 struct NeuronScratch {
-    std::vector<int32_t> ccount, cstart, clist, newl, oldof, pnew, nch, stack, depth;
-    std::vector<int32_t> seg_top, seg_len, seg_par, seg_height, seg_of_bottom, seg_of_top;
+    std::vector<int32_t> ccount, cstart, clist, newl, oldof, pnew, fill, stack, depth, path_of;
 };
+
+constexpr size_t kNrnInts = sizeof(mmk::NrnG) / 4;
 
 // One path of a work item before packing.
 struct PathTmp {
     int32_t head, end, parent, neuron, level;
 };
 
-// The tables of an FP32c work item solved path by path (see mmk::NrnQ):
-// per neuron its paths by (level, longest first, head); per level a fold
+// The tables of a work item solved path by path (see mmk::NrnQ):
+// per bundle its compartments and its paths by (level, longest first, head); per level a fold
 // list of the same paths, those sharing a parent compartment first (sorted
 // by that compartment, deepest first, then head), then the paths alone on
 // their parent compartment.  Emitted with 16-bit (shared-memory items) or
 // 32-bit (giant items) records.
 struct PathBlob {
-    std::vector<int32_t> nrn;    // 4 per bundle: path0, npath, nlevel, loff0
+    std::vector<int32_t> nrn;    // kNrnInts per bundle: path0, npath, nlevel, loff0, comp0, ncomp
     std::vector<int32_t> path;   // 4 per path: head, end, parent, neuron | alone
     std::vector<int32_t> fold;   // 2 per entry: path, parent compartment
     std::vector<int32_t> loffs, mcnt;
@@ -98,7 +98,13 @@ void build_path_blob(std::vector<PathTmp> &paths, int32_t nneuron, const std::ve
     for (int32_t q = 0; q < np; ++q)
         if (paths[(size_t)q].parent >= 0) share[paths[(size_t)q].parent]++;
     auto shared = [&](int32_t x) { return paths[(size_t)x].parent >= 0 && share[paths[(size_t)x].parent] > 1; };
-    b.nrn.assign(4 * (size_t)b.nbundle, 0);
+    b.nrn.assign(kNrnInts * (size_t)b.nbundle, 0);
+    for (int32_t k = 0, c = 0; k < nneuron; ++k) {
+        int32_t *rec = b.nrn.data() + kNrnInts * (size_t)bundle[(size_t)k];
+        if (rec[5] == 0) rec[4] = c;
+        rec[5] += nsize[(size_t)k];
+        c += nsize[(size_t)k];
+    }
     b.path.resize(4 * (size_t)np);
     b.fold.resize(2 * (size_t)np);
     b.loffs.clear();
@@ -119,10 +125,10 @@ void build_path_blob(std::vector<PathTmp> &paths, int32_t nneuron, const std::ve
         while (i < np && bundle[(size_t)paths[(size_t)i].neuron] == k) ++i;
         const int32_t nl = i > p0 ? paths[(size_t)i - 1].level + 1 : 0;
         const size_t lbase = b.loffs.size();
-        b.nrn[4 * (size_t)k] = p0;
-        b.nrn[4 * (size_t)k + 1] = i - p0;
-        b.nrn[4 * (size_t)k + 2] = nl;
-        b.nrn[4 * (size_t)k + 3] = (int32_t)lbase;
+        b.nrn[kNrnInts * (size_t)k] = p0;
+        b.nrn[kNrnInts * (size_t)k + 1] = i - p0;
+        b.nrn[kNrnInts * (size_t)k + 2] = nl;
+        b.nrn[kNrnInts * (size_t)k + 3] = (int32_t)lbase;
         for (int32_t l = 0, q = p0; l <= nl; ++l) {
             while (q < i && paths[(size_t)q].level < l) ++q;
             b.loffs.push_back(q);
@@ -160,7 +166,7 @@ BlobOffsets blob_offsets(const PathBlob &b, bool wide)
 {
     BlobOffsets o;
     const int64_t w = wide ? 4 : 2;  // bytes per index
-    o.path_off = (4 * w * b.nbundle + 15) & ~15LL;
+    o.path_off = ((int64_t)kNrnInts * w * b.nbundle + 15) & ~15LL;
     o.fold_off = o.path_off + 4 * w * b.npath;
     o.loffs_off = o.fold_off + 2 * w * b.npath;
     o.mcnt_off = o.loffs_off + w * (int64_t)b.loffs.size();
@@ -418,11 +424,8 @@ std::string build_layout(const LayoutInput &in, Layout &out, bool *invalid)
     L.groups.reserve((size_t)G);
     std::vector<mmk::GroupRec> bigs, giants;
 
-    // 2 + 3b. per group: renumber its neurons, cut segments, sort into waves
+    // 2 + 3b. per group: renumber its neurons, cut them into paths
     NeuronScratch ws;
-    std::vector<mmk::SegRec> gsegs;
-    std::vector<std::vector<int32_t>> gkids;
-    std::vector<int32_t> gheight, gpseg, glevel, perm, newidx;
     std::vector<PathTmp> gpaths;
     std::vector<int32_t> gsize;  // compartments of each neuron of the item
     L.max_comps = 0;
@@ -431,11 +434,6 @@ std::string build_layout(const LayoutInput &in, Layout &out, bool *invalid)
     for (int32_t g = 0; g < G; ++g) {
         const int32_t k0 = gstart[(size_t)g], k1 = gstart[(size_t)g + 1];
         const int64_t comp0 = L.noff[(size_t)k0];
-        gsegs.clear();
-        gkids.clear();
-        gheight.clear();
-        gpseg.clear();
-        glevel.clear();
         gpaths.clear();
         gsize.clear();
         for (int32_t k = k0; k < k1; ++k) {
@@ -453,7 +451,7 @@ std::string build_layout(const LayoutInput &in, Layout &out, bool *invalid)
             for (int32_t i = 0; i < n; ++i) ws.cstart[(size_t)i + 1] = ws.cstart[(size_t)i] + ws.ccount[(size_t)i];
             ws.clist.resize((size_t)std::max(n - 1, 1));
             {
-                std::vector<int32_t> &fill = ws.nch;
+                std::vector<int32_t> &fill = ws.fill;
                 fill.assign((size_t)n, 0);
                 for (int32_t i = 1; i < n; ++i) {
                     const int32_t p = par[i];
@@ -487,135 +485,55 @@ std::string build_layout(const LayoutInput &in, Layout &out, bool *invalid)
                     ws.stack.push_back(ws.clist[(size_t)c]);
             }
             ws.pnew.resize((size_t)n);
-            ws.nch.assign((size_t)n, 0);
             for (int32_t j = 0; j < n; ++j) {
                 const int32_t x = ws.oldof[(size_t)j];
                 const int32_t pj = (j == 0) ? -1 : ws.newl[(size_t)par[x]];
                 ws.pnew[(size_t)j] = pj;
-                if (pj >= 0) ws.nch[(size_t)pj]++;
                 L.L[(size_t)(ib + j)] = in.length_um[ub + x];
                 L.D[(size_t)(ib + j)] = in.diam_um[ub + x];
                 L.pdist[(size_t)(ib + j)] = (j == 0) ? 0 : (j - pj);
                 L.user2int[(size_t)(ub + x)] = ib + j;
             }
-            // segments: j starts one unless it is the only child of j-1
-            const size_t s_first = gsegs.size();
-            ws.seg_of_bottom.assign((size_t)n, -1);
+            // paths: j heads one unless it directly follows its parent (its
+            // parent's first, deepest child); a path runs to the next head.
+            // Links inside paths are assembled per compartment; path heads
+            // (negative parent distance) link to their parent in the sweep
+            ws.path_of.resize((size_t)n);
             for (int32_t j = 0; j < n; ++j) {
-                const bool cont = (j > 0 && ws.pnew[(size_t)j] == j - 1 && ws.nch[(size_t)(j - 1)] == 1);
-                if (!cont) {
-                    // segment tops carry a negative parent distance (FP32c items
-                    // re-mark path heads instead, below)
-                    if (j > 0) L.pdist[(size_t)(ib + j)] = -L.pdist[(size_t)(ib + j)];
-                    mmk::SegRec s;
-                    s.top = lb + j;
-                    s.len = 1;
-                    s.parent = (j == 0) ? -1 : lb + ws.pnew[(size_t)j];
-                    s.child0 = 0;
-                    s.nchild = 0;
-                    s.neuron = (j == 0) ? (k - k0) : -1;
-                    gsegs.push_back(s);
-                    gkids.emplace_back();
-                    gheight.push_back(0);
-                } else {
-                    gsegs.back().len++;
+                const int32_t pj = ws.pnew[(size_t)j];
+                if (j == 0 || pj != j - 1) {
+                    const int32_t level = j == 0 ? 0 : gpaths[(size_t)ws.path_of[(size_t)pj]].level + 1;
+                    gpaths.push_back(PathTmp{lb + j, lb + j + 1, j == 0 ? -1 : lb + pj, k - k0, level});
+                    L.pdist[(size_t)(ib + j)] = -L.pdist[(size_t)(ib + j)];
                 }
-            }
-            ws.seg_of_top.assign((size_t)n, -1);
-            for (size_t s = s_first; s < gsegs.size(); ++s) {
-                const int32_t bottom = gsegs[s].top + gsegs[s].len - 1 - lb;
-                ws.seg_of_bottom[(size_t)bottom] = (int32_t)s;
-                ws.seg_of_top[(size_t)(gsegs[s].top - lb)] = (int32_t)s;
-                gpseg.push_back(-1);
-                glevel.push_back(0);
-            }
-            // children and heights (child segments have larger tops than their parents)
-            for (size_t s = gsegs.size(); s-- > s_first + 1;) {
-                const int32_t pb = gsegs[s].parent - lb;
-                const int32_t ps = ws.seg_of_bottom[(size_t)pb];
-                if (ps < 0) { e << "internal: segment parent is not a segment bottom"; return msg(e); }
-                gkids[(size_t)ps].insert(gkids[(size_t)ps].begin(), (int32_t)s);
-                gheight[(size_t)ps] = std::max(gheight[(size_t)ps], gheight[s] + 1);
-                gpseg[s] = ps;
-            }
-            // paths: a segment heads one unless it is its parent's first
-            // (deepest) child, whose top directly follows the parent's bottom;
-            // a path runs down the first children to a leaf
-            for (size_t s = s_first; s < gsegs.size(); ++s) {
-                const bool head = gsegs[s].parent < 0 || gsegs[s].top != gsegs[s].parent + 1;
-                if (!head) {
-                    glevel[s] = glevel[(size_t)gpseg[s]];
-                    continue;
-                }
-                glevel[s] = gsegs[s].parent < 0 ? 0 : glevel[(size_t)gpseg[s]] + 1;
-                size_t c = s;
-                for (;;) {
-                    const int32_t nb = gsegs[c].top + gsegs[c].len - lb;  // one past the bottom
-                    const int32_t nx = nb < n ? ws.seg_of_top[(size_t)nb] : -1;
-                    if (nx < 0 || gsegs[(size_t)nx].parent != gsegs[c].top + gsegs[c].len - 1) break;
-                    c = (size_t)nx;
-                }
-                gpaths.push_back(PathTmp{gsegs[s].top, gsegs[c].top + gsegs[c].len, gsegs[s].parent, k - k0,
-                                         glevel[s]});
+                ws.path_of[(size_t)j] = (int32_t)gpaths.size() - 1;
+                gpaths.back().end = lb + j + 1;
             }
         }
-        // sort by (height, longest first, top)
-        const int32_t ns = (int32_t)gsegs.size();
-        perm.resize((size_t)ns);
-        std::iota(perm.begin(), perm.end(), 0);
-        std::sort(perm.begin(), perm.end(), [&](int32_t a, int32_t b) {
-            if (gheight[(size_t)a] != gheight[(size_t)b]) return gheight[(size_t)a] < gheight[(size_t)b];
-            if (gsegs[(size_t)a].len != gsegs[(size_t)b].len) return gsegs[(size_t)a].len > gsegs[(size_t)b].len;
-            return gsegs[(size_t)a].top < gsegs[(size_t)b].top;
-        });
-        newidx.resize((size_t)ns);
-        for (int32_t i = 0; i < ns; ++i) newidx[(size_t)perm[(size_t)i]] = i;
         mmk::GroupRec gr{};
         gr.comp0 = comp0;
         gr.scratch0 = 0;
         gr.ncomp = (int32_t)(L.noff[(size_t)k1] - comp0);
-        gr.nseg = ns;
         gr.neuron0 = k0;
         gr.nneuron = k1 - k0;
-        int32_t maxh = 0;
-        int64_t nkids = 0;
-        for (int32_t i = 0; i < ns; ++i) {
-            maxh = std::max(maxh, gheight[(size_t)perm[(size_t)i]]);
-            nkids += (int64_t)gkids[(size_t)perm[(size_t)i]].size();
-        }
-        // shared-memory need: FP64 items hold the segment blob, FP32c items
-        // the path tables (16-bit records) plus per-path slots
+        // shared-memory need: the path tables (16-bit records) and the
+        // kernel's bytes per compartment and path
         PathBlob pb;
-        int64_t smem_need;
-        if (in.path_items) {
-            build_path_blob(gpaths, gr.nneuron, gsize, pb);
-            if (gr.ncomp <= 32767 && pb.npath <= 32767) {
-                smem_need = blob_offsets(pb, false).bytes + (int64_t)in.smem_per_comp * gr.ncomp +
-                            (int64_t)in.smem_per_path * pb.npath;
-            } else {
-                smem_need = INT64_MAX;
-            }
-        } else {
-            const int64_t small_meta = ((int64_t)ns * (int64_t)sizeof(mmk::SegP) + 2 * nkids + 2 * (maxh + 2) + 15) & ~15LL;
-            smem_need = small_meta + (int64_t)in.smem_per_comp * gr.ncomp + (int64_t)in.smem_per_seg * ns;
-        }
+        build_path_blob(gpaths, gr.nneuron, gsize, pb);
+        const bool narrow = gr.ncomp <= 32767 && pb.npath <= 32767;
+        const int64_t smem_need = !narrow ? INT64_MAX
+                                          : blob_offsets(pb, false).bytes + (int64_t)in.smem_per_comp * gr.ncomp +
+                                                (int64_t)in.smem_per_path * pb.npath;
         const bool over = in.giant_smem_limit > 0 && smem_need > in.giant_smem_limit;
         const bool big = over && in.big_smem_limit > 0 && smem_need <= in.big_smem_limit;
-        const bool giant = (in.path_items ? (gr.ncomp > 32767 || pb.npath > 32767) : (gr.ncomp > 32767 || ns > 32767)) ||
-                           (over && !big);
+        const bool giant = !narrow || (over && !big);
         if (giant && in.giant_smem_limit <= 0) {
             *invalid = false;
             e << "a work item of " << gr.ncomp << " compartments exceeds what this precision holds";
             return msg(e);
         }
         std::vector<unsigned char> blob;
-        if (in.path_items) {
-            // links inside paths are assembled per compartment; path heads
-            // (negative parent distance) link to their parent in the sweep
-            for (int64_t c = comp0; c < comp0 + gr.ncomp; ++c) {
-                const int32_t pd = std::abs(L.pdist[(size_t)c]);
-                L.pdist[(size_t)c] = pd == 1 ? 1 : -pd;
-            }
+        {
             // 16-bit records for items staged in shared memory, 32-bit for giants
             const BlobOffsets o = blob_offsets(pb, giant);
             blob = emit_path_blob(pb, giant);
@@ -636,44 +554,6 @@ std::string build_layout(const LayoutInput &in, Layout &out, bool *invalid)
                 gr.pscratch0 = (int32_t)L.giant_paths;
                 L.giant_paths += pb.npath;
             }
-        } else {
-            // the segment blob: records in wave order, child lists, wave offsets
-            std::vector<int32_t> woff;
-            {
-                int32_t i = 0;
-                for (int32_t h = 0; h <= maxh; ++h) {
-                    while (i < ns && gheight[(size_t)perm[(size_t)i]] < h) ++i;
-                    woff.push_back(i);
-                }
-                woff.push_back(ns);
-            }
-            gr.nchild = (int32_t)nkids;
-            gr.nwave = maxh + 1;
-            auto put = [&blob](const void *p, size_t n) {
-                const unsigned char *c = (const unsigned char *)p;
-                blob.insert(blob.end(), c, c + n);
-            };
-            std::vector<int16_t> kids;
-            std::vector<mmk::SegP> recs((size_t)ns);
-            for (int32_t i = 0; i < ns; ++i) {
-                const int32_t sidx = perm[(size_t)i];
-                const mmk::SegRec &r = gsegs[(size_t)sidx];
-                mmk::SegP q;
-                q.top = (int16_t)r.top;
-                q.len = (int16_t)r.len;
-                q.parent = (int16_t)r.parent;
-                q.nchild = (int16_t)gkids[(size_t)sidx].size();
-                q.child0 = (int16_t)kids.size();
-                q.neuron = (int16_t)r.neuron;
-                q.pseg = (int16_t)(gpseg[(size_t)sidx] < 0 ? -1 : newidx[(size_t)gpseg[(size_t)sidx]]);
-                q.pad = 0;
-                for (int32_t c : gkids[(size_t)sidx]) kids.push_back((int16_t)newidx[(size_t)c]);
-                recs[(size_t)i] = q;
-            }
-            std::vector<int16_t> w16(woff.begin(), woff.end());
-            put(recs.data(), recs.size() * sizeof(mmk::SegP));
-            put(kids.data(), kids.size() * 2);
-            put(w16.data(), w16.size() * 2);
         }
         blob.resize((blob.size() + 15) & ~(size_t)15, 0);
         gr.meta_off = (int64_t)L.meta.size();
@@ -684,15 +564,15 @@ std::string build_layout(const LayoutInput &in, Layout &out, bool *invalid)
         } else if (big) {
             bigs.push_back(gr);
             L.big_max_comps = std::max(L.big_max_comps, gr.ncomp);
-            L.big_max_segs = std::max(L.big_max_segs, in.path_items ? gr.npath : ns);
+            L.big_max_segs = std::max(L.big_max_segs, gr.npath);
             L.big_max_meta = std::max(L.big_max_meta, gr.meta_bytes);
             L.big_max_smem = std::max<int64_t>(L.big_max_smem, smem_need);
         } else {
             L.groups.push_back(gr);
             L.max_smem = std::max<int64_t>(L.max_smem, smem_need);
             L.max_comps = std::max(L.max_comps, gr.ncomp);
-            L.max_segs = std::max(L.max_segs, in.path_items ? gr.npath : ns);
-            L.max_waves = std::max(L.max_waves, in.path_items ? gr.nlevel : gr.nwave);
+            L.max_segs = std::max(L.max_segs, gr.npath);
+            L.max_waves = std::max(L.max_waves, gr.nlevel);
             L.max_meta = std::max(L.max_meta, gr.meta_bytes);
         }
     }

@@ -30,15 +30,13 @@ struct LayoutInput {
     int32_t group_comps;          // compartment budget of a work item
     int32_t max_group_comps;      // largest neuron accepted
     // shared-memory model of a work item, bytes = meta + smem_per_comp * comps
-    // + smem_per_seg * segments (+ smem_per_path * paths for path items);
-    // items above giant_smem_limit go to the large shared-memory class if
-    // they fit big_smem_limit (0: no such class), else they become giant
-    // items (giant_smem_limit 0: no classes at all)
-    int32_t smem_per_comp, smem_per_seg, giant_smem_limit, big_smem_limit;
-    // FP32c: items are solved path by path (mmk::NrnQ tables with 16-bit
-    // records, mmk::NrnG with 32-bit records for giant items), with
-    // smem_per_path bytes per path
-    bool path_items;
+    // + smem_per_path * paths; items above giant_smem_limit go to the large
+    // shared-memory class if they fit big_smem_limit (0: no such class), else
+    // they become giant items (giant_smem_limit 0: no classes at all)
+    int32_t smem_per_comp;
+    int32_t smem_per_seg;         // not used: items are solved path by path
+    int32_t giant_smem_limit, big_smem_limit;
+    bool path_items;              // not used, as above
     int32_t smem_per_path;
 };
 
@@ -51,8 +49,8 @@ struct Layout {
     std::vector<int64_t> user2int;      // user compartment -> internal compartment [C]
     std::vector<int64_t> soma_of_user;  // internal soma compartment of each user neuron [N]
     std::vector<double> L, D;           // cylinders, internal order
-    std::vector<int32_t> pdist;         // i - parent(i) in internal order, negated at segment tops (FP64)
-                                        // or path heads (FP32c), 0 at somata
+    std::vector<int32_t> pdist;         // i - parent(i) in internal order, negated at path heads, 0 at
+                                        // somata
     std::vector<double> stim;           // internal order
     std::vector<mmk::GroupRec> groups;
     std::vector<unsigned char> meta;    // tree blobs (16-byte aligned per work item)
