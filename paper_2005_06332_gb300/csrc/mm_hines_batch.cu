@@ -1,14 +1,16 @@
 // mm_hines_batch.cu -- a standalone batched Hines solve on the device.
 //
-// Algorithm 1 (Sec. 2) exactly as the paper states it, for many independent
-// trees at once: one thread per tree walks the backward sweep (leaves to
-// root over parent[]) and the forward substitution.  Inputs are const; the
-// eliminated diagonal lives in a scratch array and the rhs is worked on in
-// the output array.  Device pointers in and out.
+// Algorithm 1 (Sec. 2) for many independent trees at once, any numbering with
+// parent[j] < j.  Inputs are const; the eliminated diagonal lives in a scratch
+// array and the rhs is worked on in the output array.  Device pointers in and
+// out.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "mm.h"
+#include "mm_fp64_math.h"
 
 // Scratch of mm_hines_solve_noalloc: a fixed device array in this library
 // image, so that the call never allocates.  The first 256 bytes hold the
@@ -19,67 +21,516 @@ static __device__ __align__(256) double g_noalloc_scratch[32 + MM_NOALLOC_MAX_CO
 
 namespace {
 
-// status word: 0 = ok, 1 = a tree violates parent[0] = -1, 0 <= parent[i] < i,
-// or its entry range tree_offset[t] .. tree_offset[t+1]-1 is not inside
-// [0, n_comp) (such a tree is skipped before any of its entries is touched)
-__global__ void hines_batch_kernel(int32_t n_trees, int64_t n_comp, const int64_t *__restrict__ off,
-                                   const int32_t *__restrict__ parent, const double *__restrict__ a,
-                                   const double *__restrict__ b, const double *__restrict__ c,
-                                   const double *__restrict__ rhs, double *__restrict__ x,
-                                   double *__restrict__ work, int *__restrict__ status)
+struct Batch {
+    int32_t n_trees;
+    int64_t n_comp;
+    const int64_t *off;
+    const int32_t *parent;
+    const double *a, *b, *c, *rhs;
+    double *x, *work;
+    int *status;             // bit 0: a tree violates the parent rule or its entries lie outside n_comp; bit 1: see
+                             // hines_rest_kernel
+    int32_t trees_per_block; // 1 .. kMaxTrees
+};
+
+// One tree by one thread, exactly as Algorithm 1 is stated: the path of trees
+// that the block's tables do not hold, and of blocks with an invalid tree (such
+// a tree is skipped before any of its entries is touched).
+__device__ void solve_serial(const Batch &B, int32_t t)
 {
-    for (int32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < n_trees; t += gridDim.x * blockDim.x) {
-        const int64_t base = off[t], end = off[t + 1];
-        if (base < 0 || end < base || end > n_comp) {
-            atomicOr(status, 1);
-            continue;
-        }
-        const int64_t n = end - base;
-        if (n == 0) continue;
-        const int32_t *p = parent + base;
-        bool ok = p[0] == -1;
-        for (int64_t i = 1; ok && i < n; ++i) ok = p[i] >= 0 && p[i] < i;
-        if (!ok) {
-            atomicOr(status, 1);
-            continue;
-        }
-        double *w = work + base;
-        double *r = x + base;
-        for (int64_t i = 0; i < n; ++i) {
-            w[i] = b[base + i];
-            r[i] = rhs[base + i];
-        }
-        // backward sweep, leaves to root
-        for (int64_t i = n - 1; i >= 1; --i) {
-            const double factor = a[base + i] / w[i];
-            w[p[i]] -= factor * c[base + i];
-            r[p[i]] -= factor * r[i];
-        }
-        r[0] /= w[0];
-        // forward sweep, root to leaves
-        for (int64_t i = 1; i < n; ++i) {
-            r[i] -= c[base + i] * r[p[i]];
-            r[i] /= w[i];
-        }
+    const int64_t base = B.off[t], end = B.off[t + 1];
+    if (base < 0 || end < base || end > B.n_comp) {
+        atomicOr(B.status, 1);
+        return;
+    }
+    const int64_t n = end - base;
+    if (n == 0) return;
+    const int32_t *p = B.parent + base;
+    bool ok = p[0] == -1;
+    for (int64_t i = 1; ok && i < n; ++i) ok = p[i] >= 0 && p[i] < i;
+    if (!ok) {
+        atomicOr(B.status, 1);
+        return;
+    }
+    double *w = B.work + base;
+    double *r = B.x + base;
+    for (int64_t i = 0; i < n; ++i) {
+        w[i] = B.b[base + i];
+        r[i] = B.rhs[base + i];
+    }
+    // backward sweep, leaves to root
+    for (int64_t i = n - 1; i >= 1; --i) {
+        const double factor = B.a[base + i] / w[i];
+        w[p[i]] -= factor * B.c[base + i];
+        r[p[i]] -= factor * r[i];
+    }
+    r[0] /= w[0];
+    // forward sweep, root to leaves
+    for (int64_t i = 1; i < n; ++i) {
+        r[i] -= B.c[base + i] * r[p[i]];
+        r[i] /= w[i];
     }
 }
 
-mm_status run_batch(int32_t n_trees, int64_t n_comp, const int64_t *off, const int32_t *parent, const double *a,
-                    const double *b, const double *c, const double *rhs, double *x, double *work, int *status,
-                    cudaStream_t s)
+constexpr int kMaxTrees = 128;     // trees of one block
+constexpr int kBlockComps = 2048;  // compartments aimed at per block
+constexpr long long kLeft = 0x7FF8A5C3966D1E27LL;  // in the scratch, at the first entry of a block that was left
+constexpr size_t smem_of(int chains) { return (size_t)chains * 20 + 16; }
+
+// x 2^-(d >> 20); d the difference of two exponent fields
+__device__ __forceinline__ double scale_down(double x, int d)
 {
-    if (cudaMemsetAsync(status, 0, sizeof(int), s) != cudaSuccess) return MM_ECUDA;
-    if (n_trees > 0 && n_comp > 0) {
-        const int threads = 128;
-        int blocks = (int)((n_trees + threads - 1) / threads);
-        if (blocks > 152 * 16) blocks = 152 * 16;
-        hines_batch_kernel<<<blocks, threads, 0, s>>>(n_trees, n_comp, off, parent, a, b, c, rhs, x, work, status);
+    const int h = __double2hiint(x), e = h & 0x7FF00000;
+    const int ne = e - d;
+    if (e != 0 && e != 0x7FF00000 && ne > 0 && ne < 0x7FF00000) return __hiloint2double(h - d, __double2loint(x));
+    return (x == 0.0 || e == 0x7FF00000) ? x : scalbn(x, -(d >> 20));
+}
+
+// One entry of a chain's elimination: N / M is its eliminated diagonal, S / M
+// its rhs.
+struct Front {
+    double N, M, S;
+    // powers of two out, so that N lies in [1, 2); a zero pivot becomes NaN
+    // (the division by it is what fails in Algorithm 1)
+    __device__ __forceinline__ void normalise()
+    {
+        const int h = __double2hiint(N), e = h & 0x7FF00000;
+        if (e == 0 || e == 0x7FF00000) {
+            if (N == 0.0) N = __longlong_as_double(0x7FF8000000000000LL);
+            return;
+        }
+        const int d = e - 0x3FF00000;
+        N = __hiloint2double(h - d, __double2loint(N));
+        M = scale_down(M, d);
+        S = scale_down(S, d);
+    }
+};
+
+// the N that Front::normalise leaves
+__device__ __forceinline__ double normalised(double N)
+{
+    const int h = __double2hiint(N), e = h & 0x7FF00000;
+    return e == 0 || e == 0x7FF00000 ? N : __hiloint2double(h - e + 0x3FF00000, __double2loint(N));
+}
+
+// A block solves trees_per_block consecutive trees together.  Bound by the
+// FP64 pipe and, for the largest trees, by the chain of their sweeps: a warp's
+// FP64 instruction takes 64 clocks of its scheduler whatever the number of
+// active lanes, so the sweeps want many independent chains per warp, many
+// blocks per SM, and few FP64 instructions per entry:
+//   * the entries are cut into chains (runs with parent[i] = i - 1); chains
+//     of one level -- hanging off chains of the level above -- are swept by
+//     one lane each, from the deepest level up and back down;
+//   * the elimination carries N, M, S (Algorithm 1's row times M: N' = b N -
+//     (a M) c, M' = N, S' = rhs N - a S), five instructions instead of a
+//     division and three; the division is a pass of full warps afterwards
+//     (f = -c M / N, s = S / N), and the substitution is x_j = f_j x_{j-1} + s_j;
+//   * a chain's first entry is divided when its warp's chains are done, and
+//     its share goes into the entry it hangs off, b += a f, rhs -= a s, after
+//     the level, one thread per entry, larger children first as Algorithm 1
+//     does (the chains are sorted by level and that entry).
+// b and rhs, then N and S, then f and s, then x live in the scratch and the
+// output array (L2).  Measured (whole call, allocation included): 3,000 trees of
+// 50 to 5,000 entries 12.4 ms with a thread per tree, 0.89 ms so (0.82 ms in
+// the kernel, FP64 pipe 36 % busy); 3,000 of 8 to 300 0.78 -> 0.33 ms; 64 of 200
+// to 5,000 9.0 -> 0.57 ms.  128 threads and six blocks per SM; 32 or 64 threads
+// and more blocks 0.94 to 1.14 ms, groups of 4,096 entries 1.34 ms; eliminating
+// the diagonal alone first (with a c stored: 2 + 2 + 2 instructions in the
+// sweeps, but two passes more) 1.10 ms.  CHAINS: the chains that a block's tables hold.  FIRST:
+// every group of trees, else those that a smaller table left.
+template <int CHAINS, int NT, bool FIRST>
+__device__ __forceinline__ void solve_group(const Batch &B, int group)
+{
+    constexpr int kChunk = 2;  // entries per step of a sweep (operands loaded one step ahead)
+    constexpr int kSub = 8;    // the same of the substitution
+    constexpr int kLook = 4;   // entries that a thread takes together in the passes over all entries
+    extern __shared__ __align__(16) unsigned char smem[];
+    unsigned long long *key = (unsigned long long *)smem;  // chains by (level, entry they hang off, chain)
+    int *head = (int *)(key + CHAINS);                     // first entry of each chain, then the end
+    int *up = head + CHAINS + 1;                           // chain above (pointer jumping)
+    int *lev = up + CHAINS;                                // level; then where each level begins in key
+    __shared__ int64_t s_off[kMaxTrees + 1];
+    __shared__ int s_warp[kLook * NT / 32], s_bad, s_K, s_go;
+    static_assert(kMaxTrees < NT + 1 && (CHAINS & (CHAINS - 1)) == 0 && CHAINS <= 8192, "table sizes");
+    constexpr unsigned long long kChain = 0x1FFF;  // a key: level << 43 | entry << 13 | chain
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int32_t t0 = group * B.trees_per_block, t1 = min(t0 + B.trees_per_block, B.n_trees);
+    const int nt = t1 - t0;
+    if (tid == 0) s_bad = s_K = 0;
+    if (tid <= nt) s_off[tid] = B.off[t0 + tid];
+    if (tid == 0 && nt == NT) s_off[nt] = B.off[t1];
+    __syncthreads();
+    if (!FIRST) {
+        const int64_t first = s_off[0];
+        if (first < 0 || first >= B.n_comp || __double_as_longlong(B.work[first]) != kLeft) return;
+    }
+    if (tid < nt && (s_off[tid] < 0 || s_off[tid + 1] < s_off[tid] || s_off[tid + 1] > B.n_comp)) s_bad = 1;
+    __syncthreads();
+    const int64_t base = s_off[0];
+    const int64_t total = s_off[nt] - base;
+    if (s_bad || total > 0x3FFFFFFF) {
+        if (tid < nt) solve_serial(B, t0 + tid);
+        return;
+    }
+    const int n = (int)total;
+    if (n == 0) return;
+    const int32_t *parent = B.parent + base;
+    const double *a = B.a + base, *b = B.b + base, *c = B.c + base, *rhs = B.rhs + base;
+    double *x = B.x + base, *work = B.work + base;
+
+    // the first entry of entry i's tree, relative to the block's
+    auto tree_base = [&](int i) {
+        int lo = 0, hi = nt;  // last tree with s_off <= i (empty trees end where they begin)
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (s_off[mid] - base <= i) lo = mid; else hi = mid;
+        }
+        return (int)(s_off[lo] - base);
+    };
+    // 1. the parent rule, and the chains' first entries in order
+    int stop = 0;  // 1: an invalid tree, 2: more chains than the tables hold
+    for (int i0 = 0; i0 < n && !stop; i0 += kLook * NT) {
+        int p[kLook];
+#pragma unroll
+        for (int u = 0; u < kLook; ++u) p[u] = i0 + u * NT + tid < n ? parent[i0 + u * NT + tid] : 0;
+        bool first[kLook], bad = false;
+        unsigned m[kLook];
+#pragma unroll
+        for (int u = 0; u < kLook; ++u) {
+            const int i = i0 + u * NT + tid;
+            first[u] = false;
+            if (i < n) {
+                const int tb = tree_base(i);
+                bad |= i == tb ? p[u] != -1 : p[u] < 0 || p[u] >= i - tb;
+                first[u] = i == tb || tb + p[u] != i - 1;
+            }
+            m[u] = __ballot_sync(0xFFFFFFFFu, first[u]);
+            if (lane == 0) s_warp[u * (NT / 32) + (tid >> 5)] = __popc(m[u]);
+        }
+        __syncthreads();
+        int k = s_K;
+        int last = 0;
+        for (int u = 0, w = 0; u < kLook; ++u) {
+            for (; w < u * (NT / 32) + (tid >> 5); ++w) k += s_warp[w];
+            last = k + __popc(m[u] & ((1u << lane) - 1u));
+            if (first[u] && last < CHAINS) head[last] = i0 + u * NT + tid;
+            last += first[u] ? 1 : 0;
+        }
+        __syncthreads();
+        if (tid == NT - 1) s_K = last;
+        if (__syncthreads_or(bad)) stop = 1;
+        else if (s_K > CHAINS) stop = 2;
+    }
+    if (stop == 1) {
+        if (tid < nt) solve_serial(B, t0 + tid);
+        return;
+    }
+    if (stop == 2) {  // left to a larger table or to hines_rest_kernel
+        if (tid == 0) {
+            work[0] = __longlong_as_double(kLeft);
+            atomicOr(B.status, 2);
+        }
+        return;
+    }
+    const int K = s_K;
+    if (tid == 0) head[K] = n;
+    for (int i0 = tid; i0 < n; i0 += kLook * NT) {
+        double bv[kLook], rv[kLook];
+#pragma unroll
+        for (int u = 0; u < kLook; ++u) {
+            const int i = min(i0 + u * NT, n - 1);
+            bv[u] = b[i];
+            rv[u] = rhs[i];
+        }
+#pragma unroll
+        for (int u = 0; u < kLook; ++u) {
+            const int i = i0 + u * NT;
+            if (i < n) {
+                work[i] = bv[u];
+                x[i] = rv[u];
+            }
+        }
+    }
+    __syncthreads();
+    // 2. the entry each chain hangs off, the chain it belongs to, and levels
+    //    by pointer jumping over these
+    int P2 = 32;
+    while (P2 < K) P2 <<= 1;
+    for (int k = tid; k < P2; k += NT) {
+        unsigned long long v = ~0ull;
+        if (k < K) {
+            const int i = head[k], p = parent[i];
+            int u = -1, q = 0;
+            if (p >= 0) {
+                q = tree_base(i) + p;
+                int lo = 0, hi = k;
+                while (hi - lo > 1) {
+                    const int mid = (lo + hi) >> 1;
+                    if (head[mid] <= q) lo = mid; else hi = mid;
+                }
+                u = lo;
+            }
+            up[k] = u;
+            lev[k] = u >= 0;
+            v = ((unsigned long long)q << 13) | (unsigned)k;
+        }
+        key[k] = v;
+    }
+    for (;;) {
+        __syncthreads();
+        if (tid == 0) s_go = 0;
+        __syncthreads();
+        // rounds of NT chains read before they write; a chain's value counts
+        // the levels up to its `up`, whichever round that came from
+        for (int k0 = 0; k0 < K; k0 += NT) {
+            const int k = k0 + tid;
+            int u = -1, l = 0;
+            const bool act = k < K && up[k] >= 0;
+            if (act) {
+                l = lev[k] + lev[up[k]];
+                u = up[up[k]];
+            }
+            __syncthreads();
+            if (act) {
+                lev[k] = l;
+                up[k] = u;
+                if (u >= 0) s_go = 1;
+            }
+            __syncthreads();
+        }
+        if (!s_go) break;
+    }
+    // 3. the chains by level and the entry they hang off (bitonic), and where
+    //    each level begins
+    for (int k = tid; k < K; k += NT) key[k] |= (unsigned long long)lev[k] << 43;
+    for (int size = 2; size <= P2; size <<= 1)
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+            __syncthreads();
+            for (int q = tid; q < P2 / 2; q += NT) {
+                const int i = 2 * q - (q & (stride - 1)), j = i + stride;
+                const unsigned long long u = key[i], v = key[j];
+                if ((u > v) == ((i & size) == 0)) {
+                    key[i] = v;
+                    key[j] = u;
+                }
+            }
+        }
+    __syncthreads();
+    const int nlev = (int)(key[K - 1] >> 43) + 1;
+    int *lbeg = lev;
+    for (int q = tid; q < K; q += NT) {
+        const int l = (int)(key[q] >> 43);
+        if (q == 0 || (int)(key[q - 1] >> 43) != l) lbeg[l] = q;
+    }
+    __syncthreads();
+    auto level_end = [&](int l) { return l + 1 < nlev ? lbeg[l + 1] : K; };
+
+    // 4. elimination, deepest level first
+    for (int l = nlev - 1; l >= 0; --l) {
+        const int q0 = lbeg[l], q1 = level_end(l);
+        for (int w0 = q0 + (tid & ~31); w0 < q1; w0 += NT) {
+            // whole warps, to the longest chain's end (lanes without a chain
+            // sweep none), so that the division below is done once
+            const bool has = w0 + lane < q1;
+            const int k = has ? (int)(key[w0 + lane] & kChain) : 0, h = head[k];
+            int j = has ? head[k + 1] - 1 : h - 1;
+            const int steps = __reduce_max_sync(0xFFFFFFFFu, j - h + 1);
+            double an[kChunk], cn[kChunk], bn[kChunk], rn[kChunk];
+            auto load = [&](int jj) {
+#pragma unroll
+                for (int z = 0; z < kChunk; ++z) {
+                    const int i = max(jj - z, h);
+                    an[z] = __ldg(a + i);
+                    cn[z] = __ldg(c + i);
+                    bn[z] = work[i];
+                    rn[z] = x[i];
+                }
+            };
+            if (has) load(j);
+            Front F{1.0, 0.0, 0.0};     // below the leaf: N = b, S = rhs
+            double ab = 0.0, cb = 0.0;  // a and c of the entry below
+            double N = 0.0, S = 0.0, M = 0.0;
+            for (int t = 0; t < steps; t += kChunk, j -= kChunk) {
+                double av[kChunk], cv[kChunk], bv[kChunk], rv[kChunk];
+#pragma unroll
+                for (int z = 0; z < kChunk; ++z) {
+                    av[z] = an[z];
+                    cv[z] = cn[z];
+                    bv[z] = bn[z];
+                    rv[z] = rn[z];
+                }
+                if (j - kChunk >= h) load(j - kChunk);
+#pragma unroll
+                for (int z = 0; z < kChunk; ++z) {
+                    const int i = j - z;
+                    if (i >= h) {
+                        N = fma(bv[z], F.N, -((ab * F.M) * cb));
+                        S = fma(rv[z], F.N, -(ab * F.S));
+                        M = F.N;
+                        ab = av[z];
+                        cb = cv[z];
+                        if (i > h) {
+                            work[i] = N;
+                            x[i] = S;
+                        }
+                        F = Front{N, M, S};
+                        F.normalise();
+                    }
+                }
+            }
+            if (has) {
+                const double inv = mmk::rcp_nr(N);
+                work[h] = -mmk::div_nr(cb * M, N, inv);
+                x[h] = mmk::div_nr(S, N, inv);
+            }
+        }
+        __syncthreads();
+        if (l == 0) break;
+        for (int q = q0 + tid; q < q1; q += NT) {
+            const unsigned long long run = key[q] >> 13;  // level and entry
+            if (q + 1 < q1 && (key[q + 1] >> 13) == run) continue;  // not the last of its run
+            const int p = (int)(run & 0x3FFFFFFF);
+            double bp = work[p], rp = x[p];
+            for (int z = q; z >= q0 && (key[z] >> 13) == run; --z) {
+                const int h = head[key[z] & kChain];
+                const double ah = __ldg(a + h);
+                bp = fma(ah, work[h], bp);
+                rp = fma(-ah, x[h], rp);
+            }
+            work[p] = bp;
+            x[p] = rp;
+        }
+        __syncthreads();
+    }
+    // 5. the division of every entry that is not a chain's first
+    for (int i0 = 0; i0 < n; i0 += kLook * NT) {
+        bool todo[kLook];
+        double N[kLook], M[kLook], S[kLook], cc[kLook];
+#pragma unroll
+        for (int u = 0; u < kLook; ++u) {
+            const int i = i0 + u * NT + tid;
+            todo[u] = false;
+            if (i < n) {
+                const int tb = tree_base(i);
+                todo[u] = i != tb && tb + parent[i] == i - 1;
+                N[u] = work[i];
+                S[u] = x[i];
+                cc[u] = __ldg(c + i);
+                M[u] = i + 1 < n && parent[i + 1] >= 0 && tb + parent[i + 1] == i ? normalised(work[i + 1]) : 1.0;
+            }
+        }
+        __syncthreads();  // the entry above has read this one's N
+#pragma unroll
+        for (int u = 0; u < kLook; ++u) {
+            const int i = i0 + u * NT + tid;
+            if (todo[u]) {
+                const double inv = mmk::rcp_nr(N[u]);
+                work[i] = -mmk::div_nr(cc[u] * M[u], N[u], inv);
+                x[i] = mmk::div_nr(S[u], N[u], inv);
+            }
+        }
+    }
+    __syncthreads();
+    // 6. substitution, roots first
+    for (int l = 0; l < nlev; ++l) {
+        const int q1 = level_end(l);
+        for (int q = lbeg[l] + tid; q < q1; q += NT) {
+            const int k = (int)(key[q] & kChain), h = head[k], e = head[k + 1];
+            double xv = x[h];
+            if (l > 0) {
+                xv = fma(work[h], x[(key[q] >> 13) & 0x3FFFFFFF], xv);
+                x[h] = xv;
+            }
+            double fn[kSub], sn[kSub];
+            auto load = [&](int jj) {
+#pragma unroll
+                for (int z = 0; z < kSub; ++z) {
+                    const int i = min(jj + z, e - 1);
+                    fn[z] = work[i];
+                    sn[z] = x[i];
+                }
+            };
+            int j = h + 1;
+            if (j < e) load(j);
+            for (; j < e; j += kSub) {
+                double fv[kSub], sv[kSub];
+#pragma unroll
+                for (int z = 0; z < kSub; ++z) {
+                    fv[z] = fn[z];
+                    sv[z] = sn[z];
+                }
+                if (j + kSub < e) load(j + kSub);
+#pragma unroll
+                for (int z = 0; z < kSub; ++z) {
+                    if (j + z < e) {
+                        xv = fma(fv[z], xv, sv[z]);
+                        x[j + z] = xv;
+                    }
+                }
+            }
+        }
+        __syncthreads();
+    }
+}
+
+template <int CHAINS, int NT, int BLOCKS>
+__global__ void __launch_bounds__(NT, BLOCKS) hines_batch_kernel(Batch B)
+{
+    solve_group<CHAINS, NT, true>(B, blockIdx.x);
+}
+
+// The blocks of trees that hines_batch_kernel left, with a larger table.
+template <int CHAINS, int NT>
+__global__ void __launch_bounds__(NT, 1) hines_left_kernel(Batch B, int groups)
+{
+    if (!(*B.status & 2)) return;
+    for (int g = blockIdx.x; g < groups; g += gridDim.x) {
+        solve_group<CHAINS, NT, false>(B, g);
+        __syncthreads();
+    }
+}
+
+// The trees of blocks with more chains than the largest table holds (mostly one
+// large tree to a block), a thread for each block, so that many such trees run
+// side by side.
+__global__ void __launch_bounds__(128) hines_rest_kernel(Batch B)
+{
+    if (!(*B.status & 2)) return;
+    const int64_t groups = ((int64_t)B.n_trees + B.trees_per_block - 1) / B.trees_per_block;
+    for (int64_t g = blockIdx.x * 128LL + threadIdx.x; g < groups; g += gridDim.x * 128LL) {
+        const int64_t t0 = g * B.trees_per_block, t1 = min(t0 + B.trees_per_block, (int64_t)B.n_trees);
+        const int64_t first = B.off[t0];
+        if (first < 0 || first >= B.n_comp || __double_as_longlong(B.work[first]) != kLeft) continue;
+        for (int64_t t = t0; t < t1; ++t) solve_serial(B, (int32_t)t);
+    }
+}
+
+mm_status run_batch(Batch B, cudaStream_t s)
+{
+    if (cudaMemsetAsync(B.status, 0, sizeof(int), s) != cudaSuccess) return MM_ECUDA;
+    if (B.n_trees > 0 && B.n_comp > 0) {
+        // trees per block: about kBlockComps entries, fewer where the batch
+        // would not fill the chip's slots otherwise, at least one tree.  The
+        // tables of 1,024 chains leave room for six blocks per SM; blocks with
+        // more chains are taken up by a second launch with one block per SM, and
+        // the rest by a third (both end at once when nothing was left).
+        constexpr auto small = hines_batch_kernel<1024, 128, 6>;
+        constexpr auto large = hines_left_kernel<8192, 256>;
+        // 912: six blocks on each of 152 SMs
+        const int64_t mean = std::max<int64_t>(1, B.n_comp / B.n_trees);
+        B.trees_per_block = (int32_t)std::min<int64_t>(kMaxTrees, std::max<int64_t>(1, std::min<int64_t>(kBlockComps, B.n_comp / 912) / mean));
+        const int64_t blocks = ((int64_t)B.n_trees + B.trees_per_block - 1) / B.trees_per_block;
+        if (cudaFuncSetAttribute(large, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of(8192)) != cudaSuccess)
+            return MM_ECUDA;
+        small<<<(unsigned)blocks, 128, smem_of(1024), s>>>(B);
+        large<<<(unsigned)std::min<int64_t>(blocks, 152), 256, smem_of(8192), s>>>(B, (int)blocks);
+        hines_rest_kernel<<<(unsigned)std::min<int64_t>((blocks + 127) / 128, 152 * 16), 128, 0, s>>>(B);
         if (cudaGetLastError() != cudaSuccess) return MM_ECUDA;
     }
     int h = 0;
-    if (cudaMemcpyAsync(&h, status, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess) return MM_ECUDA;
+    if (cudaMemcpyAsync(&h, B.status, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess) return MM_ECUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess) return MM_ECUDA;
-    return h ? MM_EINVAL : MM_OK;
+    return (h & 1) ? MM_EINVAL : MM_OK;
 }
 
 bool args_ok(int32_t n_trees, int64_t n_comp, const int64_t *off, const int32_t *parent, const double *a,
@@ -108,7 +559,7 @@ extern "C" mm_status mm_hines_solve(int32_t n_trees, int64_t n_comp, const int64
     }
     double *work = (double *)scratch;
     int *status = (int *)((char *)scratch + bytes - 256);
-    const mm_status st = run_batch(n_trees, n_comp, tree_offset, parent, a, b, c, rhs, x, work, status, s);
+    const mm_status st = run_batch({n_trees, n_comp, tree_offset, parent, a, b, c, rhs, x, work, status, 1}, s);
     cudaFree(scratch);
     return st;
 }
@@ -130,6 +581,5 @@ extern "C" mm_status mm_hines_solve_noalloc(int32_t n_trees, int64_t n_comp, con
     }
     int *status = (int *)base;                       // cleared by run_batch before the kernel
     double *work = (double *)((char *)base + 256);   // fully written before it is read
-    return run_batch(n_trees, n_comp, tree_offset, parent, a, b, c, rhs, x, work, status,
-                     (cudaStream_t)cuda_stream);
+    return run_batch({n_trees, n_comp, tree_offset, parent, a, b, c, rhs, x, work, status, 1}, (cudaStream_t)cuda_stream);
 }

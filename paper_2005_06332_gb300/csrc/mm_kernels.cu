@@ -16,6 +16,7 @@
 
 #include <mutex>
 
+#include "mm_fp64_math.h"
 #include "mm_gate_table64.h"
 #include "mm_internal.h"
 #include "mm_tma.h"
@@ -186,24 +187,6 @@ __global__ void __launch_bounds__(256) deliver_ordered_kernel(DeliverArgs a)
 }
 
 // ------------------------------------------------------------ FP64 step
-
-// 1/x by Newton's iteration from the approximate reciprocal (about 20 bits):
-// two steps reach FP64 rounding.  FP64 instructions are scarce (two lanes per
-// SM and clock), and the compiled division takes about twice as many.
-__device__ __forceinline__ double rcp_nr(double x)
-{
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    r = fma(r, fma(-x, r, 1.0), r);
-    return fma(r, fma(-x, r, 1.0), r);
-}
-
-// a / x given r = rcp_nr(x): one residual correction
-__device__ __forceinline__ double div_nr(double a, double x, double r)
-{
-    const double q = a * r;
-    return fma(r, fma(-x, q, a), q);
-}
 
 // 2^-exponent(x) for a normal x (x times it lies in [1, 2)); 1 for zero,
 // infinities and NaN, which stay as they are
