@@ -210,6 +210,7 @@ struct StepArgs32 {
     const unsigned char *meta;
     int32_t smem_meta;
     int32_t item0, item1;             // this launch's work items: [item0, item1)
+    int32_t n_huge;                   // giant items: the first n_huge are solved by a cluster of blocks each
     int32_t smem_bytes;               // dynamic shared memory of the launch (largest item need)
     unsigned int *queue;              // its work-queue counter (in ctl, reset by the delivery kernel)
     const int32_t *site_comp;
@@ -357,6 +358,7 @@ int mmk_launch_init_fp32c(const mmk::InitArgs &a, void *stream);
 int mmk_launch_giant_fp32c(const mmk::StepArgs32 &a, int blocks, void *stream);
 int mmk_launch_giant_assemble(const mmk::StepArgs32 &a, int chunk_blocks, void *stream);
 int mmk_launch_giant_update(const mmk::StepArgs32 &a, int chunk_blocks, void *stream);
+int mmk_giant_blocks(int n_giant, int n_huge);
 int mmk_giant_chunk();
 int mmk_launch_deliver_fp32c(const mmk::DeliverArgs &a, int blocks, void *stream);
 int mmk_launch_deliver_ordered(const mmk::DeliverArgs &a, int blocks, void *stream);

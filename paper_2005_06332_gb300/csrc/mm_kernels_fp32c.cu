@@ -910,8 +910,16 @@ __global__ void __launch_bounds__(NT, 1024 / NT) step_fp32c_kernel(StepArgs32 a)
 }
 
 
-template <int NT>
-__global__ void __launch_bounds__(NT) giant_fp32c_kernel(StepArgs32 a)
+// Paths of a giant of at least this many compartments are swept by a warp.
+constexpr int kGiantWarpPath = 48;
+// Blocks of a cluster (the portable maximum).
+constexpr int kGiantCluster = 8;
+
+// Solve of one giant work item by a team of NTT threads, of which this is
+// thread tid: a block, or (COOP) a cluster of blocks, whose scratch is written
+// and read across SMs, past L1.
+template <int NT, bool COOP>
+__device__ __forceinline__ void giant_solve(const StepArgs32 &a, int gi, int tid, int NTT)
 {
     // Work items too large for shared memory (giant neurons, up to the
     // int32 index range): the same path-by-path solve as step_fp32c_kernel
@@ -925,271 +933,456 @@ __global__ void __launch_bounds__(NT) giant_fp32c_kernel(StepArgs32 a)
     // blob in global memory (32-bit records); each lane loads the next eight
     // compartments of its path while it eliminates (or substitutes) the
     // current eight.
-    __shared__ int s_item;
-
     const long long n = (long long)a.ctl->step_base + a.step_offset;
-    const int tid = threadIdx.x;
-
-    for (;;) {
-        __syncthreads();
-        if (tid == 0) s_item = a.item0 + (int)atomicAdd(a.queue, 1u);
-        __syncthreads();
-        const int gi = s_item;
-        if (gi >= a.item1) break;
-        const unsigned long long t_item = (a.item_ns && tid == 0) ? global_ns() : 0ull;
-        const GroupRec G = a.groups[gi];
-        const int64_t c0 = G.comp0;
-        const int32_t *Vq = a.Vq + c0;
-        const float2 *gax = a.gax + c0;
-        const float2 *dpp = a.dp + c0;
-        float2 *dr = a.dr + G.scratch0;
-        float *drl = a.drl + G.scratch0;
-        float4 *pq = a.pq + G.pscratch0;
-        const unsigned char *blob = a.meta + G.meta_off;
-        const NrnG *nrns = (const NrnG *)blob;
-        const PathG *paths = (const PathG *)(blob + G.path_off);
-        const KidG *fold = (const KidG *)(blob + G.fold_off);
-        const int32_t *loffs = (const int32_t *)(blob + G.loffs_off);
-        const int32_t *mcnt = (const int32_t *)(blob + G.mcnt_off);
-
-        // S. synaptic sites (then their decay; sites are distinct
-        //    compartments), the current across each path's head link into
-        //    its head (for the path from a soma: the stimulus), then out of
-        //    the parent compartments, summed per parent in fold-list order
-        //    (as in step_fp32c_kernel)
-        for (int t = tid; t < G.nsite; t += NT) {
-            const int st = G.site0 + t;
-            const int c = a.site_comp[st];
-            const float2 g0 = a.gsyn[st];
-            const mmf::F2 g = mmf::two_sum(g0.x, g0.y);
-            float2 v = dr[c];
-            if (a.g_implicit) v.x += g.hi;
-            const mmf::F2 r = mmf::add(mmf::F2{v.y, drl[c]}, mmf::neg(mmf::mul(g, vminus(Vq[c], a.Esyn))));
-            v.y = r.hi;
-            dr[c] = v;
-            drl[c] = r.lo;
-            a.gsyn[st] = tof2(mmf::mul(g, f2(a.decay)));
-        }
-        __syncthreads();
-        for (int pi = tid; pi < G.npath; pi += NT) {
-            const PathG P = paths[pi];
-            mmf::F2 t;
-            if (P.parent >= 0) {
-                const float2 gs = gax[P.head];
-                t = mmf::mul(mmf::F2{fabsf(gs.x), gs.y}, mmf::vdiff_df(Vq[P.parent], Vq[P.head]));
-                pq[pi].z = t.hi;
-                pq[pi].w = t.lo;
-            } else {
-                t = mmf::split_d(a.stim[G.neuron0 + (P.nflag & kPathNeuronG)]);
-            }
-            const mmf::F2 r = mmf::add(mmf::F2{dr[P.head].y, drl[P.head]}, t);
-            dr[P.head].y = r.hi;
-            drl[P.head] = r.lo;
-        }
-        __syncthreads();
-        for (int e = tid; e < G.npath; e += NT) {
-            const int att = fold[e].y;
-            if (att < 0) continue;  // a path from a soma (no parent)
-            if (e > 0 && fold[e - 1].y == att) continue;  // not the first path of its parent
-            mmf::F2 t{0.f, 0.f};
-            for (int z = e; z < G.npath && fold[z].y == att; ++z) {
-                const float4 q = pq[fold[z].x];
-                t = mmf::add(t, mmf::F2{q.z, q.w});
-            }
-            const mmf::F2 r = mmf::add(mmf::F2{dr[att].y, drl[att]}, mmf::neg(t));
-            dr[att].y = r.hi;
-            drl[att] = r.lo;
-        }
-        __syncthreads();
-
-        // B. leaves-to-root elimination path by path, from the deepest level
-        //    up (as in step_fp32c_kernel: passive diagonal plus the active
-        //    conductance carried up the tree)
-        auto eliminate_path = [&](int pi) {
-            const PathG P = paths[pi];
-            const int h = P.head;
-            int j = P.end - 1;
-            const float2 v0 = dr[j];
-            float eb = v0.x, rb = v0.y, eh = eb, rh = rb;
-            float g0[8], l0[8], d0[8], q0[8], e0[8], r0[8];
-            float g1[8], l1[8], d1[8], q1[8], e1[8], r1[8];
-            auto load = [&](int jj, float *g, float *l, float *d, float *q, float *ee, float *r) {
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const int x = max(jj - k, h + 1);
-                    const float2 gs = gax[x], w = dr[x - 1];
-                    g[k] = a.gimp * fabsf(gs.x);
-                    l[k] = a.gimp * gs.y;
-                    d[k] = dpp[x].x;
-                    q[k] = (g[k] * rcp_nr(d[k])) * g[k];
-                    ee[k] = w.x;
-                    r[k] = w.y;
-                }
-            };
-            auto chain = [&](int jj, const float *g, const float *l, const float *d, const float *q,
-                             const float *ee, const float *r) {
-                const int cnt = jj - h;
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const float dd = d[k] + eb;
-                    const float r0 = rcp_approx(dd);
-                    const float inv = fmaf(r0, fmaf(-dd, r0, 1.f), r0);
-                    const float f = fmaf(g[k], inv, l[k] * inv);
-                    if (k < cnt) dr[jj - k] = make_float2(f, rb * inv);
-                    rb = fmaf(f, rb, r[k]);
-                    eb = fmaf(q[k] * r0, eb, ee[k]);
-                    if (k == cnt - 1) {
-                        eh = eb;
-                        rh = rb;
-                    }
-                }
-            };
-            if (j > h) {
-                load(j, g0, l0, d0, q0, e0, r0);
-                for (;;) {
-                    int jn = j - 8;
-                    bool more = jn > h;
-                    if (more) load(jn, g1, l1, d1, q1, e1, r1);
-                    chain(j, g0, l0, d0, q0, e0, r0);
-                    j = jn;
-                    if (!more) break;
-                    jn = j - 8;
-                    more = jn > h;
-                    if (more) load(jn, g0, l0, d0, q0, e0, r0);
-                    chain(j, g1, l1, d1, q1, e1, r1);
-                    j = jn;
-                    if (!more) break;
-                }
-            }
-            const float dhh = dpp[h].x;
-            const float inv = rcp_nr(dhh + eh);
-            if (P.parent < 0) {  // soma: its dV
-                dr[h].y = rh * inv;
-                return;
-            }
-            const float2 gs = gax[h];
-            const float gh = a.gimp * fabsf(gs.x), gl = a.gimp * gs.y;
-            const float f = fmaf(gh, inv, gl * inv);
-            dr[h] = make_float2(f, rh * inv);
-            const float ce = gh * rcp_nr(dhh) * f * eh, cr = f * rh;
-            if (P.nflag & kPathAloneG) {
-                float2 v = dr[P.parent];
-                v.x += ce;
-                v.y += cr;
-                dr[P.parent] = v;
-            } else {
-                pq[pi].x = ce;
-                pq[pi].y = cr;
-            }
-        };
-        auto fold_shared = [&](int e0, int e1) {
-            for (int e = e0 + tid; e < e1; e += NT) {
-                const KidG kv = fold[e];
-                if (e > e0 && fold[e - 1].y == kv.y) continue;
-                float ad = pq[kv.x].x, ar = pq[kv.x].y;
-                for (int z = e + 1; z < e1; ++z) {
-                    const KidG kz = fold[z];
-                    if (kz.y != kv.y) break;
-                    ad += pq[kz.x].x;
-                    ar += pq[kz.x].y;
-                }
-                float2 v = dr[kv.y];
-                v.x += ad;
-                v.y += ar;
-                dr[kv.y] = v;
-            }
-        };
-        // F. root-to-leaves substitution path by path; the path from a soma
-        //    runs the FP64 soma accumulator and the spike test
-        auto substitute_path = [&](int pi) {
-            const PathG P = paths[pi];
-            const int h = P.head;
-            float x;
-            if (P.parent >= 0) {
-                const float2 fh = dr[h];
-                x = fmaf(fh.x, dr[P.parent].y, fh.y);
-            } else {
-                x = dr[h].y;
-                const int nrn = G.neuron0 + (P.nflag & kPathNeuronG);
-                const double v0 = a.Vsoma[nrn], v1 = v0 + (double)x;
-                a.Vsoma[nrn] = v1;
-                if (!isfinite(v1)) atomicOr(&a.ctl->err, MMK_ERR_NUMERIC);
-                if (v0 < a.threshold && v1 >= a.threshold) {
-                    const int src = soma_source(a, nrn);
-                    if (src >= 0)
-                        record_spike(a, src, a.user_id[nrn], 0,
-                                     (double)n * a.dt64 + a.dt64 * (a.threshold - v0) / (v1 - v0), n);
-                }
-            }
-            const float xh = x;
-            float f0[8], c0v[8], f1[8], c1v[8];
-            auto load = [&](int jj, float *f, float *c) {
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const float2 w = dr[min(jj + k, P.end - 1)];
-                    f[k] = w.x;
-                    c[k] = w.y;
-                }
-            };
-            auto chain = [&](int jj, const float *f, const float *c) {
-                const int cnt = P.end - jj;
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    x = fmaf(f[k], x, c[k]);
-                    if (k < cnt) dr[jj + k].y = x;
-                }
-            };
-            int j = h + 1;
-            if (j < P.end) {
-                load(j, f0, c0v);
-                for (;;) {
-                    int jn = j + 8;
-                    bool more = jn < P.end;
-                    if (more) load(jn, f1, c1v);
-                    chain(j, f0, c0v);
-                    j = jn;
-                    if (!more) break;
-                    jn = j + 8;
-                    more = jn < P.end;
-                    if (more) load(jn, f0, c0v);
-                    chain(j, f1, c1v);
-                    j = jn;
-                    if (!more) break;
-                }
-            }
-            if (P.parent >= 0) dr[h].y = xh;  // read by the next level only
-        };
-
-        for (int k = 0; k < G.nbundle; ++k) {
-            const NrnG Nk = nrns[k];
-            const int32_t *lo = loffs + Nk.loff0;
-            const int32_t *mc = mcnt + Nk.loff0;
-            for (int l = Nk.nlevel - 1; l >= 0; --l) {
-                const int pb = lo[l], pe = lo[l + 1];
-                for (int pi = pb + tid; pi < pe; pi += NT) eliminate_path(pi);
-                __syncthreads();
-                if (mc[l] > 0) {
-                    fold_shared(pb, pb + mc[l]);
-                    __syncthreads();
-                }
-            }
-            for (int l = 0; l < Nk.nlevel; ++l) {
-                const int pe = lo[l + 1];
-                for (int pi = lo[l] + tid; pi < pe; pi += NT) substitute_path(pi);
-                __syncthreads();
-            }
-        }
-
-        if (a.item_ns) {
+    auto team_sync = []() {
+        if (COOP)
+            asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        else
             __syncthreads();
-            if (tid == 0) a.item_ns[gi] += global_ns() - t_item;
+    };
+    auto ld = [](const auto *p) { return COOP ? __ldcg(p) : *p; };
+    const unsigned long long t_item = (a.item_ns && tid == 0) ? global_ns() : 0ull;
+    const GroupRec G = a.groups[gi];
+    const int64_t c0 = G.comp0;
+    const int32_t *Vq = a.Vq + c0;
+    const float2 *gax = a.gax + c0;
+    const float2 *dpp = a.dp + c0;
+    float2 *dr = a.dr + G.scratch0;
+    float *drl = a.drl + G.scratch0;
+    float4 *pq = a.pq + G.pscratch0;
+    const unsigned char *blob = a.meta + G.meta_off;
+    const NrnG *nrns = (const NrnG *)blob;
+    const PathG *paths = (const PathG *)(blob + G.path_off);
+    const KidG *fold = (const KidG *)(blob + G.fold_off);
+    const int32_t *loffs = (const int32_t *)(blob + G.loffs_off);
+    const int32_t *mcnt = (const int32_t *)(blob + G.mcnt_off);
+
+    // S. synaptic sites (then their decay; sites are distinct
+    //    compartments), the current across each path's head link into
+    //    its head (for the path from a soma: the stimulus), then out of
+    //    the parent compartments, summed per parent in fold-list order
+    //    (as in step_fp32c_kernel)
+    for (int t = tid; t < G.nsite; t += NTT) {
+        const int st = G.site0 + t;
+        const int c = a.site_comp[st];
+        const float2 g0 = a.gsyn[st];
+        const mmf::F2 g = mmf::two_sum(g0.x, g0.y);
+        float2 v = ld(dr + c);
+        if (a.g_implicit) v.x += g.hi;
+        const mmf::F2 r = mmf::add(mmf::F2{v.y, ld(drl + c)}, mmf::neg(mmf::mul(g, vminus(Vq[c], a.Esyn))));
+        v.y = r.hi;
+        dr[c] = v;
+        drl[c] = r.lo;
+        a.gsyn[st] = tof2(mmf::mul(g, f2(a.decay)));
+    }
+    team_sync();
+    for (int pi = tid; pi < G.npath; pi += NTT) {
+        const PathG P = paths[pi];
+        mmf::F2 t;
+        if (P.parent >= 0) {
+            const float2 gs = gax[P.head];
+            t = mmf::mul(mmf::F2{fabsf(gs.x), gs.y}, mmf::vdiff_df(Vq[P.parent], Vq[P.head]));
+            pq[pi].z = t.hi;
+            pq[pi].w = t.lo;
+        } else {
+            t = mmf::split_d(a.stim[G.neuron0 + (P.nflag & kPathNeuronG)]);
+        }
+        const mmf::F2 r = mmf::add(mmf::F2{ld(&dr[P.head].y), ld(drl + P.head)}, t);
+        dr[P.head].y = r.hi;
+        drl[P.head] = r.lo;
+    }
+    team_sync();
+    for (int e = tid; e < G.npath; e += NTT) {
+        const int att = fold[e].y;
+        if (att < 0) continue;  // a path from a soma (no parent)
+        if (e > 0 && fold[e - 1].y == att) continue;  // not the first path of its parent
+        mmf::F2 t{0.f, 0.f};
+        for (int z = e; z < G.npath && fold[z].y == att; ++z) {
+            const float4 q = ld(pq + fold[z].x);
+            t = mmf::add(t, mmf::F2{q.z, q.w});
+        }
+        const mmf::F2 r = mmf::add(mmf::F2{ld(&dr[att].y), ld(drl + att)}, mmf::neg(t));
+        dr[att].y = r.hi;
+        drl[att] = r.lo;
+    }
+    team_sync();
+
+    // B. leaves-to-root elimination path by path, from the deepest level
+    //    up (as in step_fp32c_kernel: passive diagonal plus the active
+    //    conductance carried up the tree)
+    // the head of path pi once its interior is eliminated
+    auto eliminate_head = [&](int pi, const PathG &P, float eh, float rh) {
+        const int h = P.head;
+        const float dhh = dpp[h].x;
+        const float inv = rcp_nr(dhh + eh);
+        if (P.parent < 0) {  // soma: its dV
+            dr[h].y = rh * inv;
+            return;
+        }
+        const float2 gs = gax[h];
+        const float gh = a.gimp * fabsf(gs.x), gl = a.gimp * gs.y;
+        const float f = fmaf(gh, inv, gl * inv);
+        dr[h] = make_float2(f, rh * inv);
+        const float ce = gh * rcp_nr(dhh) * f * eh, cr = f * rh;
+        if (P.nflag & kPathAloneG) {
+            float2 v = ld(dr + P.parent);
+            v.x += ce;
+            v.y += cr;
+            dr[P.parent] = v;
+        } else {
+            pq[pi].x = ce;
+            pq[pi].y = cr;
+        }
+    };
+    auto eliminate_path = [&](int pi) {
+        const PathG P = paths[pi];
+        const int h = P.head;
+        int j = P.end - 1;
+        const float2 v0 = ld(dr + j);
+        float eb = v0.x, rb = v0.y, eh = eb, rh = rb;
+        float g0[8], l0[8], d0[8], q0[8], e0[8], r0[8];
+        float g1[8], l1[8], d1[8], q1[8], e1[8], r1[8];
+        auto load = [&](int jj, float *g, float *l, float *d, float *q, float *ee, float *r) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int x = max(jj - k, h + 1);
+                const float2 gs = __ldg(gax + x), w = ld(dr + x - 1);
+                g[k] = a.gimp * fabsf(gs.x);
+                l[k] = a.gimp * gs.y;
+                d[k] = __ldg(&dpp[x].x);
+                q[k] = (g[k] * rcp_nr(d[k])) * g[k];
+                ee[k] = w.x;
+                r[k] = w.y;
+            }
+        };
+        auto chain = [&](int jj, const float *g, const float *l, const float *d, const float *q,
+                         const float *ee, const float *r) {
+            const int cnt = jj - h;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const float dd = d[k] + eb;
+                const float r0 = rcp_approx(dd);
+                const float inv = fmaf(r0, fmaf(-dd, r0, 1.f), r0);
+                const float f = fmaf(g[k], inv, l[k] * inv);
+                if (k < cnt) dr[jj - k] = make_float2(f, rb * inv);
+                rb = fmaf(f, rb, r[k]);
+                eb = fmaf(q[k] * r0, eb, ee[k]);
+                if (k == cnt - 1) {
+                    eh = eb;
+                    rh = rb;
+                }
+            }
+        };
+        if (j > h) {
+            load(j, g0, l0, d0, q0, e0, r0);
+            for (;;) {
+                int jn = j - 8;
+                bool more = jn > h;
+                if (more) load(jn, g1, l1, d1, q1, e1, r1);
+                chain(j, g0, l0, d0, q0, e0, r0);
+                j = jn;
+                if (!more) break;
+                jn = j - 8;
+                more = jn > h;
+                if (more) load(jn, g0, l0, d0, q0, e0, r0);
+                chain(j, g1, l1, d1, q1, e1, r1);
+                j = jn;
+                if (!more) break;
+            }
+        }
+        eliminate_head(pi, P, eh, rh);
+    };
+    auto fold_shared = [&](int e0, int e1) {
+        for (int e = e0 + tid; e < e1; e += NTT) {
+            const KidG kv = fold[e];
+            if (e > e0 && fold[e - 1].y == kv.y) continue;
+            float4 q = ld(pq + kv.x);
+            float ad = q.x, ar = q.y;
+            for (int z = e + 1; z < e1; ++z) {
+                const KidG kz = fold[z];
+                if (kz.y != kv.y) break;
+                q = ld(pq + kz.x);
+                ad += q.x;
+                ar += q.y;
+            }
+            float2 v = ld(dr + kv.y);
+            v.x += ad;
+            v.y += ar;
+            dr[kv.y] = v;
+        }
+    };
+    // F. root-to-leaves substitution path by path; the path from a soma
+    //    runs the FP64 soma accumulator and the spike test
+    auto substitute_head = [&](const PathG &P) -> float {
+        const int h = P.head;
+        float x;
+        if (P.parent >= 0) {
+            const float2 fh = ld(dr + h);
+            x = fmaf(fh.x, ld(&dr[P.parent].y), fh.y);
+        } else {
+            x = ld(&dr[h].y);
+            const int nrn = G.neuron0 + (P.nflag & kPathNeuronG);
+            const double v0 = a.Vsoma[nrn], v1 = v0 + (double)x;
+            a.Vsoma[nrn] = v1;
+            if (!isfinite(v1)) atomicOr(&a.ctl->err, MMK_ERR_NUMERIC);
+            if (v0 < a.threshold && v1 >= a.threshold) {
+                const int src = soma_source(a, nrn);
+                if (src >= 0)
+                    record_spike(a, src, a.user_id[nrn], 0,
+                                 (double)n * a.dt64 + a.dt64 * (a.threshold - v0) / (v1 - v0), n);
+            }
+        }
+        return x;
+    };
+    auto substitute_path = [&](int pi) {
+        const PathG P = paths[pi];
+        const int h = P.head;
+        float x = substitute_head(P);
+        const float xh = x;
+        float f0[8], c0v[8], f1[8], c1v[8];
+        auto load = [&](int jj, float *f, float *c) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const float2 w = ld(dr + min(jj + k, P.end - 1));
+                f[k] = w.x;
+                c[k] = w.y;
+            }
+        };
+        auto chain = [&](int jj, const float *f, const float *c) {
+            const int cnt = P.end - jj;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                x = fmaf(f[k], x, c[k]);
+                if (k < cnt) dr[jj + k].y = x;
+            }
+        };
+        int j = h + 1;
+        if (j < P.end) {
+            load(j, f0, c0v);
+            for (;;) {
+                int jn = j + 8;
+                bool more = jn < P.end;
+                if (more) load(jn, f1, c1v);
+                chain(j, f0, c0v);
+                j = jn;
+                if (!more) break;
+                jn = j + 8;
+                more = jn < P.end;
+                if (more) load(jn, f0, c0v);
+                chain(j, f1, c1v);
+                j = jn;
+                if (!more) break;
+            }
+        }
+        if (P.parent >= 0) dr[h].y = xh;  // read by the next level only
+    };
+
+    // Paths of at least kGiantWarpPath compartments by a whole warp, as in
+    // step_fp32c_kernel: the interior cut into 32 chunks, the elimination
+    // of a chunk as the product of its 2x2 matrices and its rhs as an
+    // affine map, combined by warp scans.  A giant's long paths are what
+    // its solve waits for: one lane spends some hundred clocks of L2
+    // latency and arithmetic on each compartment.
+    const int lane = tid & 31, wid = tid >> 5;
+    // passive diagonal, coupling pair and g^2 / D of compartment x
+    struct Coef {
+        float D, gh, gl, q;
+    };
+    auto coef = [&](int x) -> Coef {
+        const float2 gs = __ldg(gax + x);
+        Coef c;
+        c.gh = a.gimp * fabsf(gs.x);
+        c.gl = a.gimp * gs.y;
+        c.D = __ldg(&dpp[x].x);
+        c.q = (c.gh * rcp_nr(c.D)) * c.gh;
+        return c;
+    };
+    auto eliminate_path_warp = [&](int pi) {
+        const PathG P = paths[pi];
+        const int h = P.head, e = P.end;
+        const int m = e - 1 - h;  // steps t = 0 .. m-1: compartment e-1-t into e-2-t
+        const int cs = (m + 31) >> 5;
+        const int t0 = min(lane * cs, m), t1 = min(t0 + cs, m);
+        const float2 leaf = ld(dr + e - 1);
+        float m00 = 1.f, m01 = 0.f, m10 = 0.f, m11 = 1.f;
+#pragma unroll 4
+        for (int t = t0; t < t1; ++t) {
+            const int j = e - 1 - t;
+            const Coef c = coef(j);
+            const float En = ld(&dr[j - 1].x), A = c.q + En, B = En * c.D;
+            const float n00 = fmaf(A, m00, B * m10), n01 = fmaf(A, m01, B * m11);
+            const float n10 = fmaf(c.D, m10, m00), n11 = fmaf(c.D, m11, m01);
+            const float sc = rcp_approx(n00 + n01 + n10 + n11);
+            m00 = n00 * sc;
+            m01 = n01 * sc;
+            m10 = n10 * sc;
+            m11 = n11 * sc;
+        }
+        for (int off = 1; off < 32; off <<= 1) {
+            const float a00 = __shfl_up_sync(0xFFFFFFFFu, m00, off), a01 = __shfl_up_sync(0xFFFFFFFFu, m01, off);
+            const float a10 = __shfl_up_sync(0xFFFFFFFFu, m10, off), a11 = __shfl_up_sync(0xFFFFFFFFu, m11, off);
+            if (lane >= off) {  // this lane's chunks act after the earlier ones
+                const float n00 = fmaf(m00, a00, m01 * a10), n01 = fmaf(m00, a01, m01 * a11);
+                const float n10 = fmaf(m10, a00, m11 * a10), n11 = fmaf(m10, a01, m11 * a11);
+                const float sc = rcp_approx(fabsf(n00) + fabsf(n01) + fabsf(n10) + fabsf(n11));
+                m00 = n00 * sc;
+                m01 = n01 * sc;
+                m10 = n10 * sc;
+                m11 = n11 * sc;
+            }
+        }
+        const float e00 = __shfl_up_sync(0xFFFFFFFFu, m00, 1), e01 = __shfl_up_sync(0xFFFFFFFFu, m01, 1);
+        const float e10 = __shfl_up_sync(0xFFFFFFFFu, m10, 1), e11 = __shfl_up_sync(0xFFFFFFFFu, m11, 1);
+        const float eb0 = lane ? fmaf(e00, leaf.x, e01) / fmaf(e10, leaf.x, e11) : leaf.x;
+        // pass 1 (reads only): the active conductance through the chunk
+        // and the chunk's affine map of the rhs recurrence; the element
+        // after the chunk is kept for pass 2, whose writes it may see
+        float eb = eb0, A = 1.f, B = 0.f;
+        float2 nb = make_float2(0.f, 0.f);
+#pragma unroll 4
+        for (int t = t0; t < t1; ++t) {
+            const int j = e - 1 - t;
+            const Coef c = coef(j);
+            const float2 w = ld(dr + j - 1);
+            const float dd = c.D + eb, r0 = rcp_approx(dd), inv = fmaf(r0, fmaf(-dd, r0, 1.f), r0);
+            const float f = fmaf(c.gh, inv, c.gl * inv);
+            A *= f;
+            B = fmaf(f, B, w.y);
+            eb = fmaf(c.q * r0, eb, w.x);
+            nb = w;
+        }
+        for (int off = 1; off < 32; off <<= 1) {
+            const float pa = __shfl_up_sync(0xFFFFFFFFu, A, off), pb = __shfl_up_sync(0xFFFFFFFFu, B, off);
+            if (lane >= off) {
+                B = fmaf(A, pb, B);
+                A *= pa;
+            }
+        }
+        const float ea = __shfl_up_sync(0xFFFFFFFFu, A, 1), ebs = __shfl_up_sync(0xFFFFFFFFu, B, 1);
+        // pass 2: the substitution coefficients (f_j, c_j) of the chunk
+        __syncwarp();
+        eb = eb0;
+        float rb = lane ? fmaf(ea, leaf.y, ebs) : leaf.y;
+        for (int t = t0; t < t1; ++t) {
+            const int j = e - 1 - t;
+            const Coef c = coef(j);
+            const float2 w = t + 1 < t1 ? ld(dr + j - 1) : nb;
+            const float dd = c.D + eb, r0 = rcp_approx(dd), inv = fmaf(r0, fmaf(-dd, r0, 1.f), r0);
+            const float f = fmaf(c.gh, inv, c.gl * inv);
+            dr[j] = make_float2(f, rb * inv);
+            rb = fmaf(f, rb, w.y);
+            eb = fmaf(c.q * r0, eb, w.x);
+        }
+        // the head, from the lane whose chunk ends at it
+        const int lastl = (m - 1) / cs;
+        const float eh = __shfl_sync(0xFFFFFFFFu, eb, lastl), rh = __shfl_sync(0xFFFFFFFFu, rb, lastl);
+        __syncwarp();
+        if (lane == 0) eliminate_head(pi, P, eh, rh);
+        __syncwarp();
+    };
+    auto substitute_path_warp = [&](int pi) {
+        const PathG P = paths[pi];
+        const int h = P.head, e = P.end;
+        float x = 0.f;
+        if (lane == 0) x = substitute_head(P);
+        x = __shfl_sync(0xFFFFFFFFu, x, 0);
+        const int m = e - 1 - h;  // t = 0 .. m-1 <-> j = h+1+t
+        const int cs = (m + 31) >> 5;
+        const int t0 = min(lane * cs, m), t1 = min(t0 + cs, m);
+        float A = 1.f, B = 0.f;
+#pragma unroll 4
+        for (int t = t0; t < t1; ++t) {
+            const float2 w = ld(dr + h + 1 + t);
+            A *= w.x;
+            B = fmaf(w.x, B, w.y);
+        }
+        for (int off = 1; off < 32; off <<= 1) {
+            const float pa = __shfl_up_sync(0xFFFFFFFFu, A, off), pb = __shfl_up_sync(0xFFFFFFFFu, B, off);
+            if (lane >= off) {
+                B = fmaf(A, pb, B);
+                A *= pa;
+            }
+        }
+        const float ea = __shfl_up_sync(0xFFFFFFFFu, A, 1), eb = __shfl_up_sync(0xFFFFFFFFu, B, 1);
+        float xs = lane ? fmaf(ea, x, eb) : x;
+        for (int t = t0; t < t1; ++t) {
+            const int j = h + 1 + t;
+            const float2 w = ld(dr + j);
+            xs = fmaf(w.x, xs, w.y);
+            dr[j].y = xs;
+        }
+        __syncwarp();
+        if (lane == 0 && P.parent >= 0) dr[h].y = x;  // read by the next level only
+    };
+    // the number of paths at the start of a level (paths run longest
+    // first) that a whole warp takes
+    auto warp_paths = [&](int pb, int pe) {
+        int lo = pb, hi = pe;  // first path shorter than the threshold
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (paths[mid].end - paths[mid].head >= kGiantWarpPath) lo = mid + 1; else hi = mid;
+        }
+        return lo - pb;
+    };
+
+    for (int k = 0; k < G.nbundle; ++k) {
+        const NrnG Nk = nrns[k];
+        const int32_t *lo = loffs + Nk.loff0;
+        const int32_t *mc = mcnt + Nk.loff0;
+        for (int l = Nk.nlevel - 1; l >= 0; --l) {
+            const int pb = lo[l], pe = lo[l + 1];
+            const int nw = warp_paths(pb, pe);
+            for (int q = wid; q < nw; q += NTT / 32) eliminate_path_warp(pb + q);
+            for (int pi = pb + nw + tid; pi < pe; pi += NTT) eliminate_path(pi);
+            team_sync();
+            if (mc[l] > 0) {
+                fold_shared(pb, pb + mc[l]);
+                team_sync();
+            }
+        }
+        for (int l = 0; l < Nk.nlevel; ++l) {
+            const int pb = lo[l], pe = lo[l + 1];
+            const int nw = warp_paths(pb, pe);
+            for (int q = wid; q < nw; q += NTT / 32) substitute_path_warp(pb + q);
+            for (int pi = pb + nw + tid; pi < pe; pi += NTT) substitute_path(pi);
+            team_sync();
         }
     }
+
+    if (a.item_ns) {
+        team_sync();
+        if (tid == 0) a.item_ns[gi] += global_ns() - t_item;
+    }
+}
+
+template <int NT>
+__global__ void __launch_bounds__(NT) giant_fp32c_kernel(StepArgs32 a)
+{
+    // The first a.n_huge items are solved by a cluster of blocks each, all its
+    // threads as one team: a lane waits some hundred clocks for each
+    // compartment of its path, so what a huge neuron wants is more lanes than
+    // one SM's.  The other clusters' blocks take an item each, by themselves
+    // (every team has one item: the launch is sized so).  Two neurons of 100,000
+    // compartments among 19 of 9,000 to 20,000: the solve 508 us with a block per
+    // neuron and a lane per path, 298 us with clusters of eight blocks and a warp
+    // on each path of 48 compartments or more; the whole step (1,502 neurons)
+    // 554 -> 340 us.  Thresholds of 32 and 96: 350 and 390 us; clusters of 16, 504
+    // us (they wait for 16 free SMs); clusters for the small giants too, 371 us.
+    int nblk, rank;
+    asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(nblk));
+    asm("mov.u32 %0, %%cluster_ctaid.x;" : "=r"(rank));
+    const int cl = (int)blockIdx.x / nblk;
+    if (nblk > 1 && cl < a.n_huge) {
+        giant_solve<NT, true>(a, a.item0 + cl, rank * NT + (int)threadIdx.x, nblk * NT);
+        return;
+    }
+    const int gi = a.item0 + (nblk > 1 ? a.n_huge + (cl - a.n_huge) * nblk + rank : cl);
+    if (gi < a.item1) giant_solve<NT, false>(a, gi, (int)threadIdx.x, NT);
 }
 
 // The giant items' compartments in chunks of kGiantChunk: chunk ch belongs
 // to the giant item k with gchunk0[k] <= ch < gchunk0[k + 1].
-constexpr int kGiantChunk = 2048;
+constexpr int kGiantChunk = 512;  // 23 -> 15 us and 25 -> 17 us for 0.48 M compartments, against 2,048
 
 __device__ __forceinline__ int giant_of_chunk(const StepArgs32 &a, int64_t ch)
 {
@@ -1320,8 +1513,18 @@ int set_attr_and_occupancy(int smem, int *blocks)
 
 int mmk_launch_giant_fp32c(const StepArgs32 &a, int blocks, void *stream)
 {
-    giant_fp32c_kernel<256><<<blocks, 256, 0, (cudaStream_t)stream>>>(a);
-    return (int)cudaGetLastError();
+    // clusters of eight blocks where the launch holds huge items
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(256);
+    cfg.stream = (cudaStream_t)stream;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = a.n_huge > 0 ? kGiantCluster : 1;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return (int)cudaLaunchKernelEx(&cfg, giant_fp32c_kernel<256>, a);
 }
 
 int mmk_launch_giant_assemble(const StepArgs32 &a, int chunk_blocks, void *stream)
@@ -1334,6 +1537,11 @@ int mmk_launch_giant_update(const StepArgs32 &a, int chunk_blocks, void *stream)
 {
     giant_update_kernel<<<chunk_blocks, 256, 0, (cudaStream_t)stream>>>(a);
     return (int)cudaGetLastError();
+}
+
+int mmk_giant_blocks(int n_giant, int n_huge)
+{
+    return n_huge > 0 ? kGiantCluster * (n_huge + (n_giant - n_huge + kGiantCluster - 1) / kGiantCluster) : n_giant;
 }
 
 int mmk_giant_chunk()
