@@ -93,7 +93,9 @@ struct mm_net {
 
     // device arrays (FP64 path)
     double *V = nullptr, *m = nullptr, *h = nullptr, *n = nullptr;
-    double *area = nullptr, *gax = nullptr, *dcon = nullptr, *gsyn = nullptr;
+    double *area = nullptr, *gax = nullptr, *gsyn = nullptr;
+    double *sc = nullptr, *s2a = nullptr, *dcon = nullptr;  // the scaled Hines system (StepArgs)
+    int32_t *kexp = nullptr;
     double2 *gtab64 = nullptr;        // gate table for dt (mm_gate_table64.h)
     // device arrays (FP32c path)
     int32_t *Vq = nullptr;
@@ -662,6 +664,9 @@ mm_status build(mm_net *net, const mm_morphologies *morph, const mm_channel_para
         ZR(net->area, C);
         ZR(net->gax, C);
         ZR(net->dcon, C);
+        ZR(net->sc, C);
+        ZR(net->s2a, C);
+        ZR(net->kexp, C);
         {
             std::vector<mmg::Quad64> tab((size_t)mmg::kTab64Quads * mmg::kTab64Intervals);
             mmg::build_table64(opt->dt_ms, tab.data());
@@ -775,15 +780,15 @@ mm_status build(mm_net *net, const mm_morphologies *morph, const mm_channel_para
     if (f64) {
         ia.area = net->area;
         ia.gax = net->gax;
-        ia.dcon = net->dcon;
-        ia.cm_dt = chan->Cm * 1e3 / opt->dt_ms;
-        ia.gimp = opt->scheme == MM_SCHEME_CN ? 0.5 : 1.0;
-        ia.gleak = opt->scheme == MM_SCHEME_CN ? 0.0 : chan->gL * 1e3;
         ia.V = net->V;
         ia.m = net->m;
         ia.h = net->h;
         ia.n = net->n;
         MM_CKI(net, mmk_launch_init(ia, net->stream));
+        const bool cn = opt->scheme == MM_SCHEME_CN;
+        mmk::ScaleArgs64 sa{dgroups, dmeta, net->area, net->gax, net->sc, net->s2a, net->dcon, net->kexp,
+                            cn ? 0.5 : 1.0, chan->Cm * 1e3 / opt->dt_ms + (cn ? 0.0 : chan->gL * 1e3)};
+        MM_CKI(net, mmk_launch_scale(sa, (int)L.groups.size(), net->stream));
     } else {
         ia.Vq = net->Vq;
         ia.mq = net->mq;
@@ -804,6 +809,9 @@ mm_status build(mm_net *net, const mm_morphologies *morph, const mm_channel_para
         a.area = net->area;
         a.gax = net->gax;
         a.dcon = net->dcon;
+        a.sc = net->sc;
+        a.s2a = net->s2a;
+        a.kexp = net->kexp;
         a.gtab = net->gtab64;
         a.stim = net->stim;
         a.user_id = net->user_id;
@@ -834,7 +842,6 @@ mm_status build(mm_net *net, const mm_morphologies *morph, const mm_channel_para
         a.ENa = chan->ENa;
         a.EK = chan->EK;
         a.EL = chan->EL;
-        a.gimp = opt->scheme == MM_SCHEME_CN ? 0.5 : 1.0;
         a.g_implicit = opt->scheme == MM_SCHEME_CN ? 0 : 1;
         a.e_syn = syn ? syn->e_rev_mV : 0.0;
         a.threshold = chan->threshold_mV;

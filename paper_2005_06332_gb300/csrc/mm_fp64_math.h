@@ -9,15 +9,14 @@
 
 namespace mmk {
 
-// 1/x by Newton's iteration from the approximate reciprocal (about 20 bits):
-// two steps reach FP64 rounding, half the instructions of the compiled
-// division.
+// 1/x from the approximate reciprocal (about 20 bits) by one step of third
+// order, r (1 + e + e^2) with e = 1 - x r: FP64 rounding in three instructions.
 __device__ __forceinline__ double rcp_nr(double x)
 {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    r = fma(r, fma(-x, r, 1.0), r);
-    return fma(r, fma(-x, r, 1.0), r);
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
 }
 
 // a / x given r = rcp_nr(x): one residual correction
@@ -25,6 +24,28 @@ __device__ __forceinline__ double div_nr(double a, double x, double r)
 {
     const double q = a * r;
     return fma(r, fma(-x, q, a), q);
+}
+
+// x 2^(d >> 20); d a difference of exponent fields
+__device__ __forceinline__ double scale2(double x, int d)
+{
+    const int h = __double2hiint(x), e = h & 0x7FF00000, ne = e + d;
+    if (e != 0 && e != 0x7FF00000 && ne > 0 && ne < 0x7FF00000) return __hiloint2double(h + d, __double2loint(x));
+    return (x == 0.0 || e == 0x7FF00000) ? x : scalbn(x, d >> 20);
+}
+
+// the exponent field of x less that of 1 (0 for zero, subnormals, infinities
+// and NaN, which then stay as they are): scale2(x, -that) lies in [1, 2)
+__device__ __forceinline__ int exponent2(double x)
+{
+    const uint32_t e = (uint32_t)__double2hiint(x) & 0x7FF00000u;
+    return e - 0x00100000u < 0x7FE00000u ? (int)e - 0x3FF00000 : 0;
+}
+
+// x 2^-(exponent2(x) >> 20)
+__device__ __forceinline__ double mantissa(double x)
+{
+    return __hiloint2double(__double2hiint(x) - exponent2(x), __double2loint(x));
 }
 
 }  // namespace mmk

@@ -77,15 +77,6 @@ constexpr int kBlockComps = 2048;  // compartments aimed at per block
 constexpr long long kLeft = 0x7FF8A5C3966D1E27LL;  // in the scratch, at the first entry of a block that was left
 constexpr size_t smem_of(int chains) { return (size_t)chains * 20 + 16; }
 
-// x 2^-(d >> 20); d the difference of two exponent fields
-__device__ __forceinline__ double scale_down(double x, int d)
-{
-    const int h = __double2hiint(x), e = h & 0x7FF00000;
-    const int ne = e - d;
-    if (e != 0 && e != 0x7FF00000 && ne > 0 && ne < 0x7FF00000) return __hiloint2double(h - d, __double2loint(x));
-    return (x == 0.0 || e == 0x7FF00000) ? x : scalbn(x, -(d >> 20));
-}
-
 // One entry of a chain's elimination: N / M is its eliminated diagonal, S / M
 // its rhs.
 struct Front {
@@ -94,24 +85,13 @@ struct Front {
     // (the division by it is what fails in Algorithm 1)
     __device__ __forceinline__ void normalise()
     {
-        const int h = __double2hiint(N), e = h & 0x7FF00000;
-        if (e == 0 || e == 0x7FF00000) {
-            if (N == 0.0) N = __longlong_as_double(0x7FF8000000000000LL);
-            return;
-        }
-        const int d = e - 0x3FF00000;
-        N = __hiloint2double(h - d, __double2loint(N));
-        M = scale_down(M, d);
-        S = scale_down(S, d);
+        const int d = mmk::exponent2(N);
+        if (((__double2hiint(N) & 0x7FFFFFFF) | __double2loint(N)) == 0) N = __longlong_as_double(0x7FF8000000000000LL);
+        N = __hiloint2double(__double2hiint(N) - d, __double2loint(N));
+        M = mmk::scale2(M, -d);
+        S = mmk::scale2(S, -d);
     }
 };
-
-// the N that Front::normalise leaves
-__device__ __forceinline__ double normalised(double N)
-{
-    const int h = __double2hiint(N), e = h & 0x7FF00000;
-    return e == 0 || e == 0x7FF00000 ? N : __hiloint2double(h - e + 0x3FF00000, __double2loint(N));
-}
 
 // A block solves trees_per_block consecutive trees together.  Bound by the
 // FP64 pipe and, for the largest trees, by the chain of their sweeps: a warp's
@@ -416,7 +396,7 @@ __device__ __forceinline__ void solve_group(const Batch &B, int group)
                 N[u] = work[i];
                 S[u] = x[i];
                 cc[u] = __ldg(c + i);
-                M[u] = i + 1 < n && parent[i + 1] >= 0 && tb + parent[i + 1] == i ? normalised(work[i + 1]) : 1.0;
+                M[u] = i + 1 < n && parent[i + 1] >= 0 && tb + parent[i + 1] == i ? mmk::mantissa(work[i + 1]) : 1.0;
             }
         }
         __syncthreads();  // the entry above has read this one's N

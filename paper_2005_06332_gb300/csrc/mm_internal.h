@@ -120,8 +120,11 @@ struct StepArgs {
     const double *area;               // membrane area, cm^2 [C]
     const double *gax;                // axial conductance to the parent, uS [C] (0 at a soma), negated at path
                                       // heads (somata included): their link is assembled per path
-    const double *dcon;               // constant part of the diagonal, uS [C]: C/dt, the leak (backward Euler)
-                                      // and the implicit couplings of the links inside paths
+    // the Hines system scaled by s on both sides (scale_kernel) [C]: s, or at path heads minus the coupling
+    // to the parent (s is 1 there); s^2 area; the constant part of the diagonal; and the exponent field of
+    // the coupling to the parent inside a path
+    const double *sc, *s2a, *dcon;
+    const int32_t *kexp;
     const double2 *gtab;              // gate table for dt (mm_gate_table64.h): 18 arrays of 961 16-byte quads
     const double *stim;               // soma current per internal neuron, nA [N]
     const int32_t *user_id;           // internal neuron -> user id [N]
@@ -154,12 +157,21 @@ struct StepArgs {
     double gNa, gK, gL;               // channel densities times 1e3: uS per cm^2 of membrane
     double ENa, EK, EL;
     double e_syn, threshold, dt, decay;
-    // time discretisation (MM_SCHEME_*): the implicit share of each axial
-    // coupling (1, or 1/2 for Eq. 2 as printed) and whether the membrane
-    // conductance enters the diagonal (backward Euler) or stays explicit
-    double gimp;
+    // time discretisation (MM_SCHEME_*): whether the membrane conductance
+    // enters the diagonal (backward Euler) or stays explicit
     int32_t g_implicit;
     int32_t pad_scheme;
+};
+
+// Arguments of the FP64 scaling kernel (see StepArgs).
+struct ScaleArgs64 {
+    const GroupRec *groups;
+    const unsigned char *meta;
+    const double *area, *gax;
+    double *sc, *s2a, *dcon;
+    int32_t *kexp;
+    double gimp;                      // implicit share of each axial coupling: 1, or 1/2 for Eq. 2 as printed
+    double cm_leak;                   // (Cm / dt + the implicit leak) * 1e3: uS per cm^2 of membrane
 };
 
 // Fixed-point state of the FP32c path: V = Vq * 2^-23 mV (int32, +-256 mV),
@@ -333,11 +345,8 @@ struct InitArgs {
     const int32_t *parent_dist;       // i - parent(i), negated at path heads, 0 at a soma
     int64_t C;
     double *area, *gax;
-    double *dcon;                     // FP64: see StepArgs
     double *V, *m, *h, *n;
     double Ra, v_init;
-    double cm_dt;                     // Cm * 1e3 / dt: C_i/dt = area_i * cm_dt (nF/ms = uS)
-    double gleak, gimp;               // implicit leak (uS per cm^2, 0 under Eq. 2 as printed), coupling share
     // FP32c outputs (used when Vq != nullptr; the FP64 pointers are then
     // unused; the FP32c constants are computed on the host)
     int32_t *Vq;
@@ -349,6 +358,7 @@ struct InitArgs {
 // Launch wrappers (defined in the .cu files; return a cudaError_t as int).
 extern "C++" {
 int mmk_launch_init(const mmk::InitArgs &a, void *stream);
+int mmk_launch_scale(const mmk::ScaleArgs64 &a, int n_groups, void *stream);
 int mmk_launch_deliver(const mmk::DeliverArgs &a, int blocks, void *stream);
 int mmk_launch_step_fp64(const mmk::StepArgs &a, int blocks, int threads, void *stream);
 int mmk_step_fp64_blocks_per_sm(int threads, int smem_bytes, int *blocks);

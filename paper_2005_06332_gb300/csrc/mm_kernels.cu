@@ -67,29 +67,84 @@ __device__ __forceinline__ double half_cyl_resistance(double Ra, double L_um, do
 
 // ------------------------------------------------------------------ init
 
-// Areas, axial conductances (negated at path heads), the constant part of the
-// diagonal, and the resting state.
+// Areas, axial conductances (negated at path heads) and the resting state.
 __global__ void init_kernel(InitArgs a)
 {
-    auto axial = [&](int64_t i, int64_t q) {
-        return 1.0 / (half_cyl_resistance(a.Ra, a.L[i], a.diam[i]) + half_cyl_resistance(a.Ra, a.L[q], a.diam[q]));
-    };
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.C;
          i += (int64_t)gridDim.x * blockDim.x) {
-        const double area = kPi * a.diam[i] * a.L[i] * 1e-8;
-        a.area[i] = area;
+        const double L = a.L[i], d = a.diam[i];
+        a.area[i] = kPi * d * L * 1e-8;
         const int32_t pd = a.parent_dist[i];
-        const double g = pd != 0 ? axial(i, i - abs(pd)) : 0.0;
+        double g = 0.0;
+        if (pd != 0) {
+            const int64_t q = i - abs(pd);
+            g = 1.0 / (half_cyl_resistance(a.Ra, L, d) + half_cyl_resistance(a.Ra, a.L[q], a.diam[q]));
+        }
         a.gax[i] = pd > 0 ? g : -g;
-        double coupling = g;
-        if (i + 1 < a.C && a.parent_dist[i + 1] == 1) coupling += axial(i + 1, i);
-        a.dcon[i] = area * a.cm_dt + a.gleak * area + a.gimp * coupling;
         double v = a.v_init;
         Rates r = hh_rates(v);
         a.V[i] = v;
         a.m[i] = r.am / (r.am + r.bm);
         a.h[i] = r.ah / (r.ah + r.bh);
         a.n[i] = r.an / (r.an + r.bn);
+    }
+}
+
+// The scaling of each work item's Hines system (see step_fp64_kernel), a block
+// per item: down each path s = 1 at its head and then the mantissa of
+// 1 / (w g s_parent) (w the implicit share of a coupling), so that the coupling
+// w g s s_parent inside a path is a power of two, whose exponent field is
+// stored; at a head the coupling to the parent compartment, negative.  Then the
+// constant part of the diagonal: C/dt, the implicit leak and the couplings,
+// times s^2 -- inside a path as the matrix holds them, s 2^k / s_parent.
+__global__ void __launch_bounds__(128) scale_kernel(ScaleArgs64 a)
+{
+    const GroupRec G = a.groups[blockIdx.x];
+    const unsigned char *blob = a.meta + G.meta_off;
+    const PathQ *paths = (const PathQ *)(blob + G.path_off);
+    const KidQ *fold = (const KidQ *)(blob + G.fold_off);
+    const double *area = a.area + G.comp0, *gax = a.gax + G.comp0;
+    double *sc = a.sc + G.comp0, *s2a = a.s2a + G.comp0, *dcon = a.dcon + G.comp0;
+    int32_t *kexp = a.kexp + G.comp0;
+    auto scale_of = [&](int i) { return signbit(sc[i]) ? 1.0 : sc[i]; };
+    for (int pi = threadIdx.x; pi < G.npath; pi += 128) {
+        const PathQ P = paths[pi];
+        const int h = P.head;
+        double s = 1.0, own = a.gimp * fabs(gax[h]);  // own: s^2 w g of the link to the parent
+        for (int j = h; j < P.end; ++j) {
+            double sn = 1.0, link = 0.0, next_own = 0.0;
+            if (j + 1 < P.end) {
+                const double p = 1.0 / (a.gimp * gax[j + 1] * s);
+                sn = mantissa(p);
+                const int k = -exponent2(p);
+                kexp[j + 1] = k;
+                link = scale2(s / sn, k);
+                next_own = scale2(sn / s, k);
+            }
+            const double s2 = s * s * area[j];
+            sc[j] = j == h ? -0.0 : s;
+            if (j == h) kexp[j] = 0;
+            s2a[j] = s2;
+            dcon[j] = s2 * a.cm_leak + (own + link);
+            s = sn;
+            own = next_own;
+        }
+    }
+    __syncthreads();
+    for (int pi = threadIdx.x; pi < G.npath; pi += 128) {
+        const PathQ P = paths[pi];
+        if (P.parent >= 0) sc[P.head] = -(a.gimp * fabs(gax[P.head]) * scale_of(P.parent));
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < G.npath; e += 128) {
+        const int att = (int)(fold[e] >> 16);
+        if (att >= G.ncomp) continue;  // a path from a soma (no parent)
+        if (e > 0 && (int)(fold[e - 1] >> 16) == att) continue;  // not the first path of its parent
+        double d = dcon[att];
+        const double s = scale_of(att);
+        for (int z = e; z < G.npath && (int)(fold[z] >> 16) == att; ++z)
+            d = fma(-sc[paths[fold[z] & 0xFFFFu].head], s, d);
+        dcon[att] = d;
     }
 }
 
@@ -188,21 +243,6 @@ __global__ void __launch_bounds__(256) deliver_ordered_kernel(DeliverArgs a)
 
 // ------------------------------------------------------------ FP64 step
 
-// 2^-exponent(x) for a normal x (x times it lies in [1, 2)); 1 for zero,
-// infinities and NaN, which stay as they are
-__device__ __forceinline__ double pow2_inverse(double x)
-{
-    const uint32_t e = (uint32_t)__double2hiint(x) & 0x7FF00000u;
-    return __hiloint2double(e - 0x00100000u < 0x7FD00000u ? (int)(0x7FE00000u - e) : 0x3FF00000, 0);
-}
-
-// x times pow2_inverse(x), by integer operations
-__device__ __forceinline__ double mantissa(double x)
-{
-    const uint32_t h = (uint32_t)__double2hiint(x), e = h & 0x7FF00000u;
-    return e - 0x00100000u < 0x7FD00000u ? __hiloint2double((int)(h - e + 0x3FF00000u), __double2loint(x)) : x;
-}
-
 // Exponential-Euler gate update at V^{n+1} of one compartment (its V is final
 // for this step): from the table, or beyond its range from the rates.
 __device__ __forceinline__ void gate_update(const StepArgs &a, int64_t c)
@@ -255,9 +295,6 @@ __device__ __forceinline__ void gate_chunks(const StepArgs &a, int64_t pc0, int 
 constexpr int kSweepChunk = 4;
 // Paths of at least this many compartments are swept by a whole warp.
 constexpr int kWarpPath = 96;
-// The products of a path's elimination are rescaled before every compartment
-// whose group-local index is kRescale - 1 modulo kRescale.
-constexpr int kRescale = 8;
 
 template <int NT>
 __global__ void __launch_bounds__(NT, NT <= 256 ? 512 / NT : 1) step_fp64_kernel(StepArgs a)
@@ -269,25 +306,31 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 512 / NT : 1) step_fp64_kernel
     //   * the gates come from the table (mm_gate_table64.h), with the constant
     //     part of the diagonal stored per compartment;
     //   * the sweeps are the part with few active lanes (one lane per
-    //     path), so they multiply only: the elimination carries
-    //     d'_j = N_j / M_j and rhs'_j = S_j / M_j as products,
-    //       N_{j-1} = d_{j-1} N_j - g_j^2 M_j,  M_{j-1} = N_j,
-    //       S_{j-1} = r_{j-1} N_j + g_j S_j
-    //     (Algorithm 1's row times M; powers of two are taken out along the
-    //     way), and the division for the substitution's factors
-    //     f_j = g_j M_j / N_j, c_j = S_j / N_j is a pass of full warps;
+    //     path), so they hold two instructions a compartment and no division.
+    //     The elimination carries d'_j = N_j / M_j and rhs'_j = S_j / M_j,
+    //       N_{j-1} = d_{j-1} N_j - gamma_j^2 M_j,  M_{j-1} = N_j,
+    //       S_{j-1} = r_{j-1} N_j + gamma_j S_j
+    //     (Algorithm 1's row times M) on the system scaled by s on both sides
+    //     (scale_kernel; the unknown is y = dV / s) so that gamma is a power of
+    //     two inside a path: the products by it, and the powers of two taken
+    //     out of N, M and S at each step, are integer additions.  The division
+    //     for the substitution's factors f_j = gamma_j M_j / N_j, c_j = S_j / N_j
+    //     is a pass of full warps;
     //   * warps without a sweep update the gates of the block's previous item.
     // Work items, teams, bundles, levels and the fold list are the FP32c
     // kernel's (step_fp32c_kernel), with the diagonal and rhs in FP64.
-    // Measured per step: 2,000 neurons of 50 to 5,000 compartments (2.14 M)
-    // 1.81 -> 0.74 ms (119 FP64 warp instructions per 32 compartments, pipe 75 %
-    // busy while an SM has work); 64 of 255 compartments 370 -> 159 us; 701 of
-    // 50 to 3,000, points and ordered delivery, 808 -> 262 us.
+    // Measured per step, items of 4,096 compartments: 2,000 neurons of 50 to
+    // 5,000 compartments (2.14 M) 1.81 ms with divisions in the sweeps and the
+    // rates evaluated, 0.74 ms with the table and products (five instructions a
+    // sweep step), 0.55 ms on the scaled system (two); 64 neurons of 255 370,
+    // 159, 121 us; 701 of 50 to 3,000, points and ordered delivery, 808, 262,
+    // 185 us.  Warps on paths from 48 or 160 compartments instead of 96: 5 % and
+    // 2 % slower; three or four blocks per SM (85 or 64 registers) 2 to 10 %.
     //
     // Shared memory: the item's tree blob (one bulk copy), then per
     // compartment the pair (diagonal, rhs) -- after a path's elimination
     // (N, S) for its inside and (-f, c) for its head, whose sign says that the
-    // division is done, then (f, c), after substitution (f, dV).
+    // division is done, then (f, c), after substitution (f, y).
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned char *smeta = smem_raw;
     __shared__ __align__(8) uint64_t bar;
@@ -328,7 +371,10 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 512 / NT : 1) step_fp64_kernel
         const int64_t c0 = G.comp0;
         const double *V = a.V + c0;
         const double *gax = a.gax + c0;
+        const double *sc = a.sc + c0;
+        const int32_t *kexp = a.kexp + c0;
         double2 *sdr = (double2 *)(smem_raw + G.meta_bytes);
+        auto scale_of = [&](int i) { const double s = __ldg(sc + i); return signbit(s) ? 1.0 : s; };
 
         // A. diagonal and rhs at (V^n, gates^n): membrane conductance and
         //    current, and the axial currents of the links inside paths (a
@@ -337,16 +383,18 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 512 / NT : 1) step_fp64_kernel
 #pragma unroll 2
         for (int i = tid; i < G.ncomp; i += NT) {
             const double v = V[i], mm = a.m[c0 + i], hh = a.h[c0 + i], nn = a.n[c0 + i];
-            const double s = a.area[c0 + i], g = gax[i];
+            const double ar = a.area[c0 + i], g = gax[i];
             const double gna = a.gNa * ((mm * mm) * (mm * hh)), n2 = nn * nn, gk = a.gK * (n2 * n2);
             double d = a.dcon[c0 + i];
-            if (a.g_implicit) d = fma(s, gna + gk, d);
-            double r = -s * fma(gna, v - a.ENa, fma(gk, v - a.EK, a.gL * (v - a.EL)));
+            if (a.g_implicit) d = fma(a.s2a[c0 + i], gna + gk, d);
+            double r = -ar * fma(gna, v - a.ENa, fma(gk, v - a.EK, a.gL * (v - a.EL)));
             if (!signbit(g)) r = fma(g, V[i - 1] - v, r);
             if (i + 1 < G.ncomp) {
                 const double gc = gax[i + 1];
                 if (!signbit(gc)) r = fma(gc, V[i + 1] - v, r);
             }
+            const double s = sc[i];
+            if (!signbit(s)) r *= s;
             sdr[i] = make_double2(d, r);
         }
         if (!mbar_wait_bounded(&bar, parity)) {
@@ -371,15 +419,16 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 512 / NT : 1) step_fp64_kernel
         // S. synaptic sites (then their decay; sites are distinct
         //    compartments), the current across each path's head link into its
         //    head (for the path from a soma the stimulus), then per parent
-        //    compartment the conductances and currents of the links to the
-        //    heads that hang off it, in fold-list order.
+        //    compartment the currents of the links to the heads that hang off
+        //    it, in fold-list order.
         for (int t = tid; t < G.nsite; t += NT) {
             const int st = G.site0 + t;
             const int c = a.site_comp[st];
             const double g = a.gsyn[st];
             double2 w = sdr[c];
-            if (a.g_implicit) w.x += g;
-            w.y = fma(-g, V[c] - a.e_syn, w.y);
+            const double s = scale_of(c), t1 = s * g;
+            if (a.g_implicit) w.x = fma(t1, s, w.x);
+            w.y = fma(-t1, V[c] - a.e_syn, w.y);
             sdr[c] = w;
             a.gsyn[st] = g * a.decay;
         }
@@ -396,15 +445,13 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 512 / NT : 1) step_fp64_kernel
             const int att = (int)(fold[e] >> 16);
             if (att >= G.ncomp) continue;  // a path from a soma (no parent)
             if (e > 0 && (int)(fold[e - 1] >> 16) == att) continue;  // not the first path of its parent
-            double2 w = sdr[att];
             const double vp = V[att];
+            double t = 0.0;
             for (int z = e; z < G.npath && (int)(fold[z] >> 16) == att; ++z) {
                 const int h = paths[fold[z] & 0xFFFFu].head;
-                const double g = fabs(gax[h]);
-                w.x = fma(a.gimp, g, w.x);
-                w.y = fma(g, V[h] - vp, w.y);
+                t = fma(fabs(gax[h]), V[h] - vp, t);
             }
-            sdr[att] = w;
+            sdr[att].y = fma(scale_of(att), t, sdr[att].y);
         }
         __syncthreads();
 
@@ -423,9 +470,9 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 512 / NT : 1) step_fp64_kernel
         };
 
         // The head of a path once its inside is eliminated (N, M, S of the
-        // head): for the path from a soma its dV, else its factors and, if no
+        // head): for the path from a soma its y, else its factors and, if no
         // other path hangs off the same compartment, its elimination into the
-        // parent: d_p -= g f, r_p += g c (a = c = -g).
+        // parent: d_p -= gamma f, r_p += gamma c.
         auto eliminate_head = [&](const PathQ &P, double N, double M, double S) {
             const int h = P.head;
             const double inv = rcp_nr(N), c = div_nr(S, N, inv);
@@ -433,7 +480,7 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 512 / NT : 1) step_fp64_kernel
                 sdr[h] = make_double2(-1.0, c);
                 return;
             }
-            const double g = a.gimp * fabs(gax[h]);
+            const double g = -__ldg(sc + h);
             const double f = div_nr(g * M, N, inv);
             sdr[h] = make_double2(-f, c);
             if (P.nflag & kPathAlone) {
@@ -443,57 +490,64 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 512 / NT : 1) step_fp64_kernel
                 sdr[P.parent] = w;
             }
         };
-        auto rescale = [&](double &N, double &M, double &S) {
-            const double k = pow2_inverse(N);
-            N = mantissa(N);
-            M *= k;
-            S *= k;
+        // one step: compartment j (its coupling's exponent k) into the one
+        // above (its diagonal and rhs w)
+        auto step = [](double &N, double &M, double &S, int k, const double2 &w) {
+            const int d = exponent2(N);
+            const double Nn = __hiloint2double(__double2hiint(N) - d, __double2loint(N));
+            N = fma(w.x, Nn, -scale2(M, 2 * k - d));
+            S = fma(w.y, Nn, scale2(S, k - d));
+            M = Nn;
         };
-        // One path by one lane, leaf to head; the couplings of the next
-        // kSweepChunk compartments are loaded (from L2) while the current
-        // ones are eliminated.  Indices past the head are clamped, their
-        // results dropped.
+        // One path by one lane, leaf to head: whole chunks, the couplings of
+        // the next loaded (from L2) while the current is eliminated, then the
+        // rest (indices past the head clamped, their results dropped).
         auto eliminate_path = [&](int pi) {
             const PathQ P = paths[pi];
             const int h = P.head;
             int j = P.end - 1;
             const double2 v0 = sdr[j];
             double N = v0.x, M = 1.0, S = v0.y;
-            double gn[kSweepChunk];
+            int kn[kSweepChunk];
+            auto load = [&](int jj) {
 #pragma unroll
-            for (int k = 0; k < kSweepChunk; ++k) gn[k] = __ldg(gax + max(j - k, h));
-            for (; j > h; j -= kSweepChunk) {
-                const int cnt = j - h;
-                double g[kSweepChunk];
+                for (int z = 0; z < kSweepChunk; ++z) kn[z] = __ldg(kexp + max(jj - z, h));
+            };
+            load(j);
+            for (; j - h >= kSweepChunk; j -= kSweepChunk) {
+                int k[kSweepChunk];
                 double2 w[kSweepChunk];
 #pragma unroll
-                for (int k = 0; k < kSweepChunk; ++k) {
-                    g[k] = a.gimp * gn[k];
-                    w[k] = sdr[max(j - k - 1, h)];
+                for (int z = 0; z < kSweepChunk; ++z) {
+                    k[z] = kn[z];
+                    w[z] = sdr[j - z - 1];
                 }
+                load(j - kSweepChunk);
 #pragma unroll
-                for (int k = 0; k < kSweepChunk; ++k) gn[k] = __ldg(gax + max(j - kSweepChunk - k, h));
+                for (int z = 0; z < kSweepChunk; ++z) {
+                    step(N, M, S, k[z], w[z]);
+                    if (j - z - 1 > h) sdr[j - z - 1] = make_double2(N, S);
+                }
+            }
+            const int cnt = j - h;
+            double2 w[kSweepChunk - 1];
 #pragma unroll
-                for (int k = 0; k < kSweepChunk; ++k) {
-                    if (k < cnt) {
-                        const int i = j - k - 1;
-                        if ((i & (kRescale - 1)) == kRescale - 1) rescale(N, M, S);
-                        const double N1 = fma(w[k].x, N, -((g[k] * g[k]) * M));
-                        S = fma(w[k].y, N, g[k] * S);
-                        M = N;
-                        N = N1;
-                        if (i > h) sdr[i] = make_double2(N, S);
-                    }
+            for (int z = 0; z < kSweepChunk - 1; ++z) w[z] = sdr[max(j - z - 1, h)];
+#pragma unroll
+            for (int z = 0; z < kSweepChunk - 1; ++z) {
+                if (z < cnt) {
+                    step(N, M, S, kn[z], w[z]);
+                    if (z < cnt - 1) sdr[j - z - 1] = make_double2(N, S);
                 }
             }
             eliminate_head(P, N, M, S);
         };
         // The same by a whole warp.  The elimination step is linear in
         // (N, M, S): each lane composes the steps of its chunk (the images of
-        // the three unit vectors; S's own is p times itself), an inclusive
-        // warp scan combines the chunks, and each lane runs the steps of its
-        // chunk from the vector that the chunks before it leave.  Here the
-        // lanes divide themselves and store (-f, c).
+        // the first two unit vectors; S itself is multiplied by 2^(p >> 20)), an
+        // inclusive warp scan combines the chunks, and each lane runs the steps
+        // of its chunk from the vector that the chunks before it leave.  Here
+        // the lanes divide themselves and store (-f, c).
         auto eliminate_path_warp = [&](int pi) {
             const PathQ P = paths[pi];
             const int h = P.head, e = P.end;
@@ -501,41 +555,47 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 512 / NT : 1) step_fp64_kernel
             const int cs = (m + 31) >> 5;
             const int t0 = min(lane * cs, m), t1 = min(t0 + cs, m);
             const double2 leaf = sdr[e - 1];
-            double n1 = 1.0, m1 = 0.0, s1 = 0.0, n2 = 0.0, m2 = 1.0, s2 = 0.0, p = 1.0;
-            auto scale = [&]() {
-                const double k = pow2_inverse(n1);
-                n1 *= k; m1 *= k; s1 *= k; n2 *= k; m2 *= k; s2 *= k; p *= k;
-            };
+            double n1 = 1.0, m1 = 0.0, s1 = 0.0, n2 = 0.0, m2 = 1.0, s2 = 0.0;
+            int p = 0;
+            // (a product of thousands of factors leaves FP64's range, so the
+            // exponent stops at +-1000: nothing is left of what it multiplies)
+            auto clamp = [](int x) { return max(min(x, 1000 << 20), -(1000 << 20)); };
             double2 nb = make_double2(0.0, 0.0);
             for (int t = t0; t < t1; ++t) {
-                const int j = e - 1 - t;
-                const double g = a.gimp * __ldg(gax + j), gg = g * g;
+                const int j = e - 1 - t, k = __ldg(kexp + j);
                 const double2 w = sdr[j - 1];
-                const double a1 = fma(w.x, n1, -(gg * m1)), a2 = fma(w.x, n2, -(gg * m2));
-                s1 = fma(w.y, n1, g * s1);
-                s2 = fma(w.y, n2, g * s2);
+                const int d = exponent2(n1);
+                n1 = scale2(n1, -d);
+                n2 = scale2(n2, -d);
+                const double a1 = fma(w.x, n1, -scale2(m1, 2 * k - d)), a2 = fma(w.x, n2, -scale2(m2, 2 * k - d));
+                s1 = fma(w.y, n1, scale2(s1, k - d));
+                s2 = fma(w.y, n2, scale2(s2, k - d));
                 m1 = n1;
                 n1 = a1;
                 m2 = n2;
                 n2 = a2;
-                p *= g;
+                p = clamp(p + (k - d));
                 nb = w;
-                if (((t - t0) & (kRescale - 1)) == kRescale - 1) scale();
             }
             for (int off = 1; off < 32; off <<= 1) {
                 const unsigned F = 0xFFFFFFFFu;
                 const double bn1 = __shfl_up_sync(F, n1, off), bm1 = __shfl_up_sync(F, m1, off),
                              bs1 = __shfl_up_sync(F, s1, off), bn2 = __shfl_up_sync(F, n2, off),
-                             bm2 = __shfl_up_sync(F, m2, off), bs2 = __shfl_up_sync(F, s2, off),
-                             bp = __shfl_up_sync(F, p, off);
+                             bm2 = __shfl_up_sync(F, m2, off), bs2 = __shfl_up_sync(F, s2, off);
+                const int bp = __shfl_up_sync(F, p, off);
                 if (lane >= off) {  // this lane's steps act after the earlier lanes'
                     const double an1 = fma(n1, bn1, n2 * bm1), am1 = fma(m1, bn1, m2 * bm1),
-                                 as1 = fma(s1, bn1, fma(s2, bm1, p * bs1));
+                                 as1 = fma(s1, bn1, fma(s2, bm1, scale2(bs1, p)));
                     const double an2 = fma(n1, bn2, n2 * bm2), am2 = fma(m1, bn2, m2 * bm2),
-                                 as2 = fma(s1, bn2, fma(s2, bm2, p * bs2));
-                    n1 = an1; m1 = am1; s1 = as1; n2 = an2; m2 = am2; s2 = as2;
-                    p *= bp;
-                    scale();
+                                 as2 = fma(s1, bn2, fma(s2, bm2, scale2(bs2, p)));
+                    const int d = exponent2(an1);
+                    n1 = scale2(an1, -d);
+                    m1 = scale2(am1, -d);
+                    s1 = scale2(as1, -d);
+                    n2 = scale2(an2, -d);
+                    m2 = scale2(am2, -d);
+                    s2 = scale2(as2, -d);
+                    p = clamp(clamp(p + bp) - d);
                 }
             }
             // the vector at the chunk's first compartment: the earlier
@@ -545,24 +605,19 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 512 / NT : 1) step_fp64_kernel
                 const unsigned F = 0xFFFFFFFFu;
                 const double bn1 = __shfl_up_sync(F, n1, 1), bm1 = __shfl_up_sync(F, m1, 1),
                              bs1 = __shfl_up_sync(F, s1, 1), bn2 = __shfl_up_sync(F, n2, 1),
-                             bm2 = __shfl_up_sync(F, m2, 1), bs2 = __shfl_up_sync(F, s2, 1),
-                             bp = __shfl_up_sync(F, p, 1);
+                             bm2 = __shfl_up_sync(F, m2, 1), bs2 = __shfl_up_sync(F, s2, 1);
+                const int bp = __shfl_up_sync(F, p, 1);
                 N = lane ? fma(bn1, leaf.x, bn2) : leaf.x;
                 M = lane ? fma(bm1, leaf.x, bm2) : 1.0;
-                S = lane ? fma(bs1, leaf.x, fma(bp, leaf.y, bs2)) : leaf.y;
+                S = lane ? fma(bs1, leaf.x, bs2 + scale2(leaf.y, bp)) : leaf.y;
             }
             __syncwarp();  // every lane has read its chunk and the element after it
             for (int t = t0; t < t1; ++t) {
-                const int j = e - 1 - t;
-                const double g = a.gimp * __ldg(gax + j);
+                const int j = e - 1 - t, k = __ldg(kexp + j);
                 const double2 w = t + 1 < t1 ? sdr[j - 1] : nb;
-                if (((t - t0) & (kRescale - 1)) == 0) rescale(N, M, S);
                 const double inv = rcp_nr(N);
-                sdr[j] = make_double2(-div_nr(g * M, N, inv), div_nr(S, N, inv));
-                const double N1 = fma(w.x, N, -((g * g) * M));
-                S = fma(w.y, N, g * S);
-                M = N;
-                N = N1;
+                sdr[j] = make_double2(-scale2(div_nr(M, N, inv), k), div_nr(S, N, inv));
+                step(N, M, S, k, w);
             }
             // the head, from the lane whose chunk ends at it
             const int lastl = (m - 1) / cs;
@@ -583,7 +638,7 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 512 / NT : 1) step_fp64_kernel
                 double2 w = sdr[att];
                 for (int z = e; z < e1 && (int)(fold[z] >> 16) == att; ++z) {
                     const int h = paths[fold[z] & 0xFFFFu].head;
-                    const double g = a.gimp * fabs(gax[h]);
+                    const double g = -__ldg(sc + h);
                     const double2 q = sdr[h];
                     w.x = fma(g, q.x, w.x);
                     w.y = fma(g, q.y, w.y);
@@ -592,10 +647,10 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 512 / NT : 1) step_fp64_kernel
             }
         };
         // The factors of the compartments b0 .. b1-1 whose division is not
-        // done: f = g M / N, c = S / N with M the N of the compartment below
-        // (taken back to where the elimination rescaled it), 1 at a leaf --
-        // a compartment followed by a path's head, whose first member is
-        // negative, or by the end.
+        // done: f = gamma M / N, c = S / N with M the N of the compartment below
+        // (its power of two taken out, as the elimination does), 1 at a leaf --
+        // a compartment followed by one whose first member is negative, or by
+        // the end.
         auto divide = [&](int b0, int b1) {
             for (int i0 = b0; i0 < b1; i0 += TL) {
                 const int i = i0 + tl;
@@ -605,15 +660,14 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 512 / NT : 1) step_fp64_kernel
                     w = sdr[i];
                     if (i + 1 < b1) {
                         const double x = sdr[i + 1].x;
-                        if (!signbit(x)) M = (i & (kRescale - 1)) == kRescale - 1 ? mantissa(x) : x;
+                        if (!signbit(x)) M = mantissa(x);
                     }
                 }
                 if (signbit(w.x)) {
                     w.x = -w.x;
                 } else {
                     const double inv = rcp_nr(w.x);
-                    const double f = div_nr((a.gimp * __ldg(gax + i)) * M, w.x, inv);
-                    w = make_double2(f, div_nr(w.y, w.x, inv));
+                    w = make_double2(scale2(div_nr(M, w.x, inv), __ldg(kexp + i)), div_nr(w.y, w.x, inv));
                 }
                 team_sync();  // the compartment above has read this one's N
                 if (i < b1) sdr[i] = w;
@@ -641,17 +695,26 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 512 / NT : 1) step_fp64_kernel
             const int h = P.head;
             double x = substitute_head(P);
             if (P.parent >= 0) sdr[h].y = x;
-            for (int j = h + 1; j < P.end; j += kSweepChunk) {
-                const int cnt = P.end - j;
+            int j = h + 1;
+            for (; j + kSweepChunk <= P.end; j += kSweepChunk) {
                 double2 w[kSweepChunk];
 #pragma unroll
-                for (int k = 0; k < kSweepChunk; ++k) w[k] = sdr[min(j + k, P.end - 1)];
+                for (int k = 0; k < kSweepChunk; ++k) w[k] = sdr[j + k];
 #pragma unroll
                 for (int k = 0; k < kSweepChunk; ++k) {
-                    if (k < cnt) {
-                        x = fma(w[k].x, x, w[k].y);
-                        sdr[j + k].y = x;
-                    }
+                    x = fma(w[k].x, x, w[k].y);
+                    sdr[j + k].y = x;
+                }
+            }
+            const int cnt = P.end - j;
+            double2 w[kSweepChunk - 1];
+#pragma unroll
+            for (int k = 0; k < kSweepChunk - 1; ++k) w[k] = sdr[min(j + k, P.end - 1)];
+#pragma unroll
+            for (int k = 0; k < kSweepChunk - 1; ++k) {
+                if (k < cnt) {
+                    x = fma(w[k].x, x, w[k].y);
+                    sdr[j + k].y = x;
                 }
             }
         };
@@ -725,10 +788,10 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 512 / NT : 1) step_fp64_kernel
         gate_chunks(a, s_pc0, s_pn, &s_gchunk, lane);
         __syncthreads();
 
-        // C. V^{n+1} = V^n + dV and the threshold test of the detection
+        // C. V^{n+1} = V^n + dV, dV = s y, and the threshold test of the detection
         //    points other than somata.
         for (int i = tid; i < G.ncomp; i += NT) {
-            const double v0 = V[i], v = v0 + sdr[i].y;
+            const double v0 = V[i], v = fma(scale_of(i), sdr[i].y, v0);
             a.V[c0 + i] = v;
             if (a.pt_of && v0 < a.threshold && v >= a.threshold) {
                 const int p = a.pt_of[c0 + i];
@@ -800,6 +863,12 @@ int grid_for(int64_t n, int threads)
 int mmk_launch_init(const InitArgs &a, void *stream)
 {
     init_kernel<<<grid_for(a.C, 256), 256, 0, (cudaStream_t)stream>>>(a);
+    return (int)cudaGetLastError();
+}
+
+int mmk_launch_scale(const ScaleArgs64 &a, int n_groups, void *stream)
+{
+    scale_kernel<<<n_groups, 128, 0, (cudaStream_t)stream>>>(a);
     return (int)cudaGetLastError();
 }
 
