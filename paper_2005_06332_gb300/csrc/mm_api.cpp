@@ -18,7 +18,7 @@
 namespace {
 
 constexpr int kStepThreads = 256;
-constexpr int kDefaultGroupComps = 4096;
+constexpr int kDefaultGroupComps = 4096;    // with block_threads given: its budgets as ever
 constexpr int kDefaultGroupComps32 = 2048;  // FP32c: 24 B of shared memory per compartment
 constexpr int kMaxGroupComps = MM_FP64_MAX_NEURON_COMPS;
 constexpr int kMaxGroupComps32 = 1 << 30;
@@ -603,8 +603,13 @@ mm_status build(mm_net *net, const mm_morphologies *morph, const mm_channel_para
     li.cost = opt->schedule == MM_SCHED_COST ? opt->cost : nullptr;
     li.dt = opt->dt_ms;
     li.n_ext = opt->n_ext_sources;
+    // both launch options left open: the budget by the layout's estimate (it
+    // is fitted at the automatic block size, so a given one keeps the old budget)
     li.group_comps = opt->group_comps > 0 ? opt->group_comps
+                   : opt->block_threads <= 0 ? 0
                    : (opt->precision == MM_FP64 ? kDefaultGroupComps : kDefaultGroupComps32);
+    li.item_cost = opt->precision == MM_FP64 ? 300 : 700;
+    MM_CK(net, cudaDeviceGetAttribute(&li.sms, cudaDevAttrMultiProcessorCount, net->device));
     li.max_group_comps = opt->precision == MM_FP64 ? kMaxGroupComps : kMaxGroupComps32;
     // shared memory per item: FP64 the diagonal and rhs per compartment (16 B);
     // FP32c (active conductance, rhs) pair, the implicit coupling and the

@@ -14,7 +14,8 @@
 //      a leaf) is a contiguous range whose compartments each have the
 //      previous one as their parent;
 //   3. consecutive neurons are packed into work items of about
-//      `group_comps` compartments, each with its path tables (paths by
+//      `group_comps` compartments (given, or chosen by an estimate of the
+//      step's makespan), each with its path tables (paths by
 //      level, per-level fold lists of paths sharing a parent compartment),
 //      the schedule of the path-by-path leaves-to-root / root-to-leaves
 //      sweeps;
@@ -27,6 +28,7 @@
 #include <climits>
 #include <cstring>
 #include <cmath>
+#include <functional>
 #include <map>
 #include <numeric>
 #include <sstream>
@@ -209,6 +211,116 @@ std::vector<unsigned char> emit_path_blob(const PathBlob &b, bool wide)
         put16(o.mcnt_off, b.mcnt);
     }
     return blob;
+}
+
+// Shared memory of an automatically packed item, at most: its compartments
+// and paths, and per neuron its share of the bundle and level records (a
+// bundle of 12 B per 256 compartments or neuron, 4 B per path level).
+int64_t packed_need(const LayoutInput &in, int64_t comps, int64_t paths, int64_t neurons)
+{
+    return in.smem_per_comp * comps + (in.smem_per_path + 16) * paths + 16 * neurons + 256;
+}
+
+// Runs of whole neurons under a budget: the boundaries [items + 1].  paths
+// (per internal neuron; may be empty) closes an item before its shared
+// memory could pass giant_smem_limit, which would take it out of the regular
+// class.  In a supplied order, where neurons of all sizes follow one another,
+// items that all end short of the budget leave 9 % of it empty (10,000 neurons
+// of F-distributed sizes, 2,048): there, and in the precision with size
+// classes, an item may pass the budget by an eighth if it is then nearer to it
+// than without its last neuron (181 -> 177 us per step).  In size order
+// neighbours are alike and would all end on the same side.
+void pack_items(const LayoutInput &in, const Layout &L, const std::vector<int32_t> &paths, int64_t budget,
+                std::vector<int32_t> &gstart)
+{
+    const int64_t over = in.cost && in.giant_smem_limit > 0 ? budget / 8 : 0;
+    gstart.clear();
+    int64_t cur = 0, cp = 0;
+    int32_t cnt = 0;
+    for (int32_t k = 0; k < L.N; ++k) {
+        const int64_t n = L.noff[(size_t)k + 1] - L.noff[(size_t)k];
+        const int64_t p = paths.empty() ? 0 : paths[(size_t)k];
+        // at most kPathNeuron + 1 neurons per item, the range of a path's
+        // neuron index
+        bool close = k == 0 || cur + n - budget > std::min(over, budget - cur) || cnt > mmk::kPathNeuron;
+        if (!close && !paths.empty() && in.giant_smem_limit > 0)
+            close = packed_need(in, cur + n, cp + p, cnt + 1) > in.giant_smem_limit;
+        if (close) {
+            gstart.push_back(k);
+            cur = cp = 0;
+            cnt = 0;
+        }
+        cur += n;
+        cp += p;
+        ++cnt;
+    }
+    gstart.push_back(L.N);
+}
+
+// The budget whose items finish first by an estimate.  An item costs
+// item_cost + its compartments on an SM that runs two of them, 0.55 of that
+// alone on its SM; the queue hands the items out in order to two blocks per
+// SM (one where the largest needs over half an SM's shared memory), and an
+// item of the large class keeps an SM.  Small budgets fill the chip and even
+// out the last wave; large ones pay the fixed cost (the barriers and the
+// chain of path levels, nearly the same for 500 compartments as for 4,000)
+// less often.  item_cost: 700 in FP32c and 300 in FP64, fitted with the 0.55
+// to the step times of 12 networks (100 to 4,000 neurons, six size
+// distributions) at budgets of 256 to 4,096 on 152 SMs.  The choice is on
+// average 2 % (FP32c) and 1 % (FP64) behind each network's best budget; a
+// fixed 2,048 (FP32c) or 4,096 (FP64) was 9 % and 24 % behind.  Per step, us,
+// fixed -> chosen: 300 neurons of 450 compartments FP32c 29.0 -> 25.7, FP64
+// 174 -> 73; 2,000 of 1,500 FP32c 207 -> 162; 10,000 of 50 to 5,000 FP32c
+// 608 -> 555.  The estimate is not good for more than 3 %: within that the
+// first of the list is taken.
+int64_t choose_budget(const LayoutInput &in, const Layout &L, const std::vector<int32_t> &paths)
+{
+    static const int32_t kBudgets[] = {2048, 1536, 3072, 1024, 4096, 768, 512, 384, 256};
+    const int64_t half_sm = 110 * 1024;
+    const double alone = 0.55;
+    std::vector<double> est;
+    std::vector<int32_t> gstart;
+    std::vector<int64_t> item, heap;
+    for (const int32_t budget : kBudgets) {
+        pack_items(in, L, paths, budget, gstart);
+        item.clear();
+        int64_t large = 0, widest = 0;
+        for (size_t g = 0; g + 1 < gstart.size(); ++g) {
+            const int32_t k0 = gstart[g], k1 = gstart[g + 1];
+            const int64_t n = L.noff[(size_t)k1] - L.noff[(size_t)k0];
+            int64_t np = 0;
+            for (int32_t k = k0; k < k1; ++k) np += paths[(size_t)k];
+            const int64_t need = packed_need(in, n, np, k1 - k0);
+            if (in.giant_smem_limit > 0 && need > in.giant_smem_limit) {
+                ++large;
+            } else {
+                widest = std::max(widest, need);
+                item.push_back(in.item_cost + n);
+            }
+        }
+        const size_t sms = (size_t)std::max<int64_t>(std::max<int64_t>(in.sms - large, in.sms / 3), 1);
+        const size_t slots = widest > half_sm ? sms : 2 * sms;
+        double end = 0.0;
+        if (item.size() <= slots) {  // all at once: the i-th shares its SM with the (sms + i)-th
+            for (size_t i = 0; i < std::min(sms, item.size()); ++i) {
+                const double other = sms + i < item.size() ? (double)item[sms + i] : 0.0;
+                end = std::max(end, alone * (double)item[i] + (1.0 - alone) * other);
+            }
+        } else {
+            heap.assign(slots, 0);
+            for (const int64_t t : item) {  // the next item goes to the block that is free first
+                std::pop_heap(heap.begin(), heap.end(), std::greater<int64_t>());
+                heap.back() += t;
+                end = std::max(end, (double)heap.back());
+                std::push_heap(heap.begin(), heap.end(), std::greater<int64_t>());
+            }
+        }
+        est.push_back(end);
+    }
+    const double best = *std::min_element(est.begin(), est.end());
+    size_t i = 0;
+    while (est[i] > 1.03 * best) ++i;
+    return kBudgets[i];
 }
 
 }  // namespace
@@ -401,23 +513,22 @@ std::string build_layout(const LayoutInput &in, Layout &out, bool *invalid)
         if (in.stim) L.stim[(size_t)k] = in.stim[u];
     }
 
-    // 3a. group boundaries (at most kPathNeuron + 1 neurons per item, the
-    // range of a path's neuron index)
+    // 3a. group boundaries
     std::vector<int32_t> gstart;
-    {
-        int64_t cur = 0;
-        int32_t cnt = 0;
+    if (in.group_comps > 0 && !in.cost) {
+        pack_items(in, L, {}, in.group_comps, gstart);
+    } else {
+        std::vector<int32_t> paths((size_t)N, 0);  // a path ends at each leaf
+        std::vector<char> inner;
         for (int32_t k = 0; k < N; ++k) {
-            const int64_t n = L.noff[(size_t)k + 1] - L.noff[(size_t)k];
-            if (k == 0 || cur + n > in.group_comps || cnt > mmk::kPathNeuron) {
-                gstart.push_back(k);
-                cur = 0;
-                cnt = 0;
-            }
-            cur += n;
-            ++cnt;
+            const int32_t u = L.order[(size_t)k];
+            const int32_t *par = in.parent + in.comp_offset[u];
+            const int32_t n = (int32_t)size_of(u);
+            inner.assign((size_t)n, 0);
+            for (int32_t i = 1; i < n; ++i) inner[(size_t)par[i]] = 1;
+            paths[(size_t)k] = n - (int32_t)std::count(inner.begin(), inner.end(), (char)1);
         }
-        gstart.push_back(N);
+        pack_items(in, L, paths, in.group_comps > 0 ? in.group_comps : choose_budget(in, L, paths), gstart);
     }
     const int32_t G = (int32_t)gstart.size() - 1;
     L.groups.clear();

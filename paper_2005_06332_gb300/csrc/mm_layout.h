@@ -27,7 +27,10 @@ struct LayoutInput {
     const double *stim;           // may be NULL
     const float *cost;            // may be NULL (size order)
     double dt;
-    int32_t group_comps;          // compartment budget of a work item
+    int32_t group_comps;          // compartment budget of a work item; 0: the best of a set by the
+                                  // estimate of choose_budget, which takes the next two
+    int32_t sms;                  // SMs of the device
+    int32_t item_cost;            // fixed cost of an item, in compartments
     int32_t max_group_comps;      // largest neuron accepted
     // shared-memory model of a work item, bytes = meta + smem_per_comp * comps
     // + smem_per_path * paths; items above giant_smem_limit go to the large
