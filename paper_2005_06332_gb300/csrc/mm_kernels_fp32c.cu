@@ -492,13 +492,15 @@ __global__ void __launch_bounds__(NT, 1024 / NT) step_fp32c_kernel(StepArgs32 a)
         if (T == 2 && nwarp / 2 > 15) T = 4;
         const int team = (tid >> 5) / T, nteam = nwarp / T;
         // lane within the team; the team's first warp, which takes the longest
-        // paths, rotates over the SM's four schedulers from team to team (and
-        // between the two blocks that share an SM): all on one scheduler, they
-        // took each other's issue slots.  With this, phase C's loads four
-        // together and phase S's overlapped, per step: 64 neurons of 255
-        // compartments 30.2 -> 24.3 us, 10,000 of mean 300 206 -> 193 us, 10,000
-        // of 50 to 5,000 625 -> 608 us.
-        const int rot = team + (blockIdx.x >= gridDim.x / 2 ? 2 : 0);
+        // paths, sits on another of the SM's four schedulers from team to team
+        // (teams of two start on two of them, so those rotate every other
+        // team) and between the two blocks that share an SM: where several
+        // shared a scheduler, they took each other's issue slots.  Per step,
+        // teams of two on two schedulers -> on four: 10,000 neurons of mean 300
+        // 183 -> 169 us, 10,000 of 50 to 5,000 555 -> 549 us, 3,000 lognormal
+        // 284 -> 275 us; before that, all on one: 10,000 of mean 300 206 us.
+        const int half = blockIdx.x >= gridDim.x / 2 ? 1 : 0;
+        const int rot = T == 2 ? (team >> 1) + half : team + 2 * half;
         const int tl = ((((tid >> 5) - rot) & (T - 1)) << 5) + (tid & 31);
         const int TL = T * 32;
         auto team_sync = [&]() {
