@@ -261,7 +261,8 @@ void pack_items(const LayoutInput &in, const Layout &L, const std::vector<int32_
 // item_cost + its compartments on an SM that runs two of them, 0.55 of that
 // alone on its SM; the queue hands the items out in order to two blocks per
 // SM (one where the largest needs over half an SM's shared memory), and an
-// item of the large class keeps an SM.  Small budgets fill the chip and even
+// item beyond the regular class keeps an SM and ends no sooner than alone: a
+// small network with giants ends with them whatever the budget.  Small budgets fill the chip and even
 // out the last wave; large ones pay the fixed cost (the barriers and the
 // chain of path levels, nearly the same for 500 compartments as for 4,000)
 // less often.  item_cost: 700 in FP32c and 300 in FP64, fitted with the 0.55
@@ -284,7 +285,7 @@ int64_t choose_budget(const LayoutInput &in, const Layout &L, const std::vector<
     for (const int32_t budget : kBudgets) {
         pack_items(in, L, paths, budget, gstart);
         item.clear();
-        int64_t large = 0, widest = 0;
+        int64_t large = 0, widest = 0, longest = 0;
         for (size_t g = 0; g + 1 < gstart.size(); ++g) {
             const int32_t k0 = gstart[g], k1 = gstart[g + 1];
             const int64_t n = L.noff[(size_t)k1] - L.noff[(size_t)k0];
@@ -293,6 +294,7 @@ int64_t choose_budget(const LayoutInput &in, const Layout &L, const std::vector<
             const int64_t need = packed_need(in, n, np, k1 - k0);
             if (in.giant_smem_limit > 0 && need > in.giant_smem_limit) {
                 ++large;
+                longest = std::max(longest, in.item_cost + n);
             } else {
                 widest = std::max(widest, need);
                 item.push_back(in.item_cost + n);
@@ -300,7 +302,7 @@ int64_t choose_budget(const LayoutInput &in, const Layout &L, const std::vector<
         }
         const size_t sms = (size_t)std::max<int64_t>(std::max<int64_t>(in.sms - large, in.sms / 3), 1);
         const size_t slots = widest > half_sm ? sms : 2 * sms;
-        double end = 0.0;
+        double end = alone * (double)longest;
         if (item.size() <= slots) {  // all at once: the i-th shares its SM with the (sms + i)-th
             for (size_t i = 0; i < std::min(sms, item.size()); ++i) {
                 const double other = sms + i < item.size() ? (double)item[sms + i] : 0.0;
