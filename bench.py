@@ -63,9 +63,9 @@ PROFILED = {
     # ncu counters of one regular-class launch of the step kernel (multi10k,
     # 512 threads, 4096-compartment items, a step inside the timed window)
     ("multi10k", "fp32c", "step", "soma"): {
-        "sha256": "f442347e16f327b6adfd673c0fa934f5e2714eac09b925479dac6083f08d09c0",
-        "dram_bytes": 495057920 + 111741184,
-        "warp_instructions": 285126986,
+        "sha256": "132602ec0c1958b1e29253aa36b97739ae9a1e6e2dd9edc34f60a967316c841c",
+        "dram_bytes": 494440192 + 111394560,
+        "warp_instructions": 283394194,
         "comps": 9484756,
     },
 }

@@ -456,8 +456,8 @@ typedef struct {
     int32_t blocks_per_sm;     /* resident blocks per SM at this shared-memory size */
     int32_t smem_bytes;        /* dynamic shared memory per block */
     int32_t max_item_comps;    /* compartments of the largest work item */
-    int32_t max_item_segments; /* unbranched segments of the largest work item */
-    int32_t max_item_waves;    /* height waves of the deepest work item */
+    int32_t max_item_segments; /* paths of the work item that has most */
+    int32_t max_item_waves;    /* path levels of the deepest work item */
     int32_t giant_items;       /* FP32c work items solved from global memory (too big for shared memory) */
     /* FP32c work items above the regular shared-memory budget that still fit
      * one block's shared memory: solved by a second launch of the per-step
