@@ -28,6 +28,7 @@
 
 #include <cmath>
 #include <cstring>
+#include <limits>
 
 #ifdef __CUDACC__
 #define MMG_HD __host__ __device__ __forceinline__
@@ -189,7 +190,7 @@ inline void build_table64(double dt, void *tab)
             const bool e_form = y[g][K / 2] >= -0.6931471805599453L;  // E <= 1/2
             for (int k = 0; k < K; ++k) {
                 const double yh = (double)y[g][k], dy = (double)(y[g][k] - yh);
-                f[2 * g + 1][k] = e_form ? -(std::expm1(yh) + (LD)(std::exp(yh) * dy)) : -(LD)std::exp(yh) * (1.0L + dy);
+                f[2 * g + 1][k] = e_form ? -(std::expm1(yh) + (LD)(std::exp(yh) * dy)) : -fabsl(std::exp(yh) * (1.0L + dy));
             }
         }
         for (int fn = 0; fn < kTab64Funcs; ++fn) {
@@ -200,8 +201,19 @@ inline void build_table64(double dt, void *tab)
                 for (int k = 0; k < K; ++k)
                     if (k != K / 2) c[d] += M[d][k] * (f[fn][k] - f[fn][K / 2]);
             }
-            const Quad64 p{(double)f[fn][K / 2], (double)c[1]}, q{(double)c[2], (double)c[3]};
-            const Quad32 s{(float)c[4], (float)c[5], (float)c[6], (float)(f[fn][K / 2] - p.a)};
+            Quad64 p{(double)f[fn][K / 2], (double)c[1]}, q{(double)c[2], (double)c[3]};
+            Quad32 s{(float)c[4], (float)c[5], (float)c[6], (float)(f[fn][K / 2] - p.a)};
+            // F below 2^-100 (a step far below the time constant, or far above
+            // it): the tail leaves FP32's range, and widen's 2^-127 for a zero
+            // could turn F's sign, which step64 goes by.  F is then its value at
+            // the centre (within 2^-98 of it), all other terms zero with F's sign,
+            // so that widen's 2^-127 u^4 has it too
+            if (fn % 2 == 1 && std::fabs(p.a) < 0x1p-100) {
+                const float z = std::copysign(0.0f, (float)p.a);
+                p = Quad64{p.a == 0.0 ? std::copysign(std::numeric_limits<double>::min(), p.a) : p.a, (double)z};
+                q = Quad64{(double)z, (double)z};
+                s = Quad32{z, z, z, z};
+            }
             const void *src[3] = {&p, &q, &s};
             for (int x = 0; x < 3; ++x)
                 std::memcpy(base + 16 * ((size_t)(3 * fn + x) * kTab64Intervals + i), src[x], 16);
