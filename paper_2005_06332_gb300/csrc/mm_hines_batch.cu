@@ -1,9 +1,9 @@
 // mm_hines_batch.cu -- a standalone batched Hines solve on the device.
 //
 // Algorithm 1 (Sec. 2) for many independent trees at once, any numbering with
-// parent[j] < j.  Inputs are const; the eliminated diagonal lives in a scratch
-// array and the rhs is worked on in the output array.  Device pointers in and
-// out.
+// parent[j] < j.  Inputs are const; the diagonal and what it becomes (see
+// solve_group) live in a scratch array, the rhs is worked on in the output
+// array.  Device pointers in and out.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -14,10 +14,12 @@
 
 // Scratch of mm_hines_solve_noalloc: a fixed device array in this library
 // image, so that the call never allocates.  The first 256 bytes hold the
-// status word, the rest the eliminated diagonal (MM_NOALLOC_MAX_COMPS doubles,
-// 8 MiB).  Every GPU that loads the library holds it until the process ends.
+// status words, the next 8 KiB the lists of left groups, the rest the working
+// values of the diagonal (MM_NOALLOC_MAX_COMPS doubles, 8 MiB).  Every GPU that
+// loads the library holds it until the process ends.
 #define MM_NOALLOC_MAX_COMPS (1 << 20)
-static __device__ __align__(256) double g_noalloc_scratch[32 + MM_NOALLOC_MAX_COMPS];
+#define MM_NOALLOC_LEFT 1024
+static __device__ __align__(256) double g_noalloc_scratch[32 + MM_NOALLOC_LEFT + MM_NOALLOC_MAX_COMPS];
 
 namespace {
 
@@ -28,8 +30,10 @@ struct Batch {
     const int32_t *parent;
     const double *a, *b, *c, *rhs;
     double *x, *work;
-    int *status;             // bit 0: a tree violates the parent rule or its entries lie outside n_comp; bit 1: see
-                             // hines_rest_kernel
+    int *status;             // [0] nonzero: a tree violates the parent rule or its entries lie outside n_comp;
+                             // [1], [2]: groups of trees left to hines_left_kernel and to hines_rest_kernel
+    int32_t *left;           // these groups, left_cap of the first kind, then left_cap of the second
+    int32_t left_cap;
     int32_t trees_per_block; // 1 .. kMaxTrees
 };
 
@@ -74,7 +78,13 @@ __device__ void solve_serial(const Batch &B, int32_t t)
 
 constexpr int kMaxTrees = 128;     // trees of one block
 constexpr int kBlockComps = 2048;  // compartments aimed at per block
-constexpr long long kLeft = 0x7FF8A5C3966D1E27LL;  // in the scratch, at the first entry of a block that was left
+constexpr int kSmallChains = 1024, kLargeChains = 8192;  // chains that a block's tables hold
+// A group that is left has more than kSmallChains entries, and the groups'
+// entries lie side by side: at most this many are left.  (Only offsets that run
+// backwards somewhere, which make the call fail, can overlap and leave more;
+// those blocks solve their trees serially at once.)
+constexpr int32_t left_cap_of(int64_t n_comp) { return (int32_t)(n_comp / (kSmallChains + 1)) + 1; }
+static_assert(left_cap_of(MM_NOALLOC_MAX_COMPS) <= MM_NOALLOC_LEFT, "lists of the fixed scratch");
 constexpr size_t smem_of(int chains) { return (size_t)chains * 20 + 16; }
 
 // One entry of a chain's elimination: N / M is its eliminated diagonal, S / M
@@ -117,7 +127,8 @@ struct Front {
 // and more blocks 0.94 to 1.14 ms, groups of 4,096 entries 1.34 ms; eliminating
 // the diagonal alone first (with a c stored: 2 + 2 + 2 instructions in the
 // sweeps, but two passes more) 1.10 ms.  CHAINS: the chains that a block's tables hold.  FIRST:
-// every group of trees, else those that a smaller table left.
+// every group of trees, else those that a smaller table left.  A group is on
+// one list at most, so that its trees are solved once, also where x is rhs.
 template <int CHAINS, int NT, bool FIRST>
 __device__ __forceinline__ void solve_group(const Batch &B, int group)
 {
@@ -140,10 +151,6 @@ __device__ __forceinline__ void solve_group(const Batch &B, int group)
     if (tid <= nt) s_off[tid] = B.off[t0 + tid];
     if (tid == 0 && nt == NT) s_off[nt] = B.off[t1];
     __syncthreads();
-    if (!FIRST) {
-        const int64_t first = s_off[0];
-        if (first < 0 || first >= B.n_comp || __double_as_longlong(B.work[first]) != kLeft) return;
-    }
     if (tid < nt && (s_off[tid] < 0 || s_off[tid + 1] < s_off[tid] || s_off[tid + 1] > B.n_comp)) s_bad = 1;
     __syncthreads();
     const int64_t base = s_off[0];
@@ -207,9 +214,12 @@ __device__ __forceinline__ void solve_group(const Batch &B, int group)
     }
     if (stop == 2) {  // left to a larger table or to hines_rest_kernel
         if (tid == 0) {
-            work[0] = __longlong_as_double(kLeft);
-            atomicOr(B.status, 2);
+            const int q = atomicAdd(B.status + (FIRST ? 1 : 2), 1);
+            s_go = q < B.left_cap;
+            if (s_go) B.left[(FIRST ? 0 : B.left_cap) + q] = group;
         }
+        __syncthreads();
+        if (!s_go && tid < nt) solve_serial(B, t0 + tid);
         return;
     }
     const int K = s_K;
@@ -459,58 +469,56 @@ __global__ void __launch_bounds__(NT, BLOCKS) hines_batch_kernel(Batch B)
     solve_group<CHAINS, NT, true>(B, blockIdx.x);
 }
 
-// The blocks of trees that hines_batch_kernel left, with a larger table.
+// The groups of trees that hines_batch_kernel left, with a larger table.
 template <int CHAINS, int NT>
-__global__ void __launch_bounds__(NT, 1) hines_left_kernel(Batch B, int groups)
+__global__ void __launch_bounds__(NT, 1) hines_left_kernel(Batch B)
 {
-    if (!(*B.status & 2)) return;
-    for (int g = blockIdx.x; g < groups; g += gridDim.x) {
-        solve_group<CHAINS, NT, false>(B, g);
+    const int left = min(B.status[1], B.left_cap);
+    for (int q = blockIdx.x; q < left; q += gridDim.x) {
+        solve_group<CHAINS, NT, false>(B, B.left[q]);
         __syncthreads();
     }
 }
 
-// The trees of blocks with more chains than the largest table holds (mostly one
-// large tree to a block), a thread for each block, so that many such trees run
+// The trees of groups with more chains than the largest table holds (mostly one
+// large tree to a group), a thread for each group, so that many such trees run
 // side by side.
 __global__ void __launch_bounds__(128) hines_rest_kernel(Batch B)
 {
-    if (!(*B.status & 2)) return;
-    const int64_t groups = ((int64_t)B.n_trees + B.trees_per_block - 1) / B.trees_per_block;
-    for (int64_t g = blockIdx.x * 128LL + threadIdx.x; g < groups; g += gridDim.x * 128LL) {
-        const int64_t t0 = g * B.trees_per_block, t1 = min(t0 + B.trees_per_block, (int64_t)B.n_trees);
-        const int64_t first = B.off[t0];
-        if (first < 0 || first >= B.n_comp || __double_as_longlong(B.work[first]) != kLeft) continue;
+    const int left = min(B.status[2], B.left_cap);
+    for (int q = blockIdx.x * 128 + threadIdx.x; q < left; q += gridDim.x * 128) {
+        const int64_t t0 = (int64_t)B.left[B.left_cap + q] * B.trees_per_block;
+        const int64_t t1 = min(t0 + B.trees_per_block, (int64_t)B.n_trees);
         for (int64_t t = t0; t < t1; ++t) solve_serial(B, (int32_t)t);
     }
 }
 
 mm_status run_batch(Batch B, cudaStream_t s)
 {
-    if (cudaMemsetAsync(B.status, 0, sizeof(int), s) != cudaSuccess) return MM_ECUDA;
+    if (cudaMemsetAsync(B.status, 0, 3 * sizeof(int), s) != cudaSuccess) return MM_ECUDA;
     if (B.n_trees > 0 && B.n_comp > 0) {
         // trees per block: about kBlockComps entries, fewer where the batch
         // would not fill the chip's slots otherwise, at least one tree.  The
-        // tables of 1,024 chains leave room for six blocks per SM; blocks with
+        // tables of 1,024 chains leave room for six blocks per SM; groups with
         // more chains are taken up by a second launch with one block per SM, and
         // the rest by a third (both end at once when nothing was left).
-        constexpr auto small = hines_batch_kernel<1024, 128, 6>;
-        constexpr auto large = hines_left_kernel<8192, 256>;
+        constexpr auto small = hines_batch_kernel<kSmallChains, 128, 6>;
+        constexpr auto large = hines_left_kernel<kLargeChains, 256>;
         // 912: six blocks on each of 152 SMs
         const int64_t mean = std::max<int64_t>(1, B.n_comp / B.n_trees);
         B.trees_per_block = (int32_t)std::min<int64_t>(kMaxTrees, std::max<int64_t>(1, std::min<int64_t>(kBlockComps, B.n_comp / 912) / mean));
         const int64_t blocks = ((int64_t)B.n_trees + B.trees_per_block - 1) / B.trees_per_block;
-        if (cudaFuncSetAttribute(large, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of(8192)) != cudaSuccess)
+        if (cudaFuncSetAttribute(large, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of(kLargeChains)) != cudaSuccess)
             return MM_ECUDA;
-        small<<<(unsigned)blocks, 128, smem_of(1024), s>>>(B);
-        large<<<(unsigned)std::min<int64_t>(blocks, 152), 256, smem_of(8192), s>>>(B, (int)blocks);
+        small<<<(unsigned)blocks, 128, smem_of(kSmallChains), s>>>(B);
+        large<<<(unsigned)std::min<int64_t>(blocks, 152), 256, smem_of(kLargeChains), s>>>(B);
         hines_rest_kernel<<<(unsigned)std::min<int64_t>((blocks + 127) / 128, 152 * 16), 128, 0, s>>>(B);
         if (cudaGetLastError() != cudaSuccess) return MM_ECUDA;
     }
     int h = 0;
     if (cudaMemcpyAsync(&h, B.status, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess) return MM_ECUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess) return MM_ECUDA;
-    return (h & 1) ? MM_EINVAL : MM_OK;
+    return h ? MM_EINVAL : MM_OK;
 }
 
 bool args_ok(int32_t n_trees, int64_t n_comp, const int64_t *off, const int32_t *parent, const double *a,
@@ -530,16 +538,19 @@ extern "C" mm_status mm_hines_solve(int32_t n_trees, int64_t n_comp, const int64
 {
     if (!args_ok(n_trees, n_comp, tree_offset, parent, a, b, c, rhs, x)) return MM_EINVAL;
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    // scratch: the eliminated diagonal, then the status word
-    const size_t bytes = (size_t)(n_comp > 0 ? n_comp : 1) * sizeof(double) + 256;
+    // scratch: the working values of the diagonal, the status words, the lists
+    const size_t values = (size_t)(n_comp > 0 ? n_comp : 1) * sizeof(double);
+    const int32_t cap = left_cap_of(n_comp);
+    const size_t bytes = values + 256 + 2 * (size_t)cap * sizeof(int32_t);
     void *scratch = nullptr;
     if (cudaMalloc(&scratch, bytes) != cudaSuccess) {
         cudaGetLastError();
         return MM_ENOMEM;
     }
     double *work = (double *)scratch;
-    int *status = (int *)((char *)scratch + bytes - 256);
-    const mm_status st = run_batch({n_trees, n_comp, tree_offset, parent, a, b, c, rhs, x, work, status, 1}, s);
+    int *status = (int *)((char *)scratch + values);
+    const mm_status st =
+        run_batch({n_trees, n_comp, tree_offset, parent, a, b, c, rhs, x, work, status, status + 64, cap, 1}, s);
     cudaFree(scratch);
     return st;
 }
@@ -559,7 +570,9 @@ extern "C" mm_status mm_hines_solve_noalloc(int32_t n_trees, int64_t n_comp, con
         cudaGetLastError();
         return MM_ECUDA;
     }
-    int *status = (int *)base;                       // cleared by run_batch before the kernel
-    double *work = (double *)((char *)base + 256);   // fully written before it is read
-    return run_batch({n_trees, n_comp, tree_offset, parent, a, b, c, rhs, x, work, status, 1}, (cudaStream_t)cuda_stream);
+    int *status = (int *)base;                                     // cleared by run_batch before the kernels
+    double *work = (double *)base + 32 + MM_NOALLOC_LEFT;          // written before it is read, as the lists are
+    return run_batch({n_trees, n_comp, tree_offset, parent, a, b, c, rhs, x, work, status, status + 64,
+                      left_cap_of(n_comp), 1},
+                     (cudaStream_t)cuda_stream);
 }

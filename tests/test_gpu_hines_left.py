@@ -1,0 +1,37 @@
+"""The batched Hines solve where a block's chain tables overflow before the
+block has seen an invalid tree of its own: the invalid tree is rejected, and
+the block's other trees are solved once -- also where the output is the rhs, so
+that a second solve would take the solution as its rhs -- through both entry
+points and on two calls in a row."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2005_06332_gb300 import mm, netgen
+
+pytestmark = pytest.mark.gpu
+
+
+def test_trees_beside_an_invalid_one_are_solved_once():
+    import torch
+    star = np.concatenate([[-1], np.zeros(1598, np.int64), [-7]])  # 1,598 chains, then an entry without a parent
+    rng = np.random.default_rng(2)
+    # blocks of two trees (mean size 500 of a million entries): an invalid and a valid one
+    trees = [t for k in range(300) for t in (star, netgen.random_tree(rng, 100, 0.2))]
+    trees += [netgen.random_tree(rng, 350, 0.1) for _ in range(1400)]
+    off = np.concatenate([[0], np.cumsum([len(t) for t in trees])]).astype(np.int64)
+    n = int(off[-1])
+    par = np.concatenate(trees).astype(np.int32)
+    a, c = -rng.uniform(0.1, 1.0, n), -rng.uniform(0.1, 1.0, n)
+    b, r = rng.uniform(30.0, 40.0, n), rng.normal(size=n)
+    dev = [torch.as_tensor(v, device="cuda") for v in (off, par, a, b, c)]
+    L = mm.load()
+    good = [k for k in range(len(trees)) if len(trees[k]) != 1600]
+    ref = {k: oracle.hines_solve(*(v[off[k]:off[k + 1]] for v in (a, b, c, r)), trees[k].astype(np.int32)) for k in good}
+    for fn in (L.mm_hines_solve, L.mm_hines_solve_noalloc, L.mm_hines_solve_noalloc):
+        x = torch.as_tensor(r, device="cuda").clone()
+        assert fn(len(trees), n, *(v.data_ptr() for v in dev), x.data_ptr(), x.data_ptr(),
+                  torch.cuda.current_stream().cuda_stream) == mm.MM_EINVAL
+        got = x.cpu().numpy()
+        for k in good:
+            np.testing.assert_allclose(got[off[k]:off[k + 1]], ref[k], rtol=1e-12, atol=1e-14)
