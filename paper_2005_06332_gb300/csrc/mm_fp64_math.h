@@ -11,15 +11,23 @@ namespace mmk {
 
 // 1/x from the approximate reciprocal (about 20 bits) by one step of third
 // order, r (1 + e + e^2) with e = 1 - x r: FP64 rounding in three instructions.
-__device__ __forceinline__ double rcp_nr(double x)
+// For normal x below 2^1022 (the approximation is zero or infinite beyond, and
+// e NaN for an infinite x or reciprocal).
+__device__ __forceinline__ double rcp_approx(double x)
 {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    const double e = fma(-x, r, 1.0);
+    return r;
+}
+
+__device__ __forceinline__ double rcp_nr(double x)
+{
+    const double r = rcp_approx(x), e = fma(-x, r, 1.0);
     return fma(r, fma(e, e, e), r);
 }
 
-// a / x given r = rcp_nr(x): one residual correction
+// a / x given r = rcp_nr(x): one residual correction.  NaN where a or the
+// quotient is infinite, and short of bits where a is below 2^-960.
 __device__ __forceinline__ double div_nr(double a, double x, double r)
 {
     const double q = a * r;
