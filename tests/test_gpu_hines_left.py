@@ -35,3 +35,20 @@ def test_trees_beside_an_invalid_one_are_solved_once():
         got = x.cpu().numpy()
         for k in good:
             np.testing.assert_allclose(got[off[k]:off[k + 1]], ref[k], rtol=1e-12, atol=1e-14)
+
+
+def test_large_trees_of_one_block_match_algorithm_1():
+    """Large bushy trees before many tiny ones: several fall into one block, whose tables hold the chains of none."""
+    import torch
+    rng = np.random.default_rng(6)
+    trees = [netgen.random_tree(rng, 9000 + 500 * k, 0.6) for k in range(7)]
+    trees += [netgen.random_tree(rng, 1 + k % 60, 0.2) for k in range(20000)]
+    off = np.concatenate([[0], np.cumsum([len(t) for t in trees])]).astype(np.int64)
+    n = int(off[-1])
+    a, c = -rng.uniform(0.1, 1.0, n), -rng.uniform(0.1, 1.0, n)
+    kids = np.concatenate([np.bincount(t[1:], minlength=len(t)) for t in trees])
+    b, r = rng.uniform(1.5, 3.0, n) + 1.5 * kids, rng.normal(size=n)
+    x = mm.hines_solve(*(torch.as_tensor(v, device="cuda")
+                         for v in (off, np.concatenate(trees).astype(np.int32), a, b, c, r))).cpu().numpy()
+    ref = [oracle.hines_solve(*(v[s:e] for v in (a, b, c, r)), t.astype(np.int32)) for s, e, t in zip(off[:-1], off[1:], trees)]
+    np.testing.assert_allclose(x, np.concatenate(ref), rtol=1e-12, atol=1e-14)
