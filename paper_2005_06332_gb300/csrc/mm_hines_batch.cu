@@ -127,6 +127,7 @@ __device__ __forceinline__ double divide(double a, double x, double r)
 
 constexpr int kMaxTrees = 128;     // trees of one block
 constexpr int kBlockComps = 2048;  // compartments aimed at per block
+constexpr int kTiny = 8;           // trees of a block up to this size: a thread each at once (see solve_group)
 constexpr int kSmallChains = 1024, kLargeChains = 8192;  // chains that a block's tables hold
 // A group that is left has more than kSmallChains entries, and the groups'
 // entries lie side by side: at most this many are left.  (Only offsets that run
@@ -178,6 +179,9 @@ struct Front {
 // sweeps, but two passes more) 1.10 ms.  CHAINS: the chains that a block's tables hold.  FIRST:
 // every group of trees, else those that a smaller table left.  A group is on
 // one list at most, so that its trees are solved once, also where x is rhs.
+// Where no tree has more than kTiny entries a thread solves each at once: what
+// comes before the sweeps takes longer (a million trees of two entries 0.41 ->
+// 0.30 ms, of five 0.61 -> 0.56; of twelve it is the other way, 1.13 -> 1.24).
 template <int CHAINS, int NT, bool FIRST>
 __device__ __forceinline__ void solve_group(const Batch &B, int group)
 {
@@ -190,21 +194,24 @@ __device__ __forceinline__ void solve_group(const Batch &B, int group)
     int *up = head + CHAINS + 1;                           // chain above (pointer jumping)
     int *lev = up + CHAINS;                                // level; then where each level begins in key
     __shared__ int64_t s_off[kMaxTrees + 1];
-    __shared__ int s_warp[kLook * NT / 32], s_bad, s_K, s_go;
+    __shared__ int s_warp[kLook * NT / 32], s_bad, s_K, s_go, s_long;
     static_assert(kMaxTrees < NT + 1 && (CHAINS & (CHAINS - 1)) == 0 && CHAINS <= 8192, "table sizes");
     constexpr unsigned long long kChain = 0x1FFF;  // a key: level << 43 | entry << 13 | chain
     const int tid = threadIdx.x, lane = tid & 31;
     const int32_t t0 = group * B.trees_per_block, t1 = min(t0 + B.trees_per_block, B.n_trees);
     const int nt = t1 - t0;
-    if (tid == 0) s_bad = s_K = 0;
+    if (tid == 0) s_bad = s_K = s_long = 0;
     if (tid <= nt) s_off[tid] = B.off[t0 + tid];
     if (tid == 0 && nt == NT) s_off[nt] = B.off[t1];
     __syncthreads();
-    if (tid < nt && (s_off[tid] < 0 || s_off[tid + 1] < s_off[tid] || s_off[tid + 1] > B.n_comp)) s_bad = 1;
+    if (tid < nt) {
+        if (s_off[tid] < 0 || s_off[tid + 1] < s_off[tid] || s_off[tid + 1] > B.n_comp) s_bad = 1;
+        else atomicMax(&s_long, (int)min(s_off[tid + 1] - s_off[tid], (int64_t)kTiny + 1));
+    }
     __syncthreads();
     const int64_t base = s_off[0];
     const int64_t total = s_off[nt] - base;
-    if (s_bad || total > 0x3FFFFFFF) {
+    if (s_bad || total > 0x3FFFFFFF || s_long <= kTiny) {
         if (tid < nt) solve_serial(B, t0 + tid);
         return;
     }
@@ -556,35 +563,48 @@ __global__ void __launch_bounds__(128) hines_rest_kernel(Batch B, int lanes)
     }
 }
 
+// The status words, once what was queued on the stream is done.
+mm_status read_status(const Batch &B, cudaStream_t s, int h[3])
+{
+    if (cudaMemcpyAsync(h, B.status, 3 * sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess) return MM_ECUDA;
+    return cudaStreamSynchronize(s) == cudaSuccess ? MM_OK : MM_ECUDA;
+}
+
 mm_status run_batch(Batch B, cudaStream_t s)
 {
+    int h[3] = {0, 0, 0};
     if (cudaMemsetAsync(B.status, 0, 3 * sizeof(int), s) != cudaSuccess) return MM_ECUDA;
     if (B.n_trees > 0 && B.n_comp > 0) {
         // trees per block: about kBlockComps entries, fewer where the batch
         // would not fill the chip's slots otherwise, at least one tree.  The
         // tables of 1,024 chains leave room for six blocks per SM; groups with
         // more chains are taken up by a second launch with one block per SM, and
-        // the rest by a third (both end at once when nothing was left).
+        // the rest by a third, which the host makes only where a group was left
+        // (it waits for the solve in any case: 12 us of every other call)
         constexpr auto small = hines_batch_kernel<kSmallChains, 128, 6>;
         constexpr auto large = hines_left_kernel<kLargeChains, 256>;
         // 912: six blocks on each of 152 SMs
         const int64_t mean = std::max<int64_t>(1, B.n_comp / B.n_trees);
         B.trees_per_block = (int32_t)std::min<int64_t>(kMaxTrees, std::max<int64_t>(1, std::min<int64_t>(kBlockComps, B.n_comp / 912) / mean));
         const int64_t blocks = ((int64_t)B.n_trees + B.trees_per_block - 1) / B.trees_per_block;
-        if (cudaFuncSetAttribute(large, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of(kLargeChains)) != cudaSuccess)
-            return MM_ECUDA;
         small<<<(unsigned)blocks, 128, smem_of(kSmallChains), s>>>(B);
-        large<<<(unsigned)std::min<int64_t>(blocks, 152), 256, smem_of(kLargeChains), s>>>(B);
-        int lanes = 1;
-        while (lanes < B.trees_per_block) lanes *= 2;
-        const int64_t rest = std::min<int64_t>(blocks, B.left_cap) * lanes;
-        hines_rest_kernel<<<(unsigned)std::min<int64_t>((rest + 127) / 128, 152 * 16), 128, 0, s>>>(B, lanes);
         if (cudaGetLastError() != cudaSuccess) return MM_ECUDA;
+        mm_status st = read_status(B, s, h);
+        if (st != MM_OK) return st;
+        if (h[1] > 0) {
+            if (cudaFuncSetAttribute(large, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of(kLargeChains)) !=
+                cudaSuccess)
+                return MM_ECUDA;
+            large<<<(unsigned)std::min(h[1], 152), 256, smem_of(kLargeChains), s>>>(B);
+            int lanes = 1;
+            while (lanes < B.trees_per_block) lanes *= 2;
+            const int64_t rest = (int64_t)std::min(h[1], B.left_cap) * lanes;
+            hines_rest_kernel<<<(unsigned)std::min<int64_t>((rest + 127) / 128, 152 * 16), 128, 0, s>>>(B, lanes);
+            if (cudaGetLastError() != cudaSuccess) return MM_ECUDA;
+            if ((st = read_status(B, s, h)) != MM_OK) return st;
+        }
     }
-    int h = 0;
-    if (cudaMemcpyAsync(&h, B.status, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess) return MM_ECUDA;
-    if (cudaStreamSynchronize(s) != cudaSuccess) return MM_ECUDA;
-    return h ? MM_EINVAL : MM_OK;
+    return h[0] ? MM_EINVAL : MM_OK;
 }
 
 bool args_ok(int32_t n_trees, int64_t n_comp, const int64_t *off, const int32_t *parent, const double *a,

@@ -52,3 +52,22 @@ def test_large_trees_of_one_block_match_algorithm_1():
                          for v in (off, np.concatenate(trees).astype(np.int32), a, b, c, r))).cpu().numpy()
     ref = [oracle.hines_solve(*(v[s:e] for v in (a, b, c, r)), t.astype(np.int32)) for s, e, t in zip(off[:-1], off[1:], trees)]
     np.testing.assert_allclose(x, np.concatenate(ref), rtol=1e-12, atol=1e-14)
+
+
+@pytest.mark.parametrize("sizes", [[1], [8], [7, 8, 0, 1], [8, 9], [1, 8, 24], [8, 2000]])
+def test_tiny_trees_match_algorithm_1(sizes):
+    """Blocks of trees of up to eight entries (a thread solves each), and of one more, empty trees and large ones among them."""
+    import torch
+    rng = np.random.default_rng(8)
+    trees = [netgen.random_tree(rng, sizes[k % len(sizes)], 0.3) if sizes[k % len(sizes)] else np.zeros(0, np.int32)
+             for k in range(1000)]
+    off = np.concatenate([[0], np.cumsum([len(t) for t in trees])]).astype(np.int64)
+    n = int(off[-1])
+    a, c = -rng.uniform(0.1, 1.0, n), -rng.uniform(0.1, 1.0, n)
+    b, r = rng.uniform(8.0, 9.0, n), rng.normal(size=n)
+    x = mm.hines_solve(*(torch.as_tensor(v, device="cuda")
+                         for v in (off, np.concatenate(trees).astype(np.int32), a, b, c, r))).cpu().numpy()
+    for s, e, t in zip(off[:-1], off[1:], trees):
+        if e > s:
+            np.testing.assert_allclose(x[s:e], oracle.hines_solve(*(v[s:e] for v in (a, b, c, r)), t.astype(np.int32)),
+                                       rtol=1e-12, atol=1e-14)
