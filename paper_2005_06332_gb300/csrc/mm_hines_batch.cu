@@ -31,7 +31,8 @@ struct Batch {
     const double *a, *b, *c, *rhs;
     double *x, *work;
     int *status;             // [0] nonzero: a tree violates the parent rule or its entries lie outside n_comp;
-                             // [1], [2]: groups of trees left to hines_left_kernel and to hines_rest_kernel
+                             // [1], [2]: groups of trees left to hines_left_kernel and to hines_rest_kernel; [3],
+                             // [4], [5]: of some of the first, how many, their levels, their largest tree
     int32_t *left;           // these groups, left_cap of the first kind, then left_cap of the second
     int32_t left_cap;
     int32_t trees_per_block; // 1 .. kMaxTrees
@@ -129,10 +130,13 @@ constexpr int kMaxTrees = 128;     // trees of one block
 constexpr int kBlockComps = 2048;  // compartments aimed at per block
 constexpr int kTiny = 8;           // trees of a block up to this size: a thread each at once (see solve_group)
 constexpr int kSmallChains = 1024, kLargeChains = 8192;  // chains that a block's tables hold
-// A group that is left has more than kSmallChains entries, and the groups'
-// entries lie side by side: at most this many are left.  (Only offsets that run
-// backwards somewhere, which make the call fail, can overlap and leave more;
-// those blocks solve their trees serially at once.)
+constexpr int kSms = 152, kSmallSlots = 6 * kSms;  // blocks on the chip at a time with the larger and the smaller tables
+enum { kFirst, kLeft, kCount };                    // solve_group
+// Groups that may be left.  One that has more chains than the tables hold has
+// more than kSmallChains entries, and the groups' entries lie side by side; deep
+// ones are about as large.  Blocks beyond that (many deep small groups, or
+// offsets that run backwards somewhere, which make the call fail) solve their
+// trees serially at once.
 constexpr int32_t left_cap_of(int64_t n_comp) { return (int32_t)(n_comp / (kSmallChains + 1)) + 1; }
 static_assert(left_cap_of(MM_NOALLOC_MAX_COMPS) <= MM_NOALLOC_LEFT, "lists of the fixed scratch");
 constexpr size_t smem_of(int chains) { return (size_t)chains * 20 + 16; }
@@ -176,14 +180,15 @@ struct Front {
 // to 5,000 9.0 -> 0.57 ms.  128 threads and six blocks per SM; 32 or 64 threads
 // and more blocks 0.94 to 1.14 ms, groups of 4,096 entries 1.34 ms; eliminating
 // the diagonal alone first (with a c stored: 2 + 2 + 2 instructions in the
-// sweeps, but two passes more) 1.10 ms.  CHAINS: the chains that a block's tables hold.  FIRST:
-// every group of trees, else those that a smaller table left.  A group is on
-// one list at most, so that its trees are solved once, also where x is rhs.
+// sweeps, but two passes more) 1.10 ms.  CHAINS: the chains that a block's tables hold.  MODE:
+// kFirst every group of trees (`groups` in all), kLeft those that a smaller table
+// left, kCount the levels of one of these and nothing else.  A group is on
+// one list at a time, so that its trees are solved once, also where x is rhs.
 // Where no tree has more than kTiny entries a thread solves each at once: what
 // comes before the sweeps takes longer (a million trees of two entries 0.41 ->
 // 0.30 ms, of five 0.61 -> 0.56; of twelve it is the other way, 1.13 -> 1.24).
-template <int CHAINS, int NT, bool FIRST>
-__device__ __forceinline__ void solve_group(const Batch &B, int group)
+template <int CHAINS, int NT, int MODE>
+__device__ __forceinline__ void solve_group(const Batch &B, int group, int groups)
 {
     constexpr int kChunk = 2;  // entries per step of a sweep (operands loaded one step ahead)
     constexpr int kSub = 8;    // the same of the substitution
@@ -194,23 +199,24 @@ __device__ __forceinline__ void solve_group(const Batch &B, int group)
     int *up = head + CHAINS + 1;                           // chain above (pointer jumping)
     int *lev = up + CHAINS;                                // level; then where each level begins in key
     __shared__ int64_t s_off[kMaxTrees + 1];
-    __shared__ int s_warp[kLook * NT / 32], s_bad, s_K, s_go, s_long;
+    __shared__ int s_warp[kLook * NT / 32], s_bad, s_K, s_go, s_lev, s_long;
     static_assert(kMaxTrees < NT + 1 && (CHAINS & (CHAINS - 1)) == 0 && CHAINS <= 8192, "table sizes");
     constexpr unsigned long long kChain = 0x1FFF;  // a key: level << 43 | entry << 13 | chain
     const int tid = threadIdx.x, lane = tid & 31;
     const int32_t t0 = group * B.trees_per_block, t1 = min(t0 + B.trees_per_block, B.n_trees);
     const int nt = t1 - t0;
-    if (tid == 0) s_bad = s_K = s_long = 0;
+    if (tid == 0) s_bad = s_K = s_lev = s_long = 0;
     if (tid <= nt) s_off[tid] = B.off[t0 + tid];
     if (tid == 0 && nt == NT) s_off[nt] = B.off[t1];
     __syncthreads();
     if (tid < nt) {
         if (s_off[tid] < 0 || s_off[tid + 1] < s_off[tid] || s_off[tid + 1] > B.n_comp) s_bad = 1;
-        else atomicMax(&s_long, (int)min(s_off[tid + 1] - s_off[tid], (int64_t)kTiny + 1));
+        else atomicMax(&s_long, (int)min(s_off[tid + 1] - s_off[tid], (int64_t)0x7FFFFFFF));
     }
     __syncthreads();
     const int64_t base = s_off[0];
     const int64_t total = s_off[nt] - base;
+    if (MODE == kCount && (s_bad || total > 0x3FFFFFFF)) return;
     if (s_bad || total > 0x3FFFFFFF || s_long <= kTiny) {
         if (tid < nt) solve_serial(B, t0 + tid);
         return;
@@ -264,48 +270,28 @@ __device__ __forceinline__ void solve_group(const Batch &B, int group)
         if (__syncthreads_or(bad)) stop = 1;
         else if (s_K > CHAINS) stop = 2;
     }
+    if (MODE == kCount && stop) return;
     if (stop == 1) {
         if (tid < nt) solve_serial(B, t0 + tid);
         return;
     }
-    if (stop == 2) {  // left to a larger table or to hines_rest_kernel
+    // leaves the group to hines_left_kernel (1) or hines_rest_kernel (2)
+    auto leave = [&](int list) {
         if (tid == 0) {
-            const int q = atomicAdd(B.status + (FIRST ? 1 : 2), 1);
+            const int q = atomicAdd(B.status + list, 1);
             s_go = q < B.left_cap;
-            if (s_go) B.left[(FIRST ? 0 : B.left_cap) + q] = group;
+            if (s_go) B.left[(list - 1) * B.left_cap + q] = group;
         }
         __syncthreads();
         if (!s_go && tid < nt) solve_serial(B, t0 + tid);
+    };
+    if (stop == 2) {  // more chains than the tables hold
+        leave(MODE == kFirst ? 1 : 2);
         return;
     }
     const int K = s_K;
     if (tid == 0) head[K] = n;
-    // (x may be rhs: the copy leaves it as it is, for solve_serial)
-    bool other = false;    // rows that the sweeps are not for
-    uint32_t largest = 0;  // high_word of the couplings
-    for (int i0 = tid; i0 < n; i0 += kLook * NT) {
-        double bv[kLook], rv[kLook];
-#pragma unroll
-        for (int u = 0; u < kLook; ++u) {
-            const int i = min(i0 + u * NT, n - 1);
-            bv[u] = b[i];
-            rv[u] = rhs[i];
-            other |= !ordinary_row(bv[u], rv[u]);
-            if (B.x == B.rhs && parent[i] >= 0) largest = max(largest, high_word(a[i], c[i]));
-        }
-#pragma unroll
-        for (int u = 0; u < kLook; ++u) {
-            const int i = i0 + u * NT;
-            if (i < n) {
-                work[i] = bv[u];
-                x[i] = rv[u];
-            }
-        }
-    }
-    if (__syncthreads_or(other || largest > kCouplingMax)) {
-        if (tid < nt) solve_serial(B, t0 + tid);
-        return;
-    }
+    __syncthreads();
     // 2. the entry each chain hangs off, the chain it belongs to, and levels
     //    by pointer jumping over these
     int P2 = 32;
@@ -353,6 +339,57 @@ __device__ __forceinline__ void solve_group(const Batch &B, int group)
             __syncthreads();
         }
         if (!s_go) break;
+    }
+    int deepest = 0;
+    for (int k = tid; k < K; k += NT) deepest = max(deepest, lev[k]);
+    deepest = __reduce_max_sync(0xFFFFFFFFu, deepest);
+    if (lane == 0) atomicMax(&s_lev, deepest);
+    __syncthreads();
+    const int levels = s_lev + 1;
+    if (MODE == kCount) {
+        if (tid == 0) {
+            atomicAdd(B.status + 3, 1);
+            atomicAdd(B.status + 4, levels);
+            atomicMax(B.status + 5, s_long);
+        }
+        return;
+    }
+    // Deep trees of many groups are left to a thread each (see deep_batch; here
+    // with six blocks on an SM).  Trees of under 64 levels, or of more than 16
+    // entries to a level, are never that slow: without these two conditions the
+    // small ones of 3,000 trees of 50 to 5,000 went there too, 1.24 ms instead
+    // of 0.89.  3,000 combs of 1,000 entries and 500 levels 3.15 -> 2.75 ms,
+    // 20,000 of 200 1.38 -> 0.86 ms.
+    if (MODE == kFirst && levels >= 64 && 16LL * levels >= s_long &&
+        8LL * max(groups, kSmallSlots) * (levels + 30) > 6LL * kSmallSlots * s_long) {
+        leave(2);
+        return;
+    }
+    // (x may be rhs: the copy leaves it as it is, for solve_serial)
+    bool other = false;    // rows that the sweeps are not for
+    uint32_t largest = 0;  // high_word of the couplings
+    for (int i0 = tid; i0 < n; i0 += kLook * NT) {
+        double bv[kLook], rv[kLook];
+#pragma unroll
+        for (int u = 0; u < kLook; ++u) {
+            const int i = min(i0 + u * NT, n - 1);
+            bv[u] = b[i];
+            rv[u] = rhs[i];
+            other |= !ordinary_row(bv[u], rv[u]);
+            if (B.x == B.rhs && parent[i] >= 0) largest = max(largest, high_word(a[i], c[i]));
+        }
+#pragma unroll
+        for (int u = 0; u < kLook; ++u) {
+            const int i = i0 + u * NT;
+            if (i < n) {
+                work[i] = bv[u];
+                x[i] = rv[u];
+            }
+        }
+    }
+    if (__syncthreads_or(other || largest > kCouplingMax)) {
+        if (tid < nt) solve_serial(B, t0 + tid);
+        return;
     }
     // 3. the chains by level and the entry they hang off (bitonic), and where
     //    each level begins
@@ -535,7 +572,7 @@ __device__ __forceinline__ void solve_group(const Batch &B, int group)
 template <int CHAINS, int NT, int BLOCKS>
 __global__ void __launch_bounds__(NT, BLOCKS) hines_batch_kernel(Batch B)
 {
-    solve_group<CHAINS, NT, true>(B, blockIdx.x);
+    solve_group<CHAINS, NT, kFirst>(B, blockIdx.x, gridDim.x);
 }
 
 // The groups of trees that hines_batch_kernel left, with a larger table.
@@ -544,36 +581,59 @@ __global__ void __launch_bounds__(NT, 1) hines_left_kernel(Batch B)
 {
     const int left = min(B.status[1], B.left_cap);
     for (int q = blockIdx.x; q < left; q += gridDim.x) {
-        solve_group<CHAINS, NT, false>(B, B.left[q]);
+        solve_group<CHAINS, NT, kLeft>(B, B.left[q], left);
         __syncthreads();
     }
 }
 
-// The trees of groups with more chains than the largest table holds, a thread
-// for each tree, so that all of them run side by side: 40 trees of 20,000
-// entries before 60,000 of 50, which fall into two groups, 892 ms with a thread
-// per group, 46 ms so.  lanes: a power of two, threads for each group.
-__global__ void __launch_bounds__(128) hines_rest_kernel(Batch B, int lanes)
+// The levels of some of the groups left (a block each, evenly over the list).
+template <int CHAINS, int NT>
+__global__ void __launch_bounds__(NT, 1) hines_look_kernel(Batch B)
 {
-    const int left = min(B.status[2], B.left_cap);
+    const int left = min(B.status[1], B.left_cap);
+    solve_group<CHAINS, NT, kCount>(B, B.left[(int64_t)blockIdx.x * left / gridDim.x], left);
+}
+
+// The trees of one of the lists, a thread for each tree, so that all of them run
+// side by side: 40 trees of 20,000 entries before 60,000 of 50, which fall into
+// two groups, 892 ms with a thread per group, 46 ms so.  lanes: a power of two,
+// threads for each group.
+__global__ void __launch_bounds__(128) hines_rest_kernel(Batch B, int list, int lanes)
+{
+    const int left = min(B.status[list], B.left_cap);
     for (int64_t i = blockIdx.x * 128LL + threadIdx.x; i < (int64_t)left * lanes; i += gridDim.x * 128LL) {
-        const int64_t t0 = (int64_t)B.left[B.left_cap + i / lanes] * B.trees_per_block;
+        const int64_t t0 = (int64_t)B.left[(list - 1) * B.left_cap + i / lanes] * B.trees_per_block;
         const int64_t t1 = min(t0 + B.trees_per_block, (int64_t)B.n_trees);
         for (int64_t t = t0 + i % lanes; t < t1; t += lanes) solve_serial(B, (int32_t)t);
     }
 }
 
-// The status words, once what was queued on the stream is done.
-mm_status read_status(const Batch &B, cudaStream_t s, int h[3])
+// Whether `left` groups, of which `some` have `levels` levels together and no
+// tree of more than `longest` entries, are solved sooner by a thread per tree than
+// one to an SM with the larger tables.  A level costs a block 1.7 us of barriers
+// and dependent loads whatever it holds, what comes before and after the sweeps
+// about 30 levels; a thread costs 2 us an entry, but all trees of the batch run
+// at once.  One answer for all of them: where only some go to a thread, the
+// others take their time besides (3,000 trees of 1,500 entries numbered breadth
+// first, some 120 levels: 5.3 ms all with tables, 4.9 all with threads, 7.2
+// mixed).  3,000 combs of 3,000 entries and 1,500 levels: 48 ms with tables, 7.9
+// with threads, 7.8 so; 2,000 stars of 4,000, two levels, 10.3 and 12.3.
+bool deep_batch(int left, int some, int levels, int longest)
 {
-    if (cudaMemcpyAsync(h, B.status, 3 * sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess) return MM_ECUDA;
+    return some > 0 && 1.7 * ((double)levels / some + 30.0) * left / kSms > 2.0 * longest;
+}
+
+// The status words, once what was queued on the stream is done.
+mm_status read_status(const Batch &B, cudaStream_t s, int h[6])
+{
+    if (cudaMemcpyAsync(h, B.status, 6 * sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess) return MM_ECUDA;
     return cudaStreamSynchronize(s) == cudaSuccess ? MM_OK : MM_ECUDA;
 }
 
 mm_status run_batch(Batch B, cudaStream_t s)
 {
-    int h[3] = {0, 0, 0};
-    if (cudaMemsetAsync(B.status, 0, 3 * sizeof(int), s) != cudaSuccess) return MM_ECUDA;
+    int h[6] = {};
+    if (cudaMemsetAsync(B.status, 0, 6 * sizeof(int), s) != cudaSuccess) return MM_ECUDA;
     if (B.n_trees > 0 && B.n_comp > 0) {
         // trees per block: about kBlockComps entries, fewer where the batch
         // would not fill the chip's slots otherwise, at least one tree.  The
@@ -583,23 +643,36 @@ mm_status run_batch(Batch B, cudaStream_t s)
         // (it waits for the solve in any case: 12 us of every other call)
         constexpr auto small = hines_batch_kernel<kSmallChains, 128, 6>;
         constexpr auto large = hines_left_kernel<kLargeChains, 256>;
-        // 912: six blocks on each of 152 SMs
         const int64_t mean = std::max<int64_t>(1, B.n_comp / B.n_trees);
-        B.trees_per_block = (int32_t)std::min<int64_t>(kMaxTrees, std::max<int64_t>(1, std::min<int64_t>(kBlockComps, B.n_comp / 912) / mean));
+        const int64_t trees = std::min<int64_t>(kBlockComps, B.n_comp / kSmallSlots) / mean;
+        B.trees_per_block = (int32_t)std::min<int64_t>(kMaxTrees, std::max<int64_t>(1, trees));
         const int64_t blocks = ((int64_t)B.n_trees + B.trees_per_block - 1) / B.trees_per_block;
         small<<<(unsigned)blocks, 128, smem_of(kSmallChains), s>>>(B);
         if (cudaGetLastError() != cudaSuccess) return MM_ECUDA;
         mm_status st = read_status(B, s, h);
         if (st != MM_OK) return st;
-        if (h[1] > 0) {
+        if (h[1] > 0 || h[2] > 0) {
+            constexpr auto look = hines_look_kernel<kLargeChains, 256>;
             if (cudaFuncSetAttribute(large, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of(kLargeChains)) !=
-                cudaSuccess)
+                    cudaSuccess ||
+                cudaFuncSetAttribute(look, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of(kLargeChains)) !=
+                    cudaSuccess)
                 return MM_ECUDA;
-            large<<<(unsigned)std::min(h[1], 152), 256, smem_of(kLargeChains), s>>>(B);
+            const int left = std::min(h[1], B.left_cap);
+            bool deep = false;  // never with two groups to an SM or fewer: levels are at most half the entries
+            if (left > 2 * kSms) {
+                look<<<kSms, 256, smem_of(kLargeChains), s>>>(B);
+                if (cudaGetLastError() != cudaSuccess) return MM_ECUDA;
+                if ((st = read_status(B, s, h)) != MM_OK) return st;
+                deep = deep_batch(left, h[3], h[4], h[5]);
+            }
+            if (left > 0 && !deep) large<<<(unsigned)std::min(left, kSms), 256, smem_of(kLargeChains), s>>>(B);
             int lanes = 1;
             while (lanes < B.trees_per_block) lanes *= 2;
-            const int64_t rest = (int64_t)std::min(h[1], B.left_cap) * lanes;
-            hines_rest_kernel<<<(unsigned)std::min<int64_t>((rest + 127) / 128, 152 * 16), 128, 0, s>>>(B, lanes);
+            const int64_t rest = (int64_t)B.left_cap * lanes;
+            const unsigned rest_blocks = (unsigned)std::min<int64_t>((rest + 127) / 128, kSms * 16);
+            if (deep) hines_rest_kernel<<<rest_blocks, 128, 0, s>>>(B, 1, lanes);
+            hines_rest_kernel<<<rest_blocks, 128, 0, s>>>(B, 2, lanes);
             if (cudaGetLastError() != cudaSuccess) return MM_ECUDA;
             if ((st = read_status(B, s, h)) != MM_OK) return st;
         }

@@ -71,3 +71,24 @@ def test_tiny_trees_match_algorithm_1(sizes):
         if e > s:
             np.testing.assert_allclose(x[s:e], oracle.hines_solve(*(v[s:e] for v in (a, b, c, r)), t.astype(np.int32)),
                                        rtol=1e-12, atol=1e-14)
+
+
+@pytest.mark.parametrize("count,n,step", [(4000, 1000, 2), (1200, 1500, 1), (160, 8300, 1), (3, 700, 1)])
+def test_deep_trees_match_algorithm_1(count, n, step):
+    """Combs (step 1: two spines, every entry a chain; step 2: a spine whose entries have a leaf each, in preorder), whose
+    levels are as many as half their entries: more blocks than the chip holds at a time, larger than the tables, and few."""
+    import torch
+    rng = np.random.default_rng(7)
+    i = np.arange(n)
+    par = np.maximum(i - 2, 0) if step == 1 else np.where(i % 2 == 1, i - 1, np.maximum(i - 2, 0))
+    par[0] = -1
+    off = np.arange(count + 1, dtype=np.int64) * n
+    N = count * n
+    a, c, r = -rng.uniform(0.1, 1.0, N), -rng.uniform(0.1, 1.0, N), rng.normal(size=N)
+    b = rng.uniform(4.0, 5.0, N)
+    x = mm.hines_solve(*(torch.as_tensor(v, device="cuda")
+                         for v in (off, np.tile(par, count).astype(np.int32), a, b, c, r))).cpu().numpy()
+    for s in range(0, N, max(n, N // 40 // n * n)):  # forty of them
+        e = s + n
+        np.testing.assert_allclose(x[s:e], oracle.hines_solve(a[s:e], b[s:e], c[s:e], r[s:e], par.astype(np.int32)),
+                                   rtol=1e-12, atol=1e-14)
