@@ -1015,11 +1015,8 @@ mm_status build(mm_net *net, const mm_morphologies *morph, const mm_channel_para
         g = net->sa32;
         g.item0 = L.n_small + L.n_big;
         g.item1 = (int32_t)L.groups.size();
-        g.n_huge = 0;
+        g.n_huge = L.n_huge;
         g.queue = &net->ctl->giant_head;
-        // items of more compartments than the shared-memory classes' records
-        // hold (the largest come first) get a cluster of blocks each
-        for (int32_t gi = g.item0; gi < g.item1 && L.groups[(size_t)gi].ncomp > 32767; ++gi) ++g.n_huge;
         net->giant_blocks = std::max(1, mmk_giant_blocks(net->n_giant, g.n_huge));
         // the giant items' compartments in chunks for the assembly and
         // update kernels: first chunk of each giant item, then the total

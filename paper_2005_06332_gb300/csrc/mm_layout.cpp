@@ -657,16 +657,6 @@ std::string build_layout(const LayoutInput &in, Layout &out, bool *invalid)
             gr.mcnt_off = (int32_t)o.mcnt_off;
             gr.npath = pb.npath;
             gr.nlevel = pb.nlevel;
-            if (giant) {
-                gr.scratch0 = L.giant_comps;
-                L.giant_comps += gr.ncomp;
-                if (L.giant_paths + pb.npath > INT32_MAX) {
-                    e << "giant work items hold more than 2^31 paths";
-                    return msg(e);
-                }
-                gr.pscratch0 = (int32_t)L.giant_paths;
-                L.giant_paths += pb.npath;
-            }
         }
         blob.resize((blob.size() + 15) & ~(size_t)15, 0);
         gr.meta_off = (int64_t)L.meta.size();
@@ -692,6 +682,21 @@ std::string build_layout(const LayoutInput &in, Layout &out, bool *invalid)
     L.n_small = (int32_t)L.groups.size();
     L.n_big = (int32_t)bigs.size();
     L.groups.insert(L.groups.end(), bigs.begin(), bigs.end());
+    // the giants beyond the 16-bit records first, whatever the neurons' order
+    // (the solve gives each a cluster of blocks), the others as they come
+    L.n_huge = (int32_t)(std::stable_partition(giants.begin(), giants.end(),
+                                               [](const mmk::GroupRec &g) { return g.ncomp > 32767; }) -
+                         giants.begin());
+    for (mmk::GroupRec &gr : giants) {
+        if (L.giant_paths + gr.npath > INT32_MAX) {
+            e << "giant work items hold more than 2^31 paths";
+            return msg(e);
+        }
+        gr.scratch0 = L.giant_comps;
+        L.giant_comps += gr.ncomp;
+        gr.pscratch0 = (int32_t)L.giant_paths;
+        L.giant_paths += gr.npath;
+    }
     L.groups.insert(L.groups.end(), giants.begin(), giants.end());
 
     // 4a. synaptic sites: one per compartment that receives a synapse

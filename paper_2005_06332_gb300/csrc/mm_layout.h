@@ -60,8 +60,9 @@ struct Layout {
     int32_t max_comps = 0, max_segs = 0;
     int32_t max_waves = 0, max_meta = 0;
     // items [0, n_small) fit the regular shared-memory budget, the next n_big
-    // the large one; the rest are giants
-    int32_t n_small = 0, n_big = 0;
+    // the large one; the rest are giants, of which the first n_huge are solved
+    // by a cluster of blocks each
+    int32_t n_small = 0, n_big = 0, n_huge = 0;
     int32_t big_max_comps = 0, big_max_segs = 0, big_max_meta = 0;
     // largest shared-memory need (model above) of one item of each class
     int64_t max_smem = 0, big_max_smem = 0;
