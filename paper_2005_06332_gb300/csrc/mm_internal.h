@@ -174,6 +174,9 @@ struct ScaleArgs64 {
     double cm_leak;                   // (Cm / dt + the implicit leak) * 1e3: uS per cm^2 of membrane
 };
 
+// Blocks of the cluster that solves a huge giant item (the portable maximum).
+constexpr int kGiantCluster = 8;
+
 // Fixed-point state of the FP32c path: V = Vq * 2^-23 mV (int32, +-256 mV),
 // gates x = q * 2^-32 (uint32).  FP32 increments are rounded once and added
 // exactly, so the state itself never accumulates rounding.

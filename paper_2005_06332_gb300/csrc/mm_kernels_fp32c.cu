@@ -912,10 +912,14 @@ __global__ void __launch_bounds__(NT, 1024 / NT) step_fp32c_kernel(StepArgs32 a)
 }
 
 
-// Paths of a giant of at least this many compartments are swept by a warp.
-constexpr int kGiantWarpPath = 48;
-// Blocks of a cluster (the portable maximum).
-constexpr int kGiantCluster = 8;
+// Paths of a giant of at least this many compartments are swept by a warp: where
+// a cluster solves it or it is a small one, whose paths leave most lanes idle,
+// and where one block solves a huge one, whose lanes are busy (the warp's three
+// passes then cost more than they hide).  us per step with 48, 160 and no such
+// paths: one block each for 2 giants of 100,000 among 2.6 M compartments 564, 489,
+// 558, for 40 880, 796, 895, for one of 300,000 1514, 1146, 1257; 174 giants of
+// 9,000 to 20,000 among 19 M 1117, 1138, 1156.
+constexpr int kGiantWarpPath = 48, kHugeWarpPath = 160;
 
 // Solve of one giant work item by a team of NTT threads, of which this is
 // thread tid: a block, or (COOP) a cluster of blocks, whose scratch is written
@@ -1318,11 +1322,12 @@ __device__ __forceinline__ void giant_solve(const StepArgs32 &a, int gi, int tid
     };
     // the number of paths at the start of a level (paths run longest
     // first) that a whole warp takes
+    const int warp_path = COOP || G.ncomp <= 32767 ? kGiantWarpPath : kHugeWarpPath;
     auto warp_paths = [&](int pb, int pe) {
         int lo = pb, hi = pe;  // first path shorter than the threshold
         while (lo < hi) {
             const int mid = (lo + hi) >> 1;
-            if (paths[mid].end - paths[mid].head >= kGiantWarpPath) lo = mid + 1; else hi = mid;
+            if (paths[mid].end - paths[mid].head >= warp_path) lo = mid + 1; else hi = mid;
         }
         return lo - pb;
     };
@@ -1364,12 +1369,14 @@ __global__ void __launch_bounds__(NT) giant_fp32c_kernel(StepArgs32 a)
     // threads as one team: a lane waits some hundred clocks for each
     // compartment of its path, so what a huge neuron wants is more lanes than
     // one SM's.  The other clusters' blocks take an item each, by themselves
-    // (every team has one item: the launch is sized so).  Two neurons of 100,000
-    // compartments among 19 of 9,000 to 20,000: the solve 508 us with a block per
-    // neuron and a lane per path, 298 us with clusters of eight blocks and a warp
-    // on each path of 48 compartments or more; the whole step (1,502 neurons)
-    // 554 -> 340 us.  Thresholds of 32 and 96: 350 and 390 us; clusters of 16, 504
-    // us (they wait for 16 free SMs); clusters for the small giants too, 371 us.
+    // (every team has one item: the launch is sized so); without huge items the
+    // launch has no clusters.  Two neurons of 100,000 compartments among 19 of
+    // 9,000 to 20,000: the solve 508 us with a block per neuron and a lane per
+    // path, 298 us with clusters of eight blocks and a warp on each path of 48
+    // compartments or more; the whole step (1,502 neurons) 533 -> 330 us.
+    // Thresholds of 32 and 96: 350 and 390 us; clusters of 16, 504 us (they wait
+    // for 16 free SMs); clusters for the small giants too, 371 us.  Which items
+    // get a cluster is the layout's choice (cluster_items).
     int nblk, rank;
     asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(nblk));
     asm("mov.u32 %0, %%cluster_ctaid.x;" : "=r"(rank));

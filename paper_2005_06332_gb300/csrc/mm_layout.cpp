@@ -325,6 +325,35 @@ int64_t choose_budget(const LayoutInput &in, const Layout &L, const std::vector<
     return kBudgets[i];
 }
 
+// How many giants are solved by a cluster of blocks each; these come first then.
+// A cluster of eight ends a neuron's solve in about 0.6 of a block's time and
+// takes eight SMs for it, so it pays where that solve is what the step waits for:
+// for the giants of over 0.6 of the largest one's size (the others end before it
+// by themselves), while the rest of the network keeps an SM busy for less than
+// about the largest one's solve (0.62 of its compartments to an SM), and while
+// the clusters take at most half of the SMs, fewer where the giants are smaller
+// than 100,000.  152 SMs, us per step with a block each and with clusters: 2.6 M
+// other compartments and 2, 8, 16, 40 giants of 100,000 489, 578, 653, 795 and
+// 329, 517, 715, 1237; 2, 8 of 50,000 342, 359 and 288, 359; 8 of 35,000 281 and
+// 345; 8.3 M and 2, 10 of 100,000 706, 744 and 564, 758; 13 M and 2, 8 669, 720
+// and 695, 828; 64 giants and nothing else 858 and 1852.
+int32_t cluster_items(const LayoutInput &in, const Layout &L, std::vector<mmk::GroupRec> &giants)
+{
+    int32_t largest = 0;
+    for (const mmk::GroupRec &g : giants) largest = std::max(largest, g.ncomp);
+    auto wants = [&](const mmk::GroupRec &g) { return g.ncomp > 32767 && g.ncomp > 0.6 * largest; };
+    int64_t count = 0, rest = L.C;
+    for (const mmk::GroupRec &g : giants)
+        if (wants(g)) {
+            ++count;
+            rest -= g.ncomp;
+        }
+    const double size = std::min(largest / 100000.0, 1.0);
+    if (rest > 0.62 * largest * in.sms || mmk::kGiantCluster * count > 0.5 * in.sms * size) return 0;
+    std::stable_partition(giants.begin(), giants.end(), wants);
+    return (int32_t)count;
+}
+
 }  // namespace
 
 void neuron_features(int32_t n, const int32_t *parent, const double *L_um, const double *d_um, float *out)
@@ -682,11 +711,7 @@ std::string build_layout(const LayoutInput &in, Layout &out, bool *invalid)
     L.n_small = (int32_t)L.groups.size();
     L.n_big = (int32_t)bigs.size();
     L.groups.insert(L.groups.end(), bigs.begin(), bigs.end());
-    // the giants beyond the 16-bit records first, whatever the neurons' order
-    // (the solve gives each a cluster of blocks), the others as they come
-    L.n_huge = (int32_t)(std::stable_partition(giants.begin(), giants.end(),
-                                               [](const mmk::GroupRec &g) { return g.ncomp > 32767; }) -
-                         giants.begin());
+    L.n_huge = cluster_items(in, L, giants);
     for (mmk::GroupRec &gr : giants) {
         if (L.giant_paths + gr.npath > INT32_MAX) {
             e << "giant work items hold more than 2^31 paths";

@@ -44,9 +44,16 @@ def packed(tmp_path_factory):
     return run
 
 
-def test_huge_giants_come_first_in_any_order(packed):
-    """A supplied order with a small giant ahead of the huge ones and one between them: the huge ones first, the others in
-    their order."""
+def test_giants_that_get_clusters(packed):
+    """In a supplied order with small giants ahead of the huge ones and between them, the huge ones come first, the others
+    in their order; giants of under 0.6 of the largest, too many giants, smaller ones, or much else in the network: none."""
     sizes, cost = [12000, 100000, 11000, 100000, 9900, 40], [9.0, 8.0, 7.0, 6.0, 5.0, 4.0]
     f, giants = packed(sizes, cost=cost)
     assert f["huge"] == 2 and giants == [100000, 100000, 12000, 11000, 9900]
+    assert packed([100000, 60001, 60000, 33000])[0]["huge"] == 2
+    f, giants = packed([33000, 60000, 500000, 60001], cost=[4.0, 3.0, 2.0, 1.0])
+    assert f["huge"] == 1 and giants == [500000, 33000, 60000, 60001]
+    assert packed([100000] * 9)[0]["huge"] == 9 and packed([100000] * 10)[0]["huge"] == 0  # 72 and 80 of 152 SMs
+    assert packed([50000] * 4)[0]["huge"] == 4 and packed([50000] * 5)[0]["huge"] == 0  # half as many
+    assert packed([32768])[0]["huge"] == 1 and packed([32767])[0]["huge"] == 0
+    assert packed([40000] + [1000] * 3760)[0]["huge"] == 1 and packed([40000] + [1000] * 3780)[0]["huge"] == 0
