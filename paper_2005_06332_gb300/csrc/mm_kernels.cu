@@ -94,7 +94,9 @@ __global__ void init_kernel(InitArgs a)
 // per item: down each path s = 1 at its head and then the mantissa of
 // 1 / (w g s_parent) (w the implicit share of a coupling), so that the coupling
 // w g s s_parent inside a path is a power of two, whose exponent field is
-// stored; at a head the coupling to the parent compartment, negative.  Then the
+// stored; at a head the coupling to the parent compartment, negative.  A coupling
+// below 2^-500 uS, or none (infinite Ra), is taken as 2^-500, which adds nothing
+// to any diagonal and whose square keeps exponent fields within 32 bits.  Then the
 // constant part of the diagonal: C/dt, the implicit leak and the couplings,
 // times s^2 -- inside a path as the matrix holds them, s 2^k / s_parent.
 __global__ void __launch_bounds__(128) scale_kernel(ScaleArgs64 a)
@@ -114,12 +116,17 @@ __global__ void __launch_bounds__(128) scale_kernel(ScaleArgs64 a)
         for (int j = h; j < P.end; ++j) {
             double sn = 1.0, link = 0.0, next_own = 0.0;
             if (j + 1 < P.end) {
-                const double p = 1.0 / (a.gimp * gax[j + 1] * s);
-                sn = mantissa(p);
-                const int k = -exponent2(p);
-                kexp[j + 1] = k;
-                link = scale2(s / sn, k);
-                next_own = scale2(sn / s, k);
+                const double c = a.gimp * gax[j + 1] * s;
+                if (c < 0x1p-500) {
+                    kexp[j + 1] = -(500 << 20);
+                } else {
+                    const double p = 1.0 / c;
+                    sn = mantissa(p);
+                    const int k = -exponent2(p);
+                    kexp[j + 1] = k;
+                    link = scale2(s / sn, k);
+                    next_own = scale2(sn / s, k);
+                }
             }
             const double s2 = s * s * area[j];
             sc[j] = j == h ? -0.0 : s;
