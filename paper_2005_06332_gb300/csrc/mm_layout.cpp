@@ -221,19 +221,20 @@ int64_t packed_need(const LayoutInput &in, int64_t comps, int64_t paths, int64_t
     return in.smem_per_comp * comps + (in.smem_per_path + 16) * paths + 16 * neurons + 256;
 }
 
-// Runs of whole neurons under a budget: the boundaries [items + 1].  paths
-// (per internal neuron; may be empty) closes an item before its shared
-// memory could pass giant_smem_limit, which would take it out of the regular
-// class.  In a supplied order, where neurons of all sizes follow one another,
-// items that all end short of the budget leave 9 % of it empty (10,000 neurons
-// of F-distributed sizes, 2,048): there, and in the precision with size
-// classes, an item may pass the budget by an eighth if it is then nearer to it
-// than without its last neuron (181 -> 177 us per step).  In size order
-// neighbours are alike and would all end on the same side.
+// Runs of whole neurons under a budget: the boundaries [items + 1].  paths (per
+// internal neuron; empty for a given budget, which is kept to the letter) closes
+// an item before its shared memory could pass giant_smem_limit, which would take
+// it out of the regular class, and lets it pass the budget: in a supplied order,
+// where neurons of all sizes follow one another, items that all end short of the
+// budget leave 9 % of it empty (10,000 neurons of F-distributed sizes, 2,048).
+// There, and in the precision with size classes, an item may pass the budget by an
+// eighth if it is then nearer to it than without its last neuron (181 -> 177 us
+// per step).  In size order neighbours are alike and would all end on the same
+// side.
 void pack_items(const LayoutInput &in, const Layout &L, const std::vector<int32_t> &paths, int64_t budget,
                 std::vector<int32_t> &gstart)
 {
-    const int64_t over = in.cost && in.giant_smem_limit > 0 ? budget / 8 : 0;
+    const int64_t over = in.cost && in.giant_smem_limit > 0 && !paths.empty() ? budget / 8 : 0;
     gstart.clear();
     int64_t cur = 0, cp = 0;
     int32_t cnt = 0;
@@ -546,7 +547,7 @@ std::string build_layout(const LayoutInput &in, Layout &out, bool *invalid)
 
     // 3a. group boundaries
     std::vector<int32_t> gstart;
-    if (in.group_comps > 0 && !in.cost) {
+    if (in.group_comps > 0) {
         pack_items(in, L, {}, in.group_comps, gstart);
     } else {
         std::vector<int32_t> paths((size_t)N, 0);  // a path ends at each leaf
@@ -559,7 +560,7 @@ std::string build_layout(const LayoutInput &in, Layout &out, bool *invalid)
             for (int32_t i = 1; i < n; ++i) inner[(size_t)par[i]] = 1;
             paths[(size_t)k] = n - (int32_t)std::count(inner.begin(), inner.end(), (char)1);
         }
-        pack_items(in, L, paths, in.group_comps > 0 ? in.group_comps : choose_budget(in, L, paths), gstart);
+        pack_items(in, L, paths, choose_budget(in, L, paths), gstart);
     }
     const int32_t G = (int32_t)gstart.size() - 1;
     L.groups.clear();

@@ -1,6 +1,7 @@
 """Host logic: work items as mm_layout.cpp packs them with the values that the
 library gives it -- the device's SMs, the items' fixed cost, a supplied order --
 checked by tests/layout_budget_check.cpp (no GPU)."""
+import heapq
 import os
 import shutil
 import subprocess
@@ -57,3 +58,64 @@ def test_giants_that_get_clusters(packed):
     assert packed([50000] * 4)[0]["huge"] == 4 and packed([50000] * 5)[0]["huge"] == 0  # half as many
     assert packed([32768])[0]["huge"] == 1 and packed([32767])[0]["huge"] == 0
     assert packed([40000] + [1000] * 3760)[0]["huge"] == 1 and packed([40000] + [1000] * 3780)[0]["huge"] == 0
+
+
+@pytest.mark.parametrize("fp64", [False, True])
+@pytest.mark.parametrize("budget", [1, 600, 2048, 8192])
+def test_a_given_budget_is_kept_in_a_supplied_order(packed, budget, fp64):
+    """No item of several neurons passes a given budget, none is closed early, whatever the order."""
+    sizes = [int(n) for n in np.random.default_rng(1).integers(50, 900, 400)]
+    cost = np.random.default_rng(2).random(400)
+    f, _ = packed(sizes, p_branch=0.6, group_comps=budget, cost=cost, fp64=fp64)
+    assert f["several"] <= budget
+    order, items, held = np.argsort(-cost.astype(np.float32), kind="stable"), 0, budget + 1
+    for k in order:  # a new item where the next neuron does not fit
+        if held + sizes[k] > budget:
+            items, held = items + 1, 0
+        held += sizes[k]
+    assert f["items"] == items
+
+
+SHAPES = [([1], 0.0), ([4097], 0.1), ([1] * 20_000, 0.0), ([300] * 700, 0.9), ([450] * 300, 0.1), ([255] * 64, 0.1),
+          ([1000] * 4000, 0.05), ([7000] + [37] * 500, 0.05)]
+
+
+@pytest.mark.parametrize("fp64", [False, True])
+@pytest.mark.parametrize("sizes,p_branch", SHAPES)
+def test_the_budget_chosen_for_152_sms(packed, sizes, p_branch, fp64):
+    """The choice that ships: items of the largest budget at most (in a supplied FP32c order an eighth more), all in the
+    regular class but for a neuron too large for it."""
+    for cost in (None, np.random.default_rng(3).random(len(sizes))):
+        f, _ = packed(sizes, p_branch=p_branch, cost=cost, fp64=fp64)
+        assert f["several"] <= 4096 + (512 if cost is not None and not fp64 else 0)
+        assert f["large"] == (1 if max(sizes) > 5000 and not fp64 else 0) and f["giant"] == 0
+        assert f["smem"] <= (227 if fp64 else 110) * 1024
+
+
+@pytest.mark.parametrize("sizes,p_branch", SHAPES)
+def test_the_chosen_budget_ends_first_by_the_estimate(packed, sizes, p_branch):
+    """FP64 in size order, the estimate computed here: the chosen packing is within 3 % of the best of the budgets."""
+    rng = np.random.default_rng(5)
+    leaves = [n - len(set(netgen.random_tree(rng, n, p_branch)[1:].tolist())) for n in sizes]
+    ends = {}
+    for budget in (256, 384, 512, 768, 1024, 1536, 2048, 3072, 4096):
+        items, wide, cur = [], 0, None
+        for k in sorted(range(len(sizes)), key=lambda k: -sizes[k]):
+            if cur is None or cur[0] + sizes[k] > budget:
+                cur = [0, 0, 0]
+                items.append(cur)
+            cur[0], cur[1], cur[2] = cur[0] + sizes[k], cur[1] + leaves[k], cur[2] + 1
+        wide = max(16 * c + 16 * p + 16 * n + 256 for c, p, n in items)
+        cost = [300 + c for c, _, _ in items]
+        slots = 152 if wide > 110 * 1024 else 304
+        if len(cost) <= slots:
+            end = max(0.55 * c + 0.45 * (cost[152 + i] if 152 + i < len(cost) else 0) for i, c in enumerate(cost[:152]))
+        else:
+            busy = [0] * slots
+            for c in cost:
+                heapq.heappush(busy, heapq.heappop(busy) + c)
+            end = max(busy)
+        ends.setdefault(len(items), end)
+        ends[len(items)] = min(end, ends[len(items)])
+    f, _ = packed(sizes, p_branch=p_branch, fp64=True)
+    assert ends[f["items"]] <= 1.03 * min(ends.values())
