@@ -164,10 +164,10 @@ typedef struct {
     int32_t graph_steps;        /* steps per captured CUDA graph; 0 = no graphs */
     int32_t block_threads;      /* threads per work item's block; 0 = automatic */
     int32_t group_comps;        /* compartment budget of one work item, which whole neurons are packed
-                                   under (a neuron larger than it is an item by itself); 0 = automatic:
-                                   the best of a set by an estimate of the step's makespan (with
-                                   block_threads given: 4096, MM_FP32C 2048), which an MM_FP32C item may
-                                   pass by an eighth under MM_SCHED_COST */
+                                   under (a neuron larger than it is an item by itself; under
+                                   MM_SCHED_COST an MM_FP32C item may pass it by an eighth, where that
+                                   is nearer to it); 0 = automatic: the best of a set by an estimate of
+                                   the step's makespan, or with block_threads given 4096, MM_FP32C 2048 */
     int32_t device;             /* CUDA device ordinal */
     int32_t time_items;         /* MM_FP32C: record each work item's solve time (mm_read_neuron_times) */
     int32_t scheme;             /* MM_SCHEME_BE | MM_SCHEME_CN */

@@ -221,31 +221,32 @@ int64_t packed_need(const LayoutInput &in, int64_t comps, int64_t paths, int64_t
     return in.smem_per_comp * comps + (in.smem_per_path + 16) * paths + 16 * neurons + 256;
 }
 
-// Runs of whole neurons under a budget: the boundaries [items + 1].  paths (per
-// internal neuron; empty for a given budget, which is kept to the letter) closes
-// an item before its shared memory could pass giant_smem_limit, which would take
-// it out of the regular class, and lets it pass the budget: in a supplied order,
-// where neurons of all sizes follow one another, items that all end short of the
-// budget leave 9 % of it empty (10,000 neurons of F-distributed sizes, 2,048).
-// There, and in the precision with size classes, an item may pass the budget by an
-// eighth if it is then nearer to it than without its last neuron (181 -> 177 us
-// per step).  In size order neighbours are alike and would all end on the same
-// side.
-void pack_items(const LayoutInput &in, const Layout &L, const std::vector<int32_t> &paths, int64_t budget,
+// Runs of whole neurons under a budget: the boundaries [items + 1].  In a supplied
+// order, where neurons of all sizes follow one another, items that all end short
+// of the budget leave 9 % of it empty (10,000 neurons of F-distributed sizes,
+// 2,048).  There, and in the precision with size classes, an item may pass the
+// budget by an eighth if it is then nearer to it than without its last neuron and
+// stays in the regular class (181 -> 177 us per step).  In size order neighbours
+// are alike and would all end on the same side.  A chosen budget (not given) also
+// closes an item before its shared memory could pass giant_smem_limit, which would
+// take it out of the regular class.  paths: per internal neuron; empty for a given
+// budget in size order, which needs none.
+void pack_items(const LayoutInput &in, const Layout &L, const std::vector<int32_t> &paths, int64_t budget, bool given,
                 std::vector<int32_t> &gstart)
 {
-    const int64_t over = in.cost && in.giant_smem_limit > 0 && !paths.empty() ? budget / 8 : 0;
+    const bool classes = in.giant_smem_limit > 0;
+    const int64_t over = in.cost && classes ? budget / 8 : 0;
     gstart.clear();
     int64_t cur = 0, cp = 0;
     int32_t cnt = 0;
     for (int32_t k = 0; k < L.N; ++k) {
         const int64_t n = L.noff[(size_t)k + 1] - L.noff[(size_t)k];
         const int64_t p = paths.empty() ? 0 : paths[(size_t)k];
+        const bool large = classes && !paths.empty() && packed_need(in, cur + n, cp + p, cnt + 1) > in.giant_smem_limit;
         // at most kPathNeuron + 1 neurons per item, the range of a path's
         // neuron index
-        bool close = k == 0 || cur + n - budget > std::min(over, budget - cur) || cnt > mmk::kPathNeuron;
-        if (!close && !paths.empty() && in.giant_smem_limit > 0)
-            close = packed_need(in, cur + n, cp + p, cnt + 1) > in.giant_smem_limit;
+        const bool close = k == 0 || cur + n - budget > (large ? 0 : std::min(over, budget - cur)) ||
+                           cnt > mmk::kPathNeuron || (large && !given);
         if (close) {
             gstart.push_back(k);
             cur = cp = 0;
@@ -284,7 +285,7 @@ int64_t choose_budget(const LayoutInput &in, const Layout &L, const std::vector<
     std::vector<int32_t> gstart;
     std::vector<int64_t> item, heap;
     for (const int32_t budget : kBudgets) {
-        pack_items(in, L, paths, budget, gstart);
+        pack_items(in, L, paths, budget, false, gstart);
         item.clear();
         int64_t large = 0, widest = 0, longest = 0;
         for (size_t g = 0; g + 1 < gstart.size(); ++g) {
@@ -547,10 +548,10 @@ std::string build_layout(const LayoutInput &in, Layout &out, bool *invalid)
 
     // 3a. group boundaries
     std::vector<int32_t> gstart;
-    if (in.group_comps > 0) {
-        pack_items(in, L, {}, in.group_comps, gstart);
-    } else {
-        std::vector<int32_t> paths((size_t)N, 0);  // a path ends at each leaf
+    const bool given = in.group_comps > 0;
+    std::vector<int32_t> paths;
+    if (!given || in.cost) {
+        paths.assign((size_t)N, 0);  // a path ends at each leaf
         std::vector<char> inner;
         for (int32_t k = 0; k < N; ++k) {
             const int32_t u = L.order[(size_t)k];
@@ -560,8 +561,8 @@ std::string build_layout(const LayoutInput &in, Layout &out, bool *invalid)
             for (int32_t i = 1; i < n; ++i) inner[(size_t)par[i]] = 1;
             paths[(size_t)k] = n - (int32_t)std::count(inner.begin(), inner.end(), (char)1);
         }
-        pack_items(in, L, paths, choose_budget(in, L, paths), gstart);
     }
+    pack_items(in, L, paths, given ? in.group_comps : choose_budget(in, L, paths), given, gstart);
     const int32_t G = (int32_t)gstart.size() - 1;
     L.groups.clear();
     L.groups.reserve((size_t)G);

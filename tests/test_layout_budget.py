@@ -63,14 +63,16 @@ def test_giants_that_get_clusters(packed):
 @pytest.mark.parametrize("fp64", [False, True])
 @pytest.mark.parametrize("budget", [1, 600, 2048, 8192])
 def test_a_given_budget_is_kept_in_a_supplied_order(packed, budget, fp64):
-    """No item of several neurons passes a given budget, none is closed early, whatever the order."""
+    """No item is closed early, and none of several neurons passes a given budget but, in FP32c, by an eighth at most: where
+    that is nearer to it and stays in the regular class (items of 8,192 do not)."""
     sizes = [int(n) for n in np.random.default_rng(1).integers(50, 900, 400)]
     cost = np.random.default_rng(2).random(400)
     f, _ = packed(sizes, p_branch=0.6, group_comps=budget, cost=cost, fp64=fp64)
-    assert f["several"] <= budget
-    order, items, held = np.argsort(-cost.astype(np.float32), kind="stable"), 0, budget + 1
+    over = budget // 8 if budget < 8192 and not fp64 else 0
+    assert f["several"] <= budget + over
+    order, items, held = np.argsort(-cost.astype(np.float32), kind="stable"), 0, 2 * budget
     for k in order:  # a new item where the next neuron does not fit
-        if held + sizes[k] > budget:
+        if held + sizes[k] - budget > min(over, budget - held):
             items, held = items + 1, 0
         held += sizes[k]
     assert f["items"] == items
