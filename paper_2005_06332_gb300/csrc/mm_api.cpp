@@ -617,7 +617,6 @@ mm_status build(mm_net *net, const mm_morphologies *morph, const mm_channel_para
     // words until the rhs is final; 24 B per compartment) and per path two
     // words (the head link's current, then the contribution to the parent)
     li.smem_per_comp = opt->precision == MM_FP64 ? 16 : 24;
-    li.path_items = true;
     li.smem_per_path = opt->precision == MM_FP64 ? 0 : 8;
     li.giant_smem_limit = opt->precision == MM_FP64 ? 0 : kGiantSmemLimit;
     li.big_smem_limit = opt->precision == MM_FP64 ? 0 : kBigSmemLimit;
@@ -803,7 +802,6 @@ mm_status build(mm_net *net, const mm_morphologies *morph, const mm_channel_para
         MM_CKI(net, mmk_launch_fill_f64(net->Vsoma, chan->v_init, (int64_t)N, net->stream));
     }
 
-    const int32_t smem_comps = std::max(L.max_comps, 1), smem_segs = std::max(L.max_segs, 1);
     const double decay = syn ? std::exp(-opt->dt_ms / syn->tau_ms) : 1.0;
     if (f64) {
         mmk::StepArgs &a = net->sa;
@@ -886,7 +884,6 @@ mm_status build(mm_net *net, const mm_morphologies *morph, const mm_channel_para
         a.item1 = L.n_small;
         a.queue = &net->ctl->queue_head;
         a.meta = dmeta;
-        a.smem_meta = L.max_meta;
         a.site_comp = dsite;
         a.gsyn = net->gsyn2;
         a.ring_nrn = net->ring_nrn;
@@ -905,8 +902,6 @@ mm_status build(mm_net *net, const mm_morphologies *morph, const mm_channel_para
         a.fired = net->fired;
         a.fired_words = net->fired_words;
         a.ctl = net->ctl;
-        a.smem_comps = smem_comps;
-        a.smem_segs = smem_segs;
         // channel densities (mS/cm^2) times 1e3: conductance in uS per cm^2 of membrane
         a.gNa = split_pair(chan->gNa * 1e3);
         a.gK = split_pair(chan->gK * 1e3);
@@ -990,9 +985,6 @@ mm_status build(mm_net *net, const mm_morphologies *morph, const mm_channel_para
         b.item0 = L.n_small;
         b.item1 = L.n_small + L.n_big;
         b.queue = &net->ctl->big_head;
-        b.smem_comps = std::max(L.big_max_comps, 1);
-        b.smem_segs = std::max(L.big_max_segs, 1);
-        b.smem_meta = L.big_max_meta;
         if (L.n_big > 0) {
             const size_t bsmem = (size_t)L.big_max_smem;
             b.smem_bytes = (int32_t)bsmem;
@@ -1016,7 +1008,6 @@ mm_status build(mm_net *net, const mm_morphologies *morph, const mm_channel_para
         g.item0 = L.n_small + L.n_big;
         g.item1 = (int32_t)L.groups.size();
         g.n_huge = L.n_huge;
-        g.queue = &net->ctl->giant_head;
         net->giant_blocks = std::max(1, mmk_giant_blocks(net->n_giant, g.n_huge));
         // the giant items' compartments in chunks for the assembly and
         // update kernels: first chunk of each giant item, then the total

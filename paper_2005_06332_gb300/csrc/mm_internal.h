@@ -108,7 +108,7 @@ struct DevCtl {
     unsigned long long spk_count;   // spikes appended to the output buffer
     unsigned int queue_head;        // next work item of the current step
     int err;                        // MMK_ERR_* bits
-    unsigned int giant_head;        // next giant work item of the current step
+    unsigned int reserved;          // (keeps the layout of saved states)
     unsigned int big_head;          // next work item of the large shared-memory class
 };
 
@@ -223,7 +223,6 @@ struct StepArgs32 {
     int32_t n_groups;
     int32_t step_offset;
     const unsigned char *meta;
-    int32_t smem_meta;
     int32_t item0, item1;             // this launch's work items: [item0, item1)
     int32_t n_huge;                   // giant items: the first n_huge are solved by a cluster of blocks each
     int32_t smem_bytes;               // dynamic shared memory of the launch (largest item need)
@@ -245,7 +244,6 @@ struct StepArgs32 {
     int32_t fired_words;              // deterministic delivery, as in StepArgs
     uint32_t *fired;
     DevCtl *ctl;
-    int32_t smem_comps, smem_segs;
     float2 gNa, gK, gL;               // channel densities times 1e3 (uS per cm^2 of membrane), pairs
     FxPot ENa, EK, EL, Esyn;
     float2 decay;                     // exp(-dt / tau_syn), pair

@@ -78,7 +78,6 @@ __global__ void __launch_bounds__(256) deliver_fp32c_kernel(DeliverArgs a)
     const long long n = (long long)a.ctl->step_base + a.step_offset;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         a.ctl->queue_head = 0u;
-        a.ctl->giant_head = 0u;
         a.ctl->big_head = 0u;
         a.ring_cnt[n % a.R] = 0;
     }
@@ -146,7 +145,6 @@ __global__ void __launch_bounds__(256) deliver_ordered_fp32c_kernel(DeliverArgs 
     const long long nt = (long long)gridDim.x * blockDim.x;
     if (gt == 0) {
         a.ctl->queue_head = 0u;
-        a.ctl->giant_head = 0u;
         a.ctl->big_head = 0u;
         a.ring_cnt[n % a.R] = 0;
     }

@@ -698,8 +698,6 @@ std::string build_layout(const LayoutInput &in, Layout &out, bool *invalid)
         } else if (big) {
             bigs.push_back(gr);
             L.big_max_comps = std::max(L.big_max_comps, gr.ncomp);
-            L.big_max_segs = std::max(L.big_max_segs, gr.npath);
-            L.big_max_meta = std::max(L.big_max_meta, gr.meta_bytes);
             L.big_max_smem = std::max<int64_t>(L.big_max_smem, smem_need);
         } else {
             L.groups.push_back(gr);
@@ -707,7 +705,6 @@ std::string build_layout(const LayoutInput &in, Layout &out, bool *invalid)
             L.max_comps = std::max(L.max_comps, gr.ncomp);
             L.max_segs = std::max(L.max_segs, gr.npath);
             L.max_waves = std::max(L.max_waves, gr.nlevel);
-            L.max_meta = std::max(L.max_meta, gr.meta_bytes);
         }
     }
     L.n_small = (int32_t)L.groups.size();

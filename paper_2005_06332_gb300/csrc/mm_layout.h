@@ -37,9 +37,9 @@ struct LayoutInput {
     // shared-memory class if they fit big_smem_limit (0: no such class), else
     // they become giant items (giant_smem_limit 0: no classes at all)
     int32_t smem_per_comp;
-    int32_t smem_per_seg;         // not used: items are solved path by path
+    int32_t smem_per_seg;         // set by callers of before, not read: items are solved path by path
     int32_t giant_smem_limit, big_smem_limit;
-    bool path_items;              // not used, as above
+    bool path_items;              // as smem_per_seg
     int32_t smem_per_path;
 };
 
@@ -58,12 +58,12 @@ struct Layout {
     std::vector<mmk::GroupRec> groups;
     std::vector<unsigned char> meta;    // tree blobs (16-byte aligned per work item)
     int32_t max_comps = 0, max_segs = 0;
-    int32_t max_waves = 0, max_meta = 0;
+    int32_t max_waves = 0;
     // items [0, n_small) fit the regular shared-memory budget, the next n_big
     // the large one; the rest are giants, of which the first n_huge are solved
     // by a cluster of blocks each
     int32_t n_small = 0, n_big = 0, n_huge = 0;
-    int32_t big_max_comps = 0, big_max_segs = 0, big_max_meta = 0;
+    int32_t big_max_comps = 0;
     // largest shared-memory need (model above) of one item of each class
     int64_t max_smem = 0, big_max_smem = 0;
     int64_t giant_comps = 0;            // compartments in giant items (size of the Hines scratch)
