@@ -292,8 +292,10 @@ mm_status mm_read_kernel_timing(mm_net *net, mm_kernel_times *out, int32_t reset
  * b = diagonal, c = lower (row j, column p(j)), rhs.  Writes the solution
  * of every system to x.  ALL pointers are DEVICE pointers; inputs are not
  * modified.  Runs on cuda_stream (NULL: the legacy default stream) and
- * returns after the solve has finished.  Allocates a device scratch of
- * n_comp doubles for the duration of the call.
+ * returns after the solve has finished.  x may be rhs.  Allocates a device
+ * scratch of n_comp doubles and about a thousandth more for the duration of the
+ * call.  Results are Algorithm 1's to rounding, its infinities and NaN included
+ * (zero pivots, entries at the ends of FP64's range).
  * Errors: MM_EINVAL (negative sizes, NULL arrays, a tree whose offsets do
  * not lie within [0, n_comp] in ascending order, or a tree that violates the
  * parent rule: such a tree is skipped and its entries of x are undefined,
@@ -308,8 +310,8 @@ mm_status mm_hines_solve(int32_t n_trees, int64_t n_comp, const int64_t *tree_of
  * device byte (a cudaMalloc there fails or breaks its accounting), or a
  * latency-critical loop where an allocation could block or fail mid-run.
  * Same arguments, results and errors as mm_hines_solve; the caller still
- * passes every input and the output x.  The scratch is a fixed 8 MiB
- * device array inside this library (loaded on every GPU that loads the
+ * passes every input and the output x.  The scratch is a fixed 8 MiB (and
+ * 8 KiB) device array inside this library (loaded on every GPU that loads the
  * library, until the process ends), so n_comp must not exceed 1,048,576
  * (MM_EINVAL otherwise).  Every call looks up that array's device address
  * (cudaGetSymbolAddress, with the caller's device current; the first call on
@@ -497,7 +499,10 @@ typedef struct {
  * -- creates the sample network with *opt otherwise unchanged, runs `warmup`
  * steps and times `steps` steps with CUDA events on opt->cuda_stream (a
  * library-owned stream when NULL).  *best receives *opt with the fastest
- * candidate's block_threads and group_comps.  points (cap entries; NULL
+ * candidate's block_threads and group_comps.  The budget that mm_create_network
+ * chooses where both are 0 is not among the candidates; it may be below 1024 and
+ * then faster for networks too small to fill the device with such items (64
+ * neurons of 255 compartments: 64 items instead of 16).  points (cap entries; NULL
  * allowed when cap == 0) receives the candidates in order, *n_points how many
  * were written.
  *
