@@ -63,9 +63,9 @@ PROFILED = {
     # ncu counters of one regular-class launch of the step kernel (multi10k,
     # 512 threads, 4096-compartment items, a step inside the timed window)
     ("multi10k", "fp32c", "step", "soma"): {
-        "sha256": "132602ec0c1958b1e29253aa36b97739ae9a1e6e2dd9edc34f60a967316c841c",
-        "dram_bytes": 494440192 + 111394560,
-        "warp_instructions": 283394194,
+        "sha256": "07ea9f2c1d0c809a5158d89a24a1277baa867291cda58b1b63160fa421144828",
+        "dram_bytes": 494356480 + 111257856,
+        "warp_instructions": 283394206,
         "comps": 9484756,
     },
 }

@@ -175,8 +175,8 @@ struct Front {
 //     does (the chains are sorted by level and that entry).
 // b and rhs, then N and S, then f and s, then x live in the scratch and the
 // output array (L2).  Measured (whole call, allocation included): 3,000 trees of
-// 50 to 5,000 entries 12.4 ms with a thread per tree, 0.89 ms so (0.82 ms in
-// the kernel, FP64 pipe 36 % busy); 3,000 of 8 to 300 0.78 -> 0.33 ms; 64 of 200
+// 50 to 5,000 entries 12.4 ms with a thread per tree, 0.87 ms so (0.65 ms in
+// the kernel, FP64 pipe 44 % busy); 3,000 of 8 to 300 0.78 -> 0.33 ms; 64 of 200
 // to 5,000 9.0 -> 0.57 ms.  128 threads and six blocks per SM; 32 or 64 threads
 // and more blocks 0.94 to 1.14 ms, groups of 4,096 entries 1.34 ms; eliminating
 // the diagonal alone first (with a c stored: 2 + 2 + 2 instructions in the
