@@ -329,8 +329,7 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 512 / NT : 1) step_fp64_kernel
     // rates evaluated, 0.74 ms with the table and products (five instructions a
     // sweep step), 0.55 ms on the scaled system (two); 64 neurons of 255 370,
     // 159, 121 us; 701 of 50 to 3,000, points and ordered delivery, 808, 262,
-    // 185 us.  Warps on paths from 48 or 160 compartments instead of 96: 5 % and
-    // 2 % slower; three or four blocks per SM (85 or 64 registers) 2 to 10 %.
+    // 185 us.  Three or four blocks per SM (85 or 64 registers) 2 to 10 %.
     //
     // Shared memory: the item's tree blob (one bulk copy), then per
     // compartment the pair (diagonal, rhs) -- after a path's elimination
@@ -547,90 +546,130 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 512 / NT : 1) step_fp64_kernel
             }
             eliminate_head(P, N, M, S);
         };
-        // The same by a whole warp.  The elimination step is linear in
-        // (N, M, S): each lane composes the steps of its chunk (the images of
-        // the first two unit vectors; S itself is multiplied by 2^(p >> 20)), an
-        // inclusive warp scan combines the chunks, and each lane runs the steps
-        // of its chunk from the vector that the chunks before it leave.  Here
-        // the lanes divide themselves and store (-f, c).
+        // The same by a whole warp.  The pivots' recursion in (N, M) would
+        // compose into matrices whose parts cancel, to the square of a chunk's
+        // length where the couplings are far above C / dt (pivots off by 1e-9 on
+        // a chain of 4,000 wide compartments).  The pivot less the link to the
+        // compartment above, X = N / M - L, only adds: with U the link as the
+        // compartment above holds it (L U = gamma^2) and d its diagonal,
+        //   X_{j-1} = (d_{j-1} - U - L_{j-1}) + U X_j / (L_j + X_j),
+        // a quotient of linear forms in X with positive factors.  Each lane
+        // composes its chunk's as a 2x2 matrix and a warp scan combines them; with
+        // the pivot at its chunk's end a lane runs the steps of its chunk, stores
+        // -f and composes the rhs recursion R_{j-1} = f_j R_j + r_{j-1}
+        // (R = S / M), which a second scan combines; then c = R M / N.
+        // 2,000 neurons of 50 to 5,000 compartments 484 -> 495 us per step, the
+        // chain of 4,000 off by 1e-13 mV after a step instead of 8e-10, as with a
+        // lane for each path; warps from 128 or 160 compartments 498 and 501 us,
+        // none 522 us, and 701 neurons of 50 to 3,000 210, 213 and 282 for 210.
         auto eliminate_path_warp = [&](int pi) {
             const PathQ P = paths[pi];
             const int h = P.head, e = P.end;
             const int m = e - 1 - h;  // steps t = 0 .. m-1: compartment e-1-t into e-2-t
             const int cs = (m + 31) >> 5;
             const int t0 = min(lane * cs, m), t1 = min(t0 + cs, m);
+            const unsigned F = 0xFFFFFFFFu;
             const double2 leaf = sdr[e - 1];
-            double n1 = 1.0, m1 = 0.0, s1 = 0.0, n2 = 0.0, m2 = 1.0, s2 = 0.0;
-            int p = 0;
-            // (a product of thousands of factors leaves FP64's range, so the
-            // exponent stops at +-1000: nothing is left of what it multiplies)
-            auto clamp = [](int x) { return max(min(x, 1000 << 20), -(1000 << 20)); };
+            // the matrix's entries by a power of two, the largest then in [1, 2)
+            double m00 = 1.0, m01 = 0.0, m10 = 0.0, m11 = 1.0;
+            auto normalise = [&]() {
+                const int x = max(max(__double2hiint(m00), __double2hiint(m01)), max(__double2hiint(m10), __double2hiint(m11)));
+                const int d = 0x3FF00000 - (x & 0x7FF00000);
+                m00 = scale2(m00, d);
+                m01 = scale2(m01, d);
+                m10 = scale2(m10, d);
+                m11 = scale2(m11, d);
+            };
+            // a link as one end (scale x) holds it; r: the reciprocal of the other end's scale
+            auto link = [](double x, double r, int k) { return scale2(x * r, k); };
             double2 nb = make_double2(0.0, 0.0);
-            for (int t = t0; t < t1; ++t) {
-                const int j = e - 1 - t, k = __ldg(kexp + j);
-                const double2 w = sdr[j - 1];
-                const int d = exponent2(n1);
-                n1 = scale2(n1, -d);
-                n2 = scale2(n2, -d);
-                const double a1 = fma(w.x, n1, -scale2(m1, 2 * k - d)), a2 = fma(w.x, n2, -scale2(m2, 2 * k - d));
-                s1 = fma(w.y, n1, scale2(s1, k - d));
-                s2 = fma(w.y, n2, scale2(s2, k - d));
-                m1 = n1;
-                n1 = a1;
-                m2 = n2;
-                n2 = a2;
-                p = clamp(p + (k - d));
-                nb = w;
-            }
-            for (int off = 1; off < 32; off <<= 1) {
-                const unsigned F = 0xFFFFFFFFu;
-                const double bn1 = __shfl_up_sync(F, n1, off), bm1 = __shfl_up_sync(F, m1, off),
-                             bs1 = __shfl_up_sync(F, s1, off), bn2 = __shfl_up_sync(F, n2, off),
-                             bm2 = __shfl_up_sync(F, m2, off), bs2 = __shfl_up_sync(F, s2, off);
-                const int bp = __shfl_up_sync(F, p, off);
-                if (lane >= off) {  // this lane's steps act after the earlier lanes'
-                    const double an1 = fma(n1, bn1, n2 * bm1), am1 = fma(m1, bn1, m2 * bm1),
-                                 as1 = fma(s1, bn1, fma(s2, bm1, scale2(bs1, p)));
-                    const double an2 = fma(n1, bn2, n2 * bm2), am2 = fma(m1, bn2, m2 * bm2),
-                                 as2 = fma(s1, bn2, fma(s2, bm2, scale2(bs2, p)));
-                    const int d = exponent2(an1);
-                    n1 = scale2(an1, -d);
-                    m1 = scale2(am1, -d);
-                    s1 = scale2(as1, -d);
-                    n2 = scale2(an2, -d);
-                    m2 = scale2(am2, -d);
-                    s2 = scale2(as2, -d);
-                    p = clamp(clamp(p + bp) - d);
+            double l0 = 0.0;  // L of the chunk's first compartment
+            if (t0 < t1) {
+                int i = e - 2 - t0, ka = __ldg(kexp + i + 1);
+                const double sl = scale_of(i + 1);
+                double sb = scale_of(i), ra = rcp_nr(sl), rb = rcp_nr(sb);
+                double L = link(sl, rb, ka);
+                l0 = L;
+                for (int t = t0; t < t1; ++t, --i) {
+                    const double2 w = sdr[i];
+                    const double U = link(sb, ra, ka);
+                    double Lu = 0.0, su = 1.0, ru = 1.0;
+                    int ku = 0;
+                    if (i > h) {
+                        ku = __ldg(kexp + i);
+                        su = scale_of(i - 1);
+                        ru = rcp_nr(su);
+                        Lu = link(sb, ru, ku);
+                    }
+                    const double A = w.x - Lu, B = (A - U) * L;
+                    const double n00 = fma(A, m00, B * m10), n01 = fma(A, m01, B * m11);
+                    m10 = fma(L, m10, m00);
+                    m11 = fma(L, m11, m01);
+                    m00 = n00;
+                    m01 = n01;
+                    normalise();
+                    ra = rb;
+                    ka = ku;
+                    sb = su;
+                    rb = ru;
+                    L = Lu;
+                    nb = w;
                 }
             }
-            // the vector at the chunk's first compartment: the earlier
-            // chunks' steps on the leaf's (d, 1, r)
-            double N, M, S;
-            {
-                const unsigned F = 0xFFFFFFFFu;
-                const double bn1 = __shfl_up_sync(F, n1, 1), bm1 = __shfl_up_sync(F, m1, 1),
-                             bs1 = __shfl_up_sync(F, s1, 1), bn2 = __shfl_up_sync(F, n2, 1),
-                             bm2 = __shfl_up_sync(F, m2, 1), bs2 = __shfl_up_sync(F, s2, 1);
-                const int bp = __shfl_up_sync(F, p, 1);
-                N = lane ? fma(bn1, leaf.x, bn2) : leaf.x;
-                M = lane ? fma(bm1, leaf.x, bm2) : 1.0;
-                S = lane ? fma(bs1, leaf.x, bs2 + scale2(leaf.y, bp)) : leaf.y;
+            for (int off = 1; off < 32; off <<= 1) {
+                const double a00 = __shfl_up_sync(F, m00, off), a01 = __shfl_up_sync(F, m01, off),
+                             a10 = __shfl_up_sync(F, m10, off), a11 = __shfl_up_sync(F, m11, off);
+                if (lane >= off) {  // this lane's steps act after the earlier lanes'
+                    const double n00 = fma(m00, a00, m01 * a10), n01 = fma(m00, a01, m01 * a11);
+                    const double n10 = fma(m10, a00, m11 * a10), n11 = fma(m10, a01, m11 * a11);
+                    m00 = n00;
+                    m01 = n01;
+                    m10 = n10;
+                    m11 = n11;
+                    normalise();
+                }
             }
+            // the pivot of the chunk's first compartment
+            double N = leaf.x;
+            {
+                const double b00 = __shfl_up_sync(F, m00, 1), b01 = __shfl_up_sync(F, m01, 1),
+                             b10 = __shfl_up_sync(F, m10, 1), b11 = __shfl_up_sync(F, m11, 1);
+                const double X = leaf.x - __shfl_sync(F, l0, 0);
+                if (lane) N = fma(b00, X, b01) / fma(b10, X, b11) + l0;
+            }
+            double M = 1.0, A = 1.0, B = 0.0, none = 0.0;
             __syncwarp();  // every lane has read its chunk and the element after it
             for (int t = t0; t < t1; ++t) {
                 const int j = e - 1 - t, k = __ldg(kexp + j);
                 const double2 w = t + 1 < t1 ? sdr[j - 1] : nb;
-                const double inv = rcp_nr(N);
-                sdr[j] = make_double2(-scale2(div_nr(M, N, inv), k), div_nr(S, N, inv));
-                step(N, M, S, k, w);
+                const double f = scale2(div_nr(M, N, rcp_nr(N)), k);
+                sdr[j].x = -f;
+                A *= f;
+                B = fma(f, B, w.y);
+                step(N, M, none, k, w);
+            }
+            for (int off = 1; off < 32; off <<= 1) {
+                const double pa = __shfl_up_sync(F, A, off), pb = __shfl_up_sync(F, B, off);
+                if (lane >= off) {
+                    B = fma(A, pb, B);
+                    A *= pa;
+                }
+            }
+            const double ea = __shfl_up_sync(F, A, 1), eb = __shfl_up_sync(F, B, 1);
+            double R = lane ? fma(ea, leaf.y, eb) : leaf.y;
+            for (int t = t0; t < t1; ++t) {
+                const int j = e - 1 - t;
+                const double f = -sdr[j].x, r = t + 1 < t1 ? sdr[j - 1].y : nb.y;
+                sdr[j].y = R * scale2(f, -__ldg(kexp + j));
+                R = fma(f, R, r);
             }
             // the head, from the lane whose chunk ends at it
             const int lastl = (m - 1) / cs;
-            N = __shfl_sync(0xFFFFFFFFu, N, lastl);
-            M = __shfl_sync(0xFFFFFFFFu, M, lastl);
-            S = __shfl_sync(0xFFFFFFFFu, S, lastl);
+            N = __shfl_sync(F, N, lastl);
+            M = __shfl_sync(F, M, lastl);
+            R = __shfl_sync(F, R, lastl);
             __syncwarp();
-            if (lane == 0) eliminate_head(P, N, M, S);
+            if (lane == 0) eliminate_head(P, N, M, R * M);
             __syncwarp();
         };
         // eliminations into the compartments that several paths of the level
