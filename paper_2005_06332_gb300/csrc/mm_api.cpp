@@ -96,6 +96,7 @@ struct mm_net {
     double *area = nullptr, *gax = nullptr, *gsyn = nullptr;
     double *sc = nullptr, *s2a = nullptr, *dcon = nullptr;  // the scaled Hines system (StepArgs)
     int32_t *kexp = nullptr;
+    float *drest = nullptr;
     double2 *gtab64 = nullptr;        // gate table for dt (mm_gate_table64.h)
     // device arrays (FP32c path)
     int32_t *Vq = nullptr;
@@ -671,6 +672,7 @@ mm_status build(mm_net *net, const mm_morphologies *morph, const mm_channel_para
         ZR(net->sc, C);
         ZR(net->s2a, C);
         ZR(net->kexp, C);
+        ZR(net->drest, C);
         {
             std::vector<mmg::Quad64> tab((size_t)mmg::kTab64Quads * mmg::kTab64Intervals);
             mmg::build_table64(opt->dt_ms, tab.data());
@@ -790,7 +792,7 @@ mm_status build(mm_net *net, const mm_morphologies *morph, const mm_channel_para
         ia.n = net->n;
         MM_CKI(net, mmk_launch_init(ia, net->stream));
         const bool cn = opt->scheme == MM_SCHEME_CN;
-        mmk::ScaleArgs64 sa{dgroups, dmeta, net->area, net->gax, net->sc, net->s2a, net->dcon, net->kexp,
+        mmk::ScaleArgs64 sa{dgroups, dmeta, net->area, net->gax, net->sc, net->s2a, net->dcon, net->kexp, net->drest,
                             cn ? 0.5 : 1.0, chan->Cm * 1e3 / opt->dt_ms + (cn ? 0.0 : chan->gL * 1e3)};
         MM_CKI(net, mmk_launch_scale(sa, (int)L.groups.size(), net->stream));
     } else {
@@ -815,6 +817,7 @@ mm_status build(mm_net *net, const mm_morphologies *morph, const mm_channel_para
         a.sc = net->sc;
         a.s2a = net->s2a;
         a.kexp = net->kexp;
+        a.drest = net->drest;
         a.gtab = net->gtab64;
         a.stim = net->stim;
         a.user_id = net->user_id;

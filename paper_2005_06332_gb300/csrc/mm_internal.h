@@ -125,6 +125,7 @@ struct StepArgs {
     // the coupling to the parent inside a path
     const double *sc, *s2a, *dcon;
     const int32_t *kexp;
+    const float *drest;               // what dcon's rounding left out
     const double2 *gtab;              // gate table for dt (mm_gate_table64.h): 18 arrays of 961 16-byte quads
     const double *stim;               // soma current per internal neuron, nA [N]
     const int32_t *user_id;           // internal neuron -> user id [N]
@@ -170,6 +171,7 @@ struct ScaleArgs64 {
     const double *area, *gax;
     double *sc, *s2a, *dcon;
     int32_t *kexp;
+    float *drest;
     double gimp;                      // implicit share of each axial coupling: 1, or 1/2 for Eq. 2 as printed
     double cm_leak;                   // (Cm / dt + the implicit leak) * 1e3: uS per cm^2 of membrane
 };

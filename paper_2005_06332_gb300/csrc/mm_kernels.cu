@@ -98,7 +98,12 @@ __global__ void init_kernel(InitArgs a)
 // below 2^-500 uS, or none (infinite Ra), is taken as 2^-500, which adds nothing
 // to any diagonal and whose square keeps exponent fields within 32 bits.  Then the
 // constant part of the diagonal: C/dt, the implicit leak and the couplings,
-// times s^2 -- inside a path as the matrix holds them, s 2^k / s_parent.
+// times s^2 -- as the matrix holds them, s 2^k / s_parent inside a path, the
+// rounded coupling times or over s_parent at a head.  It is the same at every
+// step, so what its rounding leaves out is kept in FP32: it would add up over the
+// steps, as a part of the couplings (18 neurons of 20 to 4,000 compartments with
+// couplings up to 1e4 C/dt, 80 steps: 6.4e-14 mV in the mean square without it,
+// 7.5e-15 with it; 1.5 % of the step's time).
 __global__ void __launch_bounds__(128) scale_kernel(ScaleArgs64 a)
 {
     const GroupRec G = a.groups[blockIdx.x];
@@ -108,13 +113,32 @@ __global__ void __launch_bounds__(128) scale_kernel(ScaleArgs64 a)
     const double *area = a.area + G.comp0, *gax = a.gax + G.comp0;
     double *sc = a.sc + G.comp0, *s2a = a.s2a + G.comp0, *dcon = a.dcon + G.comp0;
     int32_t *kexp = a.kexp + G.comp0;
+    float *drest = a.drest + G.comp0;
     auto scale_of = [&](int i) { return signbit(sc[i]) ? 1.0 : sc[i]; };
+    // a value and the rest of it; x y, x / y, and the sum
+    struct Two {
+        double v, r;
+    };
+    auto times = [](double x, double y) { const double p = x * y; return Two{p, fma(x, y, -p)}; };
+    auto over = [](double x, double y) { const double q = x / y; return Two{q, fma(-q, y, x) / y}; };
+    auto plus = [](const Two &x, const Two &y) {
+        const double t = x.v + y.v, u = t - x.v;
+        return Two{t, ((x.v - (t - u)) + (y.v - u)) + (x.r + y.r)};
+    };
+    auto scaled = [](const Two &x, int k) { return Two{scale2(x.v, k), scale2(x.r, k)}; };
+    auto store = [&](int j, const Two &d) {
+        const double v = d.v + d.r;
+        dcon[j] = v;
+        drest[j] = (float)((d.v - v) + d.r);
+    };
     for (int pi = threadIdx.x; pi < G.npath; pi += 128) {
         const PathQ P = paths[pi];
         const int h = P.head;
-        double s = 1.0, own = a.gimp * fabs(gax[h]);  // own: s^2 w g of the link to the parent
+        double s = 1.0;
+        Two own{0.0, 0.0};  // s^2 w g of the link to the parent (a head's is added below)
         for (int j = h; j < P.end; ++j) {
-            double sn = 1.0, link = 0.0, next_own = 0.0;
+            double sn = 1.0;
+            Two link{0.0, 0.0}, next_own{0.0, 0.0};
             if (j + 1 < P.end) {
                 const double c = a.gimp * gax[j + 1] * s;
                 if (c < 0x1p-500) {
@@ -124,15 +148,19 @@ __global__ void __launch_bounds__(128) scale_kernel(ScaleArgs64 a)
                     sn = mantissa(p);
                     const int k = -exponent2(p);
                     kexp[j + 1] = k;
-                    link = scale2(s / sn, k);
-                    next_own = scale2(sn / s, k);
+                    link = scaled(over(s, sn), k);
+                    next_own = scaled(over(sn, s), k);
                 }
             }
-            const double s2 = s * s * area[j];
+            const Two ss = times(s, s);
+            Two s2 = times(ss.v, area[j]);
+            s2.r = fma(ss.r, area[j], s2.r);
+            Two cm = times(s2.v, a.cm_leak);
+            cm.r = fma(s2.r, a.cm_leak, cm.r);
             sc[j] = j == h ? -0.0 : s;
             if (j == h) kexp[j] = 0;
-            s2a[j] = s2;
-            dcon[j] = s2 * a.cm_leak + (own + link);
+            s2a[j] = s2.v;
+            store(j, plus(cm, plus(own, link)));
             s = sn;
             own = next_own;
         }
@@ -140,18 +168,21 @@ __global__ void __launch_bounds__(128) scale_kernel(ScaleArgs64 a)
     __syncthreads();
     for (int pi = threadIdx.x; pi < G.npath; pi += 128) {
         const PathQ P = paths[pi];
-        if (P.parent >= 0) sc[P.head] = -(a.gimp * fabs(gax[P.head]) * scale_of(P.parent));
+        if (P.parent < 0) continue;
+        const double sp = scale_of(P.parent), g = a.gimp * fabs(gax[P.head]) * sp;
+        sc[P.head] = -g;
+        store(P.head, plus(Two{dcon[P.head], drest[P.head]}, over(g, sp)));
     }
     __syncthreads();
     for (int e = threadIdx.x; e < G.npath; e += 128) {
         const int att = (int)(fold[e] >> 16);
         if (att >= G.ncomp) continue;  // a path from a soma (no parent)
         if (e > 0 && (int)(fold[e - 1] >> 16) == att) continue;  // not the first path of its parent
-        double d = dcon[att];
+        Two d{dcon[att], drest[att]};
         const double s = scale_of(att);
         for (int z = e; z < G.npath && (int)(fold[z] >> 16) == att; ++z)
-            d = fma(-sc[paths[fold[z] & 0xFFFFu].head], s, d);
-        dcon[att] = d;
+            d = plus(d, times(-sc[paths[fold[z] & 0xFFFFu].head], s));
+        store(att, d);
     }
 }
 
@@ -390,7 +421,7 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 512 / NT : 1) step_fp64_kernel
             const double ar = a.area[c0 + i], g = gax[i];
             const double gna = a.gNa * ((mm * mm) * (mm * hh)), n2 = nn * nn, gk = a.gK * (n2 * n2);
             double d = a.dcon[c0 + i];
-            if (a.g_implicit) d = fma(a.s2a[c0 + i], gna + gk, d);
+            if (a.g_implicit) d += fma(a.s2a[c0 + i], gna + gk, mmg::widen(a.drest[c0 + i]));
             double r = -ar * fma(gna, v - a.ENa, fma(gk, v - a.EK, a.gL * (v - a.EL)));
             if (!signbit(g)) r = fma(g, V[i - 1] - v, r);
             if (i + 1 < G.ncomp) {
