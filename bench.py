@@ -63,9 +63,9 @@ PROFILED = {
     # ncu counters of one regular-class launch of the step kernel (multi10k,
     # 512 threads, 4096-compartment items, a step inside the timed window)
     ("multi10k", "fp32c", "step", "soma"): {
-        "sha256": "07ea9f2c1d0c809a5158d89a24a1277baa867291cda58b1b63160fa421144828",
-        "dram_bytes": 494356480 + 111257856,
-        "warp_instructions": 283394206,
+        "sha256": "fde6f654a8551a41bc61462f13835ae6f3145a25915c1de802ff302d99bb5724",
+        "dram_bytes": 494649856 + 111322880,
+        "warp_instructions": 283394241,
         "comps": 9484756,
     },
 }
